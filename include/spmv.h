@@ -436,13 +436,16 @@ int spmv_csr_error(int64_t* out);
  * resident in HBM and multiplied in one persistent launch per layout
  * (CSR modes, sliced layout).  Work items are blocks of up to 256 rows of
  * one matrix (CSR modes) or up to 8 slices or 32 long rows of one matrix
- * (sliced layout), claimed by warps through an atomic ticket, matrix by
- * matrix with each matrix's heaviest items first; each row is summed by
- * `lanes` lanes (set per matrix, e.g. by an autotuner), a row longer than
- * 64 entries by a whole warp, in a fixed order, so y is the same, bit for
+ * (sliced layout), taken by warps whole or, so that a small batch fills the
+ * chip, in parts, matrix by matrix with each matrix's heaviest work first;
+ * each row is summed by `lanes` lanes (set per matrix, e.g. by an autotuner),
+ * a row longer than 64 entries by a whole warp, a row longer than 512, 1024 or
+ * 2048 entries (by the batch's size) in pieces of that length whose sums are
+ * added, in a fixed order, so y is the same, bit for
  * bit, as with spmv_batch_run_separate, which launches the same row code
  * once per matrix.  Not part of the paper's method: a way of running many
- * of its SpMVs at once.
+ * of its SpMVs at once.  One spmv_batch_run of a batch may be in flight at a
+ * time.
  * spmv_batch_create: `count` matrices given as HOST CSR arrays (n[m],
  *   row_ptr[m][n[m]+1] int64, col_idx[m] int32 in [0, n[m]), vals[m]),
  *   copied to the current device.  Errors as spmv_part_create.

@@ -3,12 +3,20 @@
 // The matrices of a batch live back to back in HBM (row pointers local to
 // each matrix, entries padded to a multiple of 4 so every matrix starts
 // 16-byte aligned).  A work item is a block of up to 256 rows of one matrix;
-// the warps of a persistent grid claim items with an atomic ticket and
-// compute every row with the pair-per-lane scheme or warp-staged rows
+// the warps of a persistent grid claim items, or parts of them where the batch
+// is small, with an atomic ticket (the smallest batches are dealt out without
+// one) and compute every row with the pair-per-lane scheme or warp-staged rows
 // (chosen per matrix by the autotuner); rows longer than 64 entries are
-// summed by a whole warp.  The plain alternative launches the same per-row
-// code once per matrix; both give bit-identical results because each row
-// is summed by the same lanes in the same order.
+// summed by a whole warp, the longest in pieces shared between warps.  The
+// plain alternative launches the same per-row code once per matrix; both give
+// bit-identical results because each row is summed by the same lanes in the
+// same order.
+//
+// What bounds it: a small batch by the dependent loads of one warp's work
+// (12 matrices of up to 30000 rows, two lanes a row: 18 us against 71 us with
+// whole items of 256 rows and uncut rows; sliced 21 against 62 us), a large one
+// by HBM and the x gathers (48 matrices of up to 1 M rows, sliced: 205 us
+// against 217 us; two lanes a row 361 against 386 us).
 #include "batch.h"
 
 #include <cuda_runtime.h>
@@ -25,6 +33,7 @@ constexpr int kItemRows = 256;
 constexpr int kThreads = 256;
 
 using spmvk::BatchItem;
+using spmvk::BatchPiece;
 using spmvk::BSlice;
 
 constexpr int kSliced = 64;   // lanes value selecting the sliced layout
@@ -34,11 +43,15 @@ struct BatchArgs {
     const int32_t* col;
     const double* val;
     const BatchMat* mats;
-    const BatchItem* items;
-    const int* order;         // claim order of the persistent launch
+    const BatchItem* items;   // range kernels: the items, matrix by matrix
+    const BatchItem* units;   // other launches: n_units work units in claim order
     const double* x;
     double* y;
-    int n_items;
+    int n_units;
+    int piece_len;            // a row longer than this is cut into pieces
+    const BatchPiece* pieces;
+    double* piece_sum;
+    int* piece_cnt;
     int* ticket;
 };
 
@@ -67,50 +80,136 @@ __device__ __forceinline__ int32_t ld_stream(const int32_t* p) {
 constexpr int kLongRow = 64;   // rows longer than this are summed by a whole warp
 
 // One row summed by the 32 lanes of a warp: lane l takes entries l, l+32,
-// ... in order (four loads in flight), then a fixed xor-butterfly; every
-// lane returns the total.
+// ... in order (D of them in flight), then a fixed xor-butterfly; every lane
+// returns the total, the same for every D.  D = 4 leaves registers for many
+// warps, which hide each other's latency; D = 16 also loads the columns one
+// round ahead, for launches with so few warps that a long row's chain of
+// load-then-gather rounds is what the launch waits for.
+template <int D>
 __device__ __forceinline__ double warp_row(const int32_t* col, const double* val, const double* x, int kb, int ke,
                                            uint64_t pol) {
     const int lane = threadIdx.x & 31;
     double part = 0.0;
     int k = kb + lane;
-    for (; k + 96 < ke; k += 128) {
-        double v[4], xv[4];
+    if (D <= 4) {
+        for (; k + 32 * (D - 1) < ke; k += 32 * D) {
+            double v[D], xv[D];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            v[u] = __ldg(val + k + 32 * u);
-            xv[u] = ldg_keep(x + __ldg(col + k + 32 * u), pol);
+            for (int u = 0; u < D; ++u) {
+                v[u] = __ldg(val + k + 32 * u);
+                xv[u] = ldg_keep(x + __ldg(col + k + 32 * u), pol);
+            }
+#pragma unroll
+            for (int u = 0; u < D; ++u) part = fma(v[u], xv[u], part);
         }
+        for (; k < ke; k += 32) part = fma(__ldg(val + k), ldg_keep(x + __ldg(col + k), pol), part);
+    } else {
+        int32_t c[D];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) part = fma(v[u], xv[u], part);
+        for (int u = 0; u < D; ++u) c[u] = k + 32 * u < ke ? __ldg(col + k + 32 * u) : 0;
+        for (int base = kb; base < ke; base += 32 * D, k += 32 * D) {
+            double v[D], xv[D];
+#pragma unroll
+            for (int u = 0; u < D; ++u) {
+                const bool m = k + 32 * u < ke;
+                v[u] = m ? __ldg(val + k + 32 * u) : 0.0;
+                xv[u] = m ? ldg_keep(x + c[u], pol) : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < D; ++u) c[u] = k + 32 * (D + u) < ke ? __ldg(col + k + 32 * (D + u)) : 0;
+#pragma unroll
+            for (int u = 0; u < D; ++u) {
+                if (base + 32 * u >= ke) break;   // warp-uniform
+                const double t = fma(v[u], xv[u], part);
+                part = k + 32 * u < ke ? t : part;
+            }
+        }
     }
-    for (; k < ke; k += 32) part = fma(__ldg(val + k), ldg_keep(x + __ldg(col + k), pol), part);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
     return part;
 }
 
+// Sum over the pieces of a cut row, lane l holding the sum of pieces l, l+32,
+// ... in order: the fixed butterfly of warp_row.
+__device__ __forceinline__ double piece_total(double acc) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+    return acc;
+}
+
+// A long row [kb, ke) by the calling warp, stored by lane 0.  A row longer than
+// the batch's piece length is summed piece by piece, so that one such row (the
+// longest hold thousands of entries, a chain of 30 or more load-then-gather
+// rounds) can be shared out: with INLINE by this warp alone, the pieces one
+// after another; else it is left to the launch's piece items (batch_piece),
+// which give the same sum.
+template <int D, bool INLINE>
+__device__ __forceinline__ void long_row(const int32_t* col, const double* val, const double* x, double* y, int row,
+                                         int kb, int ke, int piece_len, uint64_t pol) {
+    const int lane = threadIdx.x & 31;
+    if (ke - kb <= piece_len) {
+        const double t = warp_row<D>(col, val, x, kb, ke, pol);
+        if (lane == 0) y[row] = t;
+    } else if (INLINE) {
+        double acc = 0.0;
+        int p = 0;
+        for (int k = kb; k < ke; k += piece_len, ++p) {
+            const double t = warp_row<D>(col, val, x, k, k + piece_len < ke ? k + piece_len : ke, pol);
+            if (lane == (p & 31)) acc += t;
+        }
+        acc = piece_total(acc);
+        if (lane == 0) y[row] = acc;
+    }
+}
+
+// Sum t of a piece into its slot; the warp that completes the row adds the
+// row's slots, lane l taking slots l, l+32, ... in order, and sets the counter
+// back to zero.  Not inlined: its few live values would otherwise push the
+// sliced persistent kernel out of its 40 registers.
+__device__ __noinline__ void publish_piece(const BatchPiece* piece, double* piece_sum, int* piece_cnt, double* y,
+                                           double t) {
+    const BatchPiece& pc = *piece;
+    const int lane = threadIdx.x & 31;
+    int last = 0;
+    if (lane == 0) {
+        piece_sum[pc.first + pc.part] = t;
+        __threadfence();
+        last = atomicAdd(piece_cnt + pc.cidx, 1) == pc.nparts - 1;
+    }
+    if (!__shfl_sync(0xffffffffu, last, 0)) return;
+    __threadfence();
+    double acc = 0.0;
+    for (int p = lane; p < pc.nparts; p += 32) acc += __ldcg(piece_sum + pc.first + p);
+    acc = piece_total(acc);
+    if (lane == 0) {
+        y[pc.row] = acc;
+        piece_cnt[pc.cidx] = 0;   // ready for the next launch
+    }
+}
+
 // The long rows flagged in `mask` (bit = the lane holding the row's kb, ke
 // and row index), one after another, each by the whole warp.
+template <int D, bool INLINE>
 __device__ __forceinline__ void warp_long_rows(unsigned mask, int kb, int ke, int row, const int32_t* col,
-                                               const double* val, const double* x, double* y, uint64_t pol) {
+                                               const double* val, const double* x, double* y, int piece_len,
+                                               uint64_t pol) {
     while (mask) {
         const int src = __ffs(mask) - 1;
         mask &= mask - 1;
         const int rkb = __shfl_sync(0xffffffffu, kb, src);
         const int rke = __shfl_sync(0xffffffffu, ke, src);
         const int rrow = __shfl_sync(0xffffffffu, row, src);
-        const double t = warp_row(col, val, x, rkb, rke, pol);
-        if ((threadIdx.x & 31) == 0) y[rrow] = t;
+        long_row<D, INLINE>(col, val, x, y, rrow, rkb, rke, piece_len, pol);
     }
 }
 
 // Rows [r0, r1) of one matrix by one warp: V lanes per row, lane h takes the
 // aligned entry pairs h, h+V, ...; the FMA loop runs the warp's longest
-// share.  Rows longer than kLongRow are left out of that loop and summed
-// afterwards by the whole warp, so one long row never holds 32 / V short
+// share.  Rows longer than kLongRow (than piece_len when a row has the whole warp
+// anyway) are left out of that loop and summed afterwards by long_row, so one long row never holds 32 / V short
 // ones (or the warp) for its whole length.
-template <int V>
+template <int V, int D, bool INLINE>
 __device__ __forceinline__ void batch_rows(const BatchArgs& a, const BatchMat& m, int r0, int r1, uint64_t pol) {
     constexpr int GROUPS = 32 / V;
     constexpr int U = 4;
@@ -128,7 +227,7 @@ __device__ __forceinline__ void batch_rows(const BatchArgs& a, const BatchMat& m
         if (row < r1) {
             kb = __ldg(ptr + row);
             ke = __ldg(ptr + row + 1);
-            is_long = V < 32 && ke - kb > kLongRow;
+            is_long = ke - kb > (V < 32 ? kLongRow : a.piece_len);
             k2 = kb & ~1;
             const int npairs = (ke - k2 + 1) >> 1;
             cnt = (!is_long && npairs > lane) ? (npairs - lane + V - 1) / V : 0;
@@ -164,7 +263,7 @@ __device__ __forceinline__ void batch_rows(const BatchArgs& a, const BatchMat& m
 #pragma unroll
         for (int off = V / 2; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off, V);
         if (row < r1 && lane == 0 && !is_long) y[row] = sum;
-        warp_long_rows(long_mask, kb, ke, row, col, val, x, y, pol);
+        warp_long_rows<D, INLINE>(long_mask, kb, ke, row, col, val, x, y, a.piece_len, pol);
     }
 }
 
@@ -176,6 +275,7 @@ constexpr int kStageEntries = 448;   // per warp: 32 rows x 14 entries
 // DFMA per entry, the FMA loop running the warp's longest short row);
 // otherwise each lane sums its short row straight from global memory.
 // Rows longer than kLongRow are summed afterwards by the whole warp.
+template <int D, bool INLINE>
 __device__ __forceinline__ void batch_rows_staged(const BatchArgs& a, const BatchMat& m, int r0, int r1,
                                                   uint64_t pol, double* sv, int32_t* sc) {
     constexpr int CH = 8;
@@ -241,7 +341,7 @@ __device__ __forceinline__ void batch_rows_staged(const BatchArgs& a, const Batc
             }
         }
         if (row < re && !is_long) y[row] = sum;
-        warp_long_rows(long_mask, kb, ke, row, col, val, x, y, pol);
+        warp_long_rows<D, INLINE>(long_mask, kb, ke, row, col, val, x, y, a.piece_len, pol);
     }
 }
 
@@ -358,45 +458,63 @@ __device__ __forceinline__ void batch_slices(const BatchArgs& a, const BatchMat&
     }
 }
 
-// Long rows at positions [p0, p1) of a matrix's sliced layout, each by the
-// whole warp straight from the CSR arrays.
-__device__ __forceinline__ void batch_long(const BatchArgs& a, const BatchMat& m, int p0, int p1, uint64_t pol) {
-    const int32_t* ptr = a.ptr + m.ptr_off;
-    const int32_t* col = a.col + m.ent_off;
-    const double* val = a.val + m.ent_off;
-    const double* x = a.x + m.row_off;
-    double* y = a.y + m.row_off;
-    for (int pos = p0; pos < p1; ++pos) {
-        const int row = m.s_perm ? __ldg(m.s_perm + pos) : pos;
-        const double t = warp_row(col, val, x, __ldg(ptr + row), __ldg(ptr + row + 1), pol);
-        if ((threadIdx.x & 31) == 0) y[row] = t;
+// Piece item p0 (piece), or the long rows at positions [p0, p1) of a matrix's
+// sliced layout, each by the whole warp straight from the CSR arrays.
+template <int D, bool INLINE>
+__device__ __forceinline__ void batch_long(const BatchArgs& a, const BatchMat& m, bool piece, int p0, int p1,
+                                           uint64_t pol) {
+    if (!INLINE && piece) {
+        const int32_t* ptr = a.ptr + m.ptr_off + a.pieces[p0].row;
+        const int kb = __ldg(ptr) + a.pieces[p0].part * a.piece_len;
+        int ke = __ldg(ptr + 1);
+        if (kb + a.piece_len < ke) ke = kb + a.piece_len;
+        const double t = warp_row<D>(a.col + m.ent_off, a.val + m.ent_off, a.x + m.row_off, kb, ke, pol);
+        publish_piece(a.pieces + p0, a.piece_sum, a.piece_cnt, a.y + m.row_off, t);
+        return;
     }
+    // the rows' numbers and bounds, one row per lane, loaded at once
+    const int pos = p0 + (int)(threadIdx.x & 31);
+    int row = 0, kb = 0, ke = 0;
+    if (pos < p1) {
+        const int32_t* ptr = a.ptr + m.ptr_off;
+        row = m.s_perm ? __ldg(m.s_perm + pos) : pos;
+        kb = __ldg(ptr + row);
+        ke = __ldg(ptr + row + 1);
+    }
+    for (int i = 0; i < p1 - p0; ++i)
+        long_row<D, INLINE>(a.col + m.ent_off, a.val + m.ent_off, a.x + m.row_off, a.y + m.row_off,
+                            __shfl_sync(0xffffffffu, row, i), __shfl_sync(0xffffffffu, kb, i),
+                            __shfl_sync(0xffffffffu, ke, i), a.piece_len, pol);
 }
 
-// Items of the CSR modes (kind 0).
-__device__ __forceinline__ void batch_item(const BatchArgs& a, int it, uint64_t pol, double* sv,
+// A unit of the CSR modes (kind 0) or a piece.
+template <int D, bool INLINE>
+__device__ __forceinline__ void batch_item(const BatchArgs& a, const BatchItem& w, uint64_t pol, double* sv,
                                            int32_t* sc) {
-    const BatchItem w = a.items[it];
     const BatchMat& m = a.mats[w.m];   // fields read where used
+    if (!INLINE && w.kind == 3) {
+        batch_long<D, false>(a, m, true, w.a, w.b, pol);
+        return;
+    }
     switch (m.lanes) {
-        case 0: batch_rows_staged(a, m, w.a, w.b, pol, sv, sc); break;
-        case 1: batch_rows<1>(a, m, w.a, w.b, pol); break;
-        case 2: batch_rows<2>(a, m, w.a, w.b, pol); break;
-        case 4: batch_rows<4>(a, m, w.a, w.b, pol); break;
-        case 8: batch_rows<8>(a, m, w.a, w.b, pol); break;
-        case 16: batch_rows<16>(a, m, w.a, w.b, pol); break;
-        default: batch_rows<32>(a, m, w.a, w.b, pol); break;
+        case 0: batch_rows_staged<D, INLINE>(a, m, w.a, w.b, pol, sv, sc); break;
+        case 1: batch_rows<1, D, INLINE>(a, m, w.a, w.b, pol); break;
+        case 2: batch_rows<2, D, INLINE>(a, m, w.a, w.b, pol); break;
+        case 4: batch_rows<4, D, INLINE>(a, m, w.a, w.b, pol); break;
+        case 8: batch_rows<8, D, INLINE>(a, m, w.a, w.b, pol); break;
+        case 16: batch_rows<16, D, INLINE>(a, m, w.a, w.b, pol); break;
+        default: batch_rows<32, D, INLINE>(a, m, w.a, w.b, pol); break;
     }
 }
 
-// Items of the sliced layout (kinds 1 and 2).
-__device__ __forceinline__ void batch_item_sliced(const BatchArgs& a, int it, uint64_t pol) {
-    const BatchItem w = a.items[it];
+// A unit of the sliced layout (kinds 1 and 2) or a piece.
+template <int D, bool INLINE>
+__device__ __forceinline__ void batch_item_sliced(const BatchArgs& a, const BatchItem& w, uint64_t pol) {
     const BatchMat& m = a.mats[w.m];   // fields read where used
-    if (w.kind == 1)
-        batch_long(a, m, w.a, w.b, pol);
-    else
+    if (w.kind == 2)
         batch_slices(a, m, w.a, w.b, pol);
+    else
+        batch_long<D, INLINE>(a, m, w.kind == 3, w.a, w.b, pol);
 }
 
 // Fill the sliced layout of one matrix from its CSR arrays: one warp per
@@ -464,10 +582,10 @@ __global__ void __launch_bounds__(256) batch_segment_copy_kernel(const int64_t* 
     }
 }
 
-// Persistent: every warp claims whole items (order[0 .. n_items)) with an
-// atomic ticket until none is left (no block-wide barrier: warps never wait
-// for each other).  One kernel for the CSR modes (shared-memory slices for
-// the staged mode), one for the sliced layout (no shared memory).
+// Persistent: every warp claims units (units[0 .. n_units)) with an atomic
+// ticket until none is left (no block-wide barrier: warps never wait for each
+// other).  One kernel for the CSR modes (shared-memory slices for the staged
+// mode), one for the sliced layout (no shared memory).
 __global__ void __launch_bounds__(kThreads, 4) batch_persistent_kernel(BatchArgs a) {
     __shared__ double s_val[kThreads / 32][kStageEntries];
     __shared__ int32_t s_col[kThreads / 32][kStageEntries];
@@ -477,8 +595,9 @@ __global__ void __launch_bounds__(kThreads, 4) batch_persistent_kernel(BatchArgs
         int t = 0;
         if ((threadIdx.x & 31) == 0) t = atomicAdd(a.ticket, 1);
         t = __shfl_sync(0xffffffffu, t, 0);
-        if (t >= a.n_items) break;
-        batch_item(a, __ldg(a.order + t), pol, s_val[w], s_col[w]);
+        if (t >= a.n_units) break;
+        const BatchItem u = a.units[t];
+        batch_item<4, false>(a, u, pol, s_val[w], s_col[w]);
     }
 }
 
@@ -488,8 +607,34 @@ __global__ void __launch_bounds__(kThreads, 6) batch_sliced_persistent_kernel(Ba
         int t = 0;
         if ((threadIdx.x & 31) == 0) t = atomicAdd(a.ticket, 1);
         t = __shfl_sync(0xffffffffu, t, 0);
-        if (t >= a.n_items) break;
-        batch_item_sliced(a, __ldg(a.order + t), pol);
+        if (t >= a.n_units) break;
+        const BatchItem u = a.units[t];
+        batch_item_sliced<4, false>(a, u, pol);
+    }
+}
+
+// Small batches: the units dealt to the warps of one wave in claim order, with
+// no ticket (nothing to reset before the launch, no atomic before the first
+// load) and with 128 registers a thread for the long rows' deep rounds: what
+// such a launch takes is the chain of dependent loads of its longest unit,
+// not bandwidth.
+__global__ void __launch_bounds__(kThreads, 2) batch_small_kernel(BatchArgs a) {
+    __shared__ double s_val[kThreads / 32][kStageEntries];
+    __shared__ int32_t s_col[kThreads / 32][kStageEntries];
+    const uint64_t pol = policy_evict_last();
+    const int w = threadIdx.x >> 5;
+    for (int t = (int)blockIdx.x * (kThreads / 32) + w; t < a.n_units; t += (int)gridDim.x * (kThreads / 32)) {
+        const BatchItem u = a.units[t];
+        batch_item<16, false>(a, u, pol, s_val[w], s_col[w]);
+    }
+}
+
+__global__ void __launch_bounds__(kThreads, 2) batch_sliced_small_kernel(BatchArgs a) {
+    const uint64_t pol = policy_evict_last();
+    for (int t = (int)blockIdx.x * (kThreads / 32) + (int)(threadIdx.x >> 5); t < a.n_units;
+         t += (int)gridDim.x * (kThreads / 32)) {
+        const BatchItem u = a.units[t];
+        batch_item_sliced<16, false>(a, u, pol);
     }
 }
 
@@ -501,14 +646,14 @@ __global__ void __launch_bounds__(kThreads, 4) batch_range_kernel(BatchArgs a, i
     const int w = threadIdx.x >> 5;
     const int nw = (int)gridDim.x * (kThreads / 32);
     for (int it = first + (int)blockIdx.x * (kThreads / 32) + w; it < last; it += nw)
-        batch_item(a, it, pol, s_val[w], s_col[w]);
+        batch_item<4, true>(a, a.items[it], pol, s_val[w], s_col[w]);
 }
 
 __global__ void __launch_bounds__(kThreads, 4) batch_sliced_range_kernel(BatchArgs a, int first, int last) {
     const uint64_t pol = policy_evict_last();
     const int nw = (int)gridDim.x * (kThreads / 32);
     for (int it = first + (int)blockIdx.x * (kThreads / 32) + (int)(threadIdx.x >> 5); it < last; it += nw)
-        batch_item_sliced(a, it, pol);
+        batch_item_sliced<4, true>(a, a.items[it], pol);
 }
 
 }  // namespace
@@ -544,50 +689,95 @@ void brelease(spmv_batch* b, void* p, size_t bytes) {
         }
 }
 
-// Item table of the current modes: each matrix's CSR or sliced items, and
-// the claim order of the persistent launch (items of long rows first: they
-// are the heaviest, so they do not end up in the tail).
+// Estimated work of `rows` long rows (or pieces) of `entries` in all: their
+// entries (weighted for the gathers) plus 8 per row.
+int64_t long_cost(int64_t entries, int64_t rows) { return entries + entries / 2 + 8 * rows; }
+
+// Largest power of two in [1, most] that is at most v.
+int pow2_at_most(int64_t v, int most) {
+    int p = 1;
+    while (p < most && 2 * (int64_t)p <= v) p *= 2;
+    return p;
+}
+
+// How coarse a batch's pieces and long-row units are: 1, 2 or 4.  Finer ones
+// end a launch sooner, coarser ones spend fewer claims and publications on the
+// same entries, and a batch with more rows for every warp in flight (48 per
+// SM) needs less of the first.  Measured (24 to 48 matrices of the batch mix,
+// sliced layout) with pieces of 512 / 1024 / 2048 entries: 0.5 M rows 42.8 /
+// 43.1 / 47.1 us, 4.4 M rows 173 / 167 / 165 us, 22 M rows 554 / 529 / 521 us.
+int grain_of(const spmv_batch* b) { return pow2_at_most(b->total_rows / ((int64_t)b->num_sms * 48 * 128), 4); }
+
+// A work unit of the launches: what one warp takes at once, with its estimated work.
+struct Unit {
+    BatchItem w;
+    int64_t cost;
+};
+
+// Tables of the current modes: each matrix's CSR or sliced items, and the
+// work units of the launches in claim order.  A unit is an item or, so that a
+// small batch still fills the chip's warps, a part of one.
 void upload_items(spmv_batch* b) {
     std::vector<BatchItem> all;
-    std::vector<int64_t> cost;   // estimated work per item (entries plus 8 per row)
     b->item_off.assign(b->count + 1, 0);
+    int64_t n_slices = 0, csr_rows = 0;
     for (int m = 0; m < b->count; ++m) {
         b->item_off[m] = (int)all.size();
         const bool sl = b->mats[m].lanes == kSliced;
         const auto& src = sl ? b->sliced_items[m] : b->csr_items[m];
-        const auto& cst = sl ? b->sliced_cost[m] : b->csr_cost[m];
         all.insert(all.end(), src.begin(), src.end());
-        cost.insert(cost.end(), cst.begin(), cst.end());
+        if (sl) n_slices += b->mats[m].n_slices;
+        else csr_rows += b->n[m];
     }
-    b->item_off[b->count] = (int)all.size();
+    b->item_off[b->count] = b->n_items = (int)all.size();
+    // rows of a CSR unit: as many (16, one pass of two lanes a row, to 256, an
+    // item) as leave 8 units for every warp in flight; 2 units for each took
+    // 279 us against 264 us at 4.4 M rows and 106 us against 97 us at 1.5 M
+    const int64_t warps = (int64_t)b->num_sms * 32;
+    const int rows_per = 16 * pow2_at_most(csr_rows / (16 * 8 * warps), kItemRows / 16);
+    // slices of a sliced unit: 1 below 12 slices for every warp in flight
+    // (6.4: 81 us against 97 us with 2), else 8 (18.8: 161 us against 168 us
+    // with 4, 171 us with 2)
+    const int slices_per = n_slices < 12 * (int64_t)b->num_sms * 48 ? 1 : 8;
+    // long rows of a unit: 4, or 16 in the largest batches (an item's 32, one
+    // after another, were what small launches waited for: 59 us against 25 us
+    // for 12 matrices of up to 30000 rows)
+    const int longs_per = 4 * grain_of(b);
     // claim order: matrix by matrix, so that the warps in flight share a
-    // few matrices' x in L2 (taking heavy items of every matrix first would
+    // few matrices' x in L2 (taking heavy units of every matrix first would
     // spread the gathers over all of them); within a matrix its heaviest
-    // items (the long rows) first, so they do not end up in the tail
-    b->order.clear();
-    for (int i = 0; i < (int)all.size(); ++i)
-        if (all[i].kind != 0) b->order.push_back(i);
-    b->n_sliced_items = (int)b->order.size();
-    for (int i = 0; i < (int)all.size(); ++i)
-        if (all[i].kind == 0) b->order.push_back(i);
-    auto first = [&](int p, int q) {
-        if (all[p].m != all[q].m) return all[p].m < all[q].m;
-        return cost[p] > cost[q];
-    };
-    std::stable_sort(b->order.begin(), b->order.begin() + b->n_sliced_items, first);
-    std::stable_sort(b->order.begin() + b->n_sliced_items, b->order.end(), first);
-    // where each matrix's items start in either part of the order (the
-    // host-buffer path claims one run of matrices at a time)
-    b->order_off.assign(2 * (b->count + 1), 0);
-    for (int part = 0; part < 2; ++part) {
-        const int lo = part == 0 ? 0 : b->n_sliced_items, hi = part == 0 ? b->n_sliced_items : (int)all.size();
-        int t = lo;
-        for (int m = 0; m <= b->count; ++m) {
-            while (t < hi && all[b->order[t]].m < m) ++t;
-            b->order_off[part * (b->count + 1) + m] = t;
+    // units (the long rows) first, so they do not end up in the tail
+    std::vector<Unit> units[2];   // sliced layout, CSR modes
+    b->unit_off.assign(2 * (b->count + 1), 0);
+    for (int m = 0, piece = 0; m < b->count; ++m) {
+        const int part = b->mats[m].lanes == kSliced ? 0 : 1;
+        std::vector<Unit>& u = units[part];
+        b->unit_off[m] = (int)units[0].size();
+        b->unit_off[b->count + 1 + m] = (int)units[1].size();
+        const size_t first = u.size();
+        for (size_t j = 0; j < b->pieces[m].size(); ++j, ++piece)
+            u.push_back(Unit{{m, 3, piece, piece + 1}, long_cost(b->piece_len, 1)});
+        const auto& items = part == 0 ? b->sliced_items[m] : b->csr_items[m];
+        const auto& cost = part == 0 ? b->sliced_cost[m] : b->csr_cost[m];
+        for (size_t i = 0; i < items.size(); ++i) {
+            const BatchItem w = items[i];
+            const int per = w.kind == 0 ? rows_per : w.kind == 1 ? longs_per : slices_per;
+            for (int a = w.a; a < w.b; a += per) {
+                const int e = std::min(w.b, a + per);
+                u.push_back(Unit{{m, w.kind, a, e}, cost[i] * (e - a) / (w.b - w.a)});
+            }
         }
+        std::stable_sort(u.begin() + (long)first, u.end(), [](const Unit& p, const Unit& q) { return p.cost > q.cost; });
     }
-    // the whole-batch launch takes the sliced items of the length-sorted
+    b->unit_off[b->count] = b->n_sliced_units = (int)units[0].size();
+    b->unit_off[2 * b->count + 1] = (int)units[1].size();
+    b->n_units = (int)(units[0].size() + units[1].size());
+    for (int m = 0; m <= b->count; ++m) b->unit_off[b->count + 1 + m] += b->n_sliced_units;
+    std::vector<BatchItem> order;
+    order.reserve((size_t)b->n_units);
+    for (const auto& part : units)
+        for (const Unit& u : part) order.push_back(u.w);
+    // the whole-batch launch takes the sliced units of the length-sorted
     // matrices (skewed rows: bound by their scattered x gathers) and of the
     // natural-order ones (stencils: bound by streaming from HBM) side by
     // side, each run advancing at the same share of its estimated work, so
@@ -595,49 +785,39 @@ void upload_items(spmv_batch* b) {
     // mix: 864 us against 894 us; weighting the gather-bound work 1.6 or 2
     // times made no difference); each run keeps the matrix-by-matrix order
     // above, and the host-buffer path keeps that order itself
-    std::vector<int> full(b->order.begin(), b->order.end());
+    std::vector<BatchItem> full(order.begin(), order.begin() + b->n_sliced_units);
     {
-        std::vector<int> ga, st;
+        std::vector<const Unit*> ga, st;
         double ca = 0.0, cs = 0.0;
-        for (int t = 0; t < b->n_sliced_items; ++t) {
-            const int i = b->order[t];
-            if (b->mats[all[i].m].s_perm) {
-                ga.push_back(i);
-                ca += (double)cost[i];
-            } else {
-                st.push_back(i);
-                cs += (double)cost[i];
-            }
+        for (const Unit& u : units[0]) {
+            const bool sorted = b->mats[u.w.m].s_perm != nullptr;
+            (sorted ? ga : st).push_back(&u);
+            (sorted ? ca : cs) += (double)u.cost;
         }
         if (!ga.empty() && !st.empty()) {
             size_t ia = 0, is = 0, t = 0;
             double da = 0.0, ds = 0.0;
             while (ia < ga.size() || is < st.size()) {
                 const bool take_a = is >= st.size() || (ia < ga.size() && da * cs <= ds * ca);
-                const int i = take_a ? ga[ia++] : st[is++];
-                (take_a ? da : ds) += (double)cost[i];
-                full[t++] = i;
+                const Unit* u = take_a ? ga[ia++] : st[is++];
+                (take_a ? da : ds) += (double)u->cost;
+                full[t++] = u->w;
             }
         }
     }
-    if (all.size() > b->items_cap) {
-        if (b->d_items) brelease(b, b->d_items, b->items_cap * sizeof(BatchItem));
-        if (b->d_order) brelease(b, b->d_order, b->items_cap * sizeof(int));
-        if (b->d_order_full) brelease(b, b->d_order_full, b->items_cap * sizeof(int));
-        b->items_cap = all.size();
-        b->d_items = balloc(b, b->items_cap * sizeof(BatchItem));
-        b->d_order = static_cast<int*>(balloc(b, b->items_cap * sizeof(int)));
-        b->d_order_full = static_cast<int*>(balloc(b, b->items_cap * sizeof(int)));
-    }
-    b->n_items = (int)all.size();
-    if (!all.empty()) {
-        spmvk::check_cuda(cudaMemcpy(b->d_items, all.data(), all.size() * sizeof(BatchItem), cudaMemcpyHostToDevice),
-                          "items");
-        spmvk::check_cuda(cudaMemcpy(b->d_order, b->order.data(), all.size() * sizeof(int), cudaMemcpyHostToDevice),
-                          "item order");
-        spmvk::check_cuda(cudaMemcpy(b->d_order_full, full.data(), all.size() * sizeof(int), cudaMemcpyHostToDevice),
-                          "item order");
-    }
+    auto put = [&](BatchItem*& d, size_t& cap, const std::vector<BatchItem>& h) {
+        if (h.size() > cap) {
+            if (d) brelease(b, d, cap * sizeof(BatchItem));
+            cap = h.size();
+            d = static_cast<BatchItem*>(balloc(b, cap * sizeof(BatchItem)));
+        }
+        if (!h.empty())
+            spmvk::check_cuda(cudaMemcpy(d, h.data(), h.size() * sizeof(BatchItem), cudaMemcpyHostToDevice),
+                              "work items");
+    };
+    put(b->d_items, b->items_cap, all);
+    put(b->d_units, b->units_cap, order);
+    put(b->d_units_full, b->units_full_cap, full);
 }
 
 // Sliced layout of matrix m.  Natural row order when no row is longer than
@@ -722,10 +902,13 @@ void build_sliced(spmv_batch* b, int m) {
     cost.clear();
     for (int p = 0; p < n_long;) {   // up to 32 long rows or 4096 of their entries
         int e = p;
-        int64_t ent = 0;
-        while (e < n_long && e - p < 32 && ent < 4096) ent += L(e++);
+        int64_t ent = 0, whole = 0;   // whole: the entries that are not left to piece items
+        while (e < n_long && e - p < 32 && ent < 4096) {
+            if (L(e) <= b->piece_len) whole += L(e);
+            ent += L(e++);
+        }
         items.push_back(BatchItem{m, 1, p, e});
-        cost.push_back(ent + ent / 2 + 8 * (e - p));
+        cost.push_back(long_cost(whole, e - p));
         p = e;
     }
     for (int s0 = 0; s0 < (int)sl.size();) {   // up to 8 slices or 4096 padded slots
@@ -865,15 +1048,43 @@ BatchArgs args_of(spmv_batch* b, const double* x, double* y) {
     a.col = b->col;
     a.val = b->val;
     a.mats = b->d_mats;
-    a.items = static_cast<const BatchItem*>(b->d_items);
-    a.order = b->d_order;
+    a.items = b->d_items;
+    a.units = b->d_units;
     a.x = x;
     a.y = y;
-    a.n_items = b->n_items;
+    a.n_units = b->n_units;
+    a.piece_len = b->piece_len;
+    a.pieces = b->d_pieces;
+    a.piece_sum = b->piece_sum[0];
+    a.piece_cnt = b->piece_cnt[0];
     a.ticket = b->ticket;
     return a;
 }
 
+// Whether `units` units are launched through the small kernels: up to two for
+// every warp that those keep in flight (12 matrices of up to 30000 rows,
+// sliced: 21 us against 25 us when the line lay at one, 62 us with whole items
+// claimed by ticket).
+bool small_launch(const spmv_batch* b, int units) {
+    return units <= 2 * b->num_sms * 2 * (kThreads / 32);
+}
+
+// Launch of a's n_units units (a.units, a.ticket set; the ticket is zero).
+void launch_units(const spmv_batch* b, const BatchArgs& a, bool sliced, cudaStream_t s) {
+    const bool small = small_launch(b, a.n_units);
+    int grid = b->num_sms * (small ? 2 : std::max(1, sliced ? b->occupancy_sliced : b->occupancy));
+    const int need = (a.n_units + kThreads / 32 - 1) / (kThreads / 32);
+    if (grid > need) grid = need;
+    if (sliced && small)
+        batch_sliced_small_kernel<<<grid, kThreads, 0, s>>>(a);
+    else if (sliced)
+        batch_sliced_persistent_kernel<<<grid, kThreads, 0, s>>>(a);
+    else if (small)
+        batch_small_kernel<<<grid, kThreads, 0, s>>>(a);
+    else
+        batch_persistent_kernel<<<grid, kThreads, 0, s>>>(a);
+    spmvk::check_cuda(cudaGetLastError(), "batch launch");
+}
 }  // namespace
 
 #define BATCH_TRY try {
@@ -922,7 +1133,9 @@ void batch_host_product(spmv_batch* b, const double* x_host, double* y_host, dou
     // goes back on s_out while later chunks are still moving or computing.
     // Issued phase by phase (all copies in, all products, all copies out) so
     // that streams sharing a hardware queue never hold a copy behind a wait.
-    const BatchArgs a = args_of(b, xd, yd);
+    BatchArgs a = args_of(b, xd, yd);
+    a.piece_sum = b->piece_sum[1];
+    a.piece_cnt = b->piece_cnt[1];
     struct Chunk {
         int m0, m1;
         long long r0, r1;
@@ -945,7 +1158,7 @@ void batch_host_product(spmv_batch* b, const double* x_host, double* y_host, dou
                               "copy x in");
         spmvk::check_cuda(cudaEventRecord(b->io_ev[2 * c], s_in), "event");
     }
-    // each chunk's items are a contiguous run of the claim order (per
+    // each chunk's units are a contiguous run of the claim order (per
     // layout), run by the persistent kernels with a ticket of their own
     if (y_free) spmvk::check_cuda(cudaStreamWaitEvent(s_compute, y_free, 0), "wait");
     spmvk::check_cuda(cudaMemsetAsync(b->io_tickets, 0, (size_t)4 * ch.size() * sizeof(int), s_compute),
@@ -954,20 +1167,13 @@ void batch_host_product(spmv_batch* b, const double* x_host, double* y_host, dou
     for (size_t c = 0; c < ch.size(); ++c) {
         spmvk::check_cuda(cudaStreamWaitEvent(s_compute, b->io_ev[2 * c], 0), "wait");
         for (int part = 0; part < 2; ++part) {
-            const int o0 = b->order_off[part * cp1 + ch[c].m0], o1 = b->order_off[part * cp1 + ch[c].m1];
+            const int o0 = b->unit_off[part * cp1 + ch[c].m0], o1 = b->unit_off[part * cp1 + ch[c].m1];
             if (o1 <= o0) continue;
             BatchArgs pa = a;
-            pa.order = b->d_order + o0;
-            pa.n_items = o1 - o0;
+            pa.units = b->d_units + o0;
+            pa.n_units = o1 - o0;
             pa.ticket = b->io_tickets + 4 * c + 2 * part;
-            int grid = b->num_sms * std::max(1, part == 0 ? b->occupancy_sliced : b->occupancy);
-            const int need = (o1 - o0 + kThreads / 32 - 1) / (kThreads / 32);
-            if (grid > need) grid = need;
-            if (part == 0)
-                batch_sliced_persistent_kernel<<<grid, kThreads, 0, s_compute>>>(pa);
-            else
-                batch_persistent_kernel<<<grid, kThreads, 0, s_compute>>>(pa);
-            spmvk::check_cuda(cudaGetLastError(), "chunk launch");
+            launch_units(b, pa, part == 0, s_compute);
         }
         spmvk::check_cuda(cudaEventRecord(b->io_ev[2 * c + 1], s_compute), "event");
     }
@@ -1038,6 +1244,22 @@ int spmv_batch_create(int count, const int64_t* n, const int64_t* const* row_ptr
     b->csr_cost.assign(count, {});
     b->sliced_cost.assign(count, {});
     b->sliced_built.assign(count, 0);
+    b->pieces.assign(count, {});
+    b->piece_len = 512 * grain_of(b);
+    std::vector<BatchPiece> pieces;
+    size_t slots = 0, cut_rows = 0;
+    for (int m = 0; m < count; ++m) {
+        for (int64_t i = 0; i < n[m]; ++i) {
+            const int64_t len = row_ptr[m][i + 1] - row_ptr[m][i];
+            if (len <= b->piece_len) continue;
+            const int np = (int)((len + b->piece_len - 1) / b->piece_len);
+            for (int p = 0; p < np; ++p)
+                b->pieces[m].push_back(BatchPiece{(int)i, p, np, (int)slots, (int)cut_rows});
+            slots += np;
+            ++cut_rows;
+        }
+        pieces.insert(pieces.end(), b->pieces[m].begin(), b->pieces[m].end());
+    }
     for (int m = 0; m < count; ++m) {
         const BatchMat& M = b->mats[m];
         const int64_t base = n[m] > 0 ? row_ptr[m][0] : 0;
@@ -1050,7 +1272,10 @@ int spmv_batch_create(int count, const int64_t* n, const int64_t* const* row_ptr
         for (int64_t r = 0; r < n[m]; r += kItemRows) {
             const int64_t e = std::min<int64_t>(n[m], r + kItemRows);
             b->csr_items[m].push_back(BatchItem{m, 0, (int)r, (int)e});
-            b->csr_cost[m].push_back((row_ptr[m][e] - row_ptr[m][r]) + 8 * (e - r));
+            int64_t whole = 0;   // entries of the rows that are not cut
+            for (int64_t i = r; i < e; ++i)
+                if (row_ptr[m][i + 1] - row_ptr[m][i] <= b->piece_len) whole += row_ptr[m][i + 1] - row_ptr[m][i];
+            b->csr_cost[m].push_back(whole + 8 * (e - r));
         }
     }
     b->ptr = static_cast<int32_t*>(balloc(b, hptr.size() * 4));
@@ -1058,6 +1283,14 @@ int spmv_batch_create(int count, const int64_t* n, const int64_t* const* row_ptr
     b->val = static_cast<double*>(balloc(b, hval.size() * 8));
     b->d_mats = static_cast<BatchMat*>(balloc(b, b->mats.size() * sizeof(BatchMat)));
     b->ticket = static_cast<int*>(balloc(b, 2 * sizeof(int)));
+    b->d_pieces = static_cast<BatchPiece*>(balloc(b, pieces.size() * sizeof(BatchPiece)));
+    for (int set = 0; set < 2; ++set) {
+        b->piece_sum[set] = static_cast<double*>(balloc(b, slots * sizeof(double)));
+        b->piece_cnt[set] = static_cast<int*>(balloc(b, cut_rows * sizeof(int)));   // zeroed
+    }
+    if (!pieces.empty())
+        spmvk::check_cuda(cudaMemcpy(b->d_pieces, pieces.data(), pieces.size() * sizeof(BatchPiece),
+                                     cudaMemcpyHostToDevice), "pieces");
     spmvk::check_cuda(cudaMemcpy(b->ptr, hptr.data(), hptr.size() * 4, cudaMemcpyHostToDevice), "upload");
     spmvk::check_cuda(cudaMemcpy(b->col, hcol.data(), hcol.size() * 4, cudaMemcpyHostToDevice), "upload");
     spmvk::check_cuda(cudaMemcpy(b->val, hval.data(), hval.size() * 8, cudaMemcpyHostToDevice), "upload");
@@ -1123,7 +1356,7 @@ int spmv_batch_query(const spmv_batch* b, int what, int m, int64_t* out) {
         case SPMV_BQ_TOTAL_NNZ: *out = b->total_nnz; break;
         case SPMV_BQ_ITEMS: *out = b->n_items; break;
         case SPMV_BQ_LAUNCHES:
-            *out = (b->n_sliced_items > 0) + (b->n_items > b->n_sliced_items);
+            *out = (b->n_sliced_units > 0) + (b->n_units > b->n_sliced_units);
             break;
         case SPMV_BQ_ALG_BYTES:
             // entries, row pointers, x read, y written, over every matrix
@@ -1149,29 +1382,21 @@ int spmv_batch_run(spmv_batch* b, const double* x, double* y, cudaStream_t s) {
     BATCH_TRY
     if (!b) spmvk::fail(SPMV_EINVAL, "batch is NULL");
     if (b->total_rows > 0 && (!x || !y)) spmvk::fail(SPMV_EINVAL, "x_dev or y_dev is NULL");
-    if (b->n_items == 0) return SPMV_OK;
-    spmvk::check_cuda(cudaMemsetAsync(b->ticket, 0, 2 * sizeof(int), s), "ticket reset");
-    const int n_sl = b->n_sliced_items, n_csr = b->n_items - b->n_sliced_items;
+    if (b->n_units == 0) return SPMV_OK;
+    const int n_sl = b->n_sliced_units, n_csr = b->n_units - b->n_sliced_units;
+    if (!small_launch(b, n_sl) || !small_launch(b, n_csr))
+        spmvk::check_cuda(cudaMemsetAsync(b->ticket, 0, 2 * sizeof(int), s), "ticket reset");
+    BatchArgs a = args_of(b, x, y);
     if (n_sl > 0) {
-        BatchArgs a = args_of(b, x, y);
-        a.order = b->d_order_full;
-        a.n_items = n_sl;
-        int grid = b->num_sms * std::max(1, b->occupancy_sliced);
-        const int need = (n_sl + kThreads / 32 - 1) / (kThreads / 32);
-        if (grid > need) grid = need;
-        batch_sliced_persistent_kernel<<<grid, kThreads, 0, s>>>(a);
-        spmvk::check_cuda(cudaGetLastError(), "batch launch (sliced)");
+        a.units = b->d_units_full;
+        a.n_units = n_sl;
+        launch_units(b, a, true, s);
     }
     if (n_csr > 0) {
-        BatchArgs a = args_of(b, x, y);
-        a.order += n_sl;
-        a.n_items = n_csr;
-        a.ticket += 1;
-        int grid = b->num_sms * std::max(1, b->occupancy);
-        const int need = (n_csr + kThreads / 32 - 1) / (kThreads / 32);
-        if (grid > need) grid = need;
-        batch_persistent_kernel<<<grid, kThreads, 0, s>>>(a);
-        spmvk::check_cuda(cudaGetLastError(), "batch launch");
+        a.units = b->d_units + n_sl;
+        a.n_units = n_csr;
+        a.ticket = b->ticket + 1;
+        launch_units(b, a, false, s);
     }
     BATCH_CATCH
     return SPMV_OK;

@@ -39,16 +39,25 @@ struct BatchMat {
 };
 
 // Work item: kind 0 = rows [a, b) in CSR form; kind 1 = positions [a, b)
-// of long rows (sliced layout); kind 2 = slices [a, b) (sliced layout).
+// of long rows (sliced layout); kind 2 = slices [a, b) (sliced layout);
+// kind 3 = piece a (b = a + 1) of a row that kinds 0 and 1 leave out.
 struct BatchItem {
     int m, kind, a, b;
+};
+
+// Piece `part` of `nparts` of a row longer than the batch's piece length L:
+// its entries [L part, L (part + 1)).  Its sum goes to slot
+// first + part; the warp that finishes the row's last piece (counter cidx)
+// adds the slots in a fixed order.
+struct BatchPiece {
+    int row, part, nparts, first, cidx;
 };
 
 }  // namespace spmvk
 
 struct spmv_batch {
     int device = 0, num_sms = 0, occupancy = 0, occupancy_sliced = 0;
-    int n_sliced_items = 0;              // leading entries of `order` that are sliced-layout items
+    int n_sliced_units = 0;              // leading units of d_units: those of sliced matrices
     int count = 0;
     std::vector<spmvk::BatchMat> mats;   // host copy
     std::vector<int64_t> n;              // rows per matrix
@@ -56,17 +65,16 @@ struct spmv_batch {
     std::vector<int> item_off;           // count+1 item offsets per matrix
     std::vector<std::vector<spmvk::BatchItem>> csr_items, sliced_items;   // per matrix
     std::vector<std::vector<int64_t>> csr_cost, sliced_cost;              // estimated work per item
-    std::vector<int> order;              // claim order of the persistent launch
     std::vector<char> sliced_built;      // per matrix
-    int* d_order = nullptr;
-    int* d_order_full = nullptr;         // claim order of a whole-batch launch (sliced items interleaved)
-    size_t items_cap = 0;                // capacity of d_items / d_order (items)
+    spmvk::BatchItem* d_items = nullptr; // the items, matrix by matrix
+    spmvk::BatchItem* d_units = nullptr; // work units (items or parts of them, and pieces) in claim order
+    spmvk::BatchItem* d_units_full = nullptr;   // of a whole-batch launch (sliced matrices interleaved)
+    size_t items_cap = 0, units_cap = 0, units_full_cap = 0;   // their capacities
     long long total_rows = 0, total_nnz = 0;
     int32_t* ptr = nullptr;
     int32_t* col = nullptr;
     double* val = nullptr;
     spmvk::BatchMat* d_mats = nullptr;
-    void* d_items = nullptr;
     int* ticket = nullptr;
     double* io_x = nullptr;              // device vectors of the host-buffer path (built on first use)
     double* io_y = nullptr;
@@ -74,8 +82,17 @@ struct spmv_batch {
     double* io_y2 = nullptr;
     std::vector<cudaEvent_t> io_ev;      // per chunk (64): x arrived, y computed; then x free, y free per pair
     int* io_tickets = nullptr;           // per chunk: a ticket per layout (4 ints)
-    std::vector<int> order_off;          // 2 x (count+1): start of matrix m's items in each part of `order`
-    int n_items = 0;
+    std::vector<int> unit_off;           // 2 x (count+1): start of matrix m's units in each part of d_units
+    int n_items = 0;                     // items (kinds 0 to 2)
+    int n_units = 0;                     // work units
+    // the pieces of each matrix's cut rows (the same in every layout), their
+    // partial sums and counters (zero between launches): one set for
+    // spmv_batch_run, one for the host-buffer path
+    int piece_len = 0;
+    std::vector<std::vector<spmvk::BatchPiece>> pieces;
+    spmvk::BatchPiece* d_pieces = nullptr;
+    double* piece_sum[2] = {nullptr, nullptr};
+    int* piece_cnt[2] = {nullptr, nullptr};
     size_t device_bytes = 0;
     std::vector<void*> allocs;
     // CSR released (spmv_batch_release_csr): ptr/col/val then hold only the
