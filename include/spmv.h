@@ -381,18 +381,18 @@ int spmv_apply_host_many(spmv_part* part, int64_t count, const double* x_host, i
 
 /*
  * Plain CSR product y = A x on caller-owned DEVICE arrays with the
- * merge-path kernel (equal work per CTA whatever the row lengths; rows cut
- * between threads or CTAs are finished in a fixed order, so y is
+ * merge-path kernel (equal work per warp whatever the row lengths; rows cut
+ * between lanes or warps are finished in a fixed order, so y is
  * deterministic).  row_ptr_dev: int32[n+1] with row_ptr[0] = 0 and
  * row_ptr[n] = nnz, non-decreasing; col_idx_dev: int32[nnz] in [0, n);
  * vals_dev: double[nnz]; x_dev, y_dev: double[n]; every array 16-byte
- * aligned.  The arrays are read only inside their bounds.  Scratch: 48 bytes
- * per 2048 merge items (rows + entries), taken with cudaMallocAsync on s and
- * released with cudaFreeAsync on s.  Preconditions on the CSR contents are
- * the caller's: they are not checked on the device.
+ * aligned.  The arrays are read only inside their bounds.  Scratch: 16 bytes
+ * for each of at most 4864 ranges of merge items (rows + entries), taken with
+ * cudaMallocAsync on s and released with cudaFreeAsync on s.  Preconditions on
+ * the CSR contents are the caller's: they are not checked on the device.
  * Errors: SPMV_EINVAL (sizes, NULL or misaligned pointers), SPMV_EBOUNDS
- * (n + nnz >= 2^31 - 2048), SPMV_ENOMEM, SPMV_ECUDA.  A bounded device
- * wait that gives up is reported by spmv_csr_error.
+ * (n + nnz >= 2^31 - 2048), SPMV_ENOMEM, SPMV_ECUDA.  A launch that gives up
+ * (spmv_selftest_merge_abort) is reported by spmv_csr_error.
  */
 int spmv_csr_merge(int64_t n, int64_t nnz, const int32_t* row_ptr_dev,
                    const int32_t* col_idx_dev, const double* vals_dev,
@@ -400,17 +400,16 @@ int spmv_csr_merge(int64_t n, int64_t nnz, const int32_t* row_ptr_dev,
 
 /*
  * spmv_csr_merge without any allocation: the same product, kernels and
- * result as spmv_csr_merge, with its scratch (tile coordinates and row
- * carries) in a fixed array compiled into the library instead of memory
+ * result as spmv_csr_merge, with its scratch (row carries) in a fixed array compiled into the library instead of memory
  * taken at call time.  The paper has no counterpart; this entry point is for
  * callers that must not allocate device memory during a call: code that
  * runs inside a host application owning every device allocation through its
  * own fixed pool, latency-bound loops where an allocation may synchronise
  * or grow a pool at an unpredictable moment, and work recorded into a CUDA
  * graph whose owner does not accept memory-allocation nodes.
- *   Limit: n + nnz <= 134 217 728 (65 536 tiles of 2048 merge items); larger
- *   inputs fail with SPMV_EBOUNDS before anything is launched.  The array
- *   takes 3 MiB on every GPU that loads the library, until the process exits.
+ *   Limit: n + nnz <= 134 217 728 merge items; larger inputs fail with
+ *   SPMV_EBOUNDS before anything is launched.  The array takes 76 KiB on every
+ *   GPU that loads the library, until the process exits.
  *   Set-up: the first call on a device looks up the array's device address
  *   (cudaGetSymbolAddress) with that device current; make that first call
  *   before any stream capture.
@@ -640,13 +639,12 @@ int spmv_probe_dfma(int64_t iters, int ctas_per_sm, int lanes, double* out_dev, 
 int spmv_probe_gather(const double* table_dev, const int32_t* idx_dev, int64_t count, int ctas_per_sm,
                       double* out_dev, int64_t out_cap, cudaStream_t s);
 
-/* Test hook of the merge-path kernel's give-up path (the path a bounded wait
- * that runs out takes), for the plan-free entry points spmv_csr_merge and
- * spmv_csr_merge_noalloc: while set (tile >= 0), their launches treat merge
- * tile `tile` and every later tile as if the wait for its staged copy had run
- * out, once that copy has landed (so no copy is left in flight).  Such a
- * launch sets the error word (spmv_csr_error reports 6), leaves the rows of
- * the abandoned tiles unfinished, marks their carries empty and writes nothing
+/* Test hook of the merge-path kernel's give-up path, for the plan-free entry
+ * points spmv_csr_merge and spmv_csr_merge_noalloc: while set (tile >= 0),
+ * their launches abandon range `tile` of the merge path (a launch has at most
+ * 4864, each of 248 merge items or more) and every later one.  Such a launch
+ * sets the error word (spmv_csr_error reports 6), leaves the rows of
+ * the abandoned ranges unfinished, marks their carries empty and writes nothing
  * outside y[0, n).  tile = -1 turns the hook off (the default).  Process-wide;
  * plans are not affected.  SPMV_EINVAL outside [-1, 2^30). */
 int spmv_selftest_merge_abort(int64_t tile);

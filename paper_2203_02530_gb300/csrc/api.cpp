@@ -1179,8 +1179,7 @@ int spmv_csr_merge(int64_t n, int64_t nnz, const int32_t* row_ptr, const int32_t
                    const double* x, double* y, cudaStream_t s) {
     API_TRY
     if (n < 0 || nnz < 0) fail(SPMV_EINVAL, "n = %lld, nnz = %lld", (long long)n, (long long)nnz);
-    const int items = spmvk::merge_items_per_tile();
-    if (n + nnz >= (int64_t(1) << 31) - items) fail(SPMV_EBOUNDS, "n + nnz too large for int32 merge paths");
+    if (n + nnz >= (int64_t(1) << 31) - 2048) fail(SPMV_EBOUNDS, "n + nnz too large for int32 merge paths");
     if (n == 0) return SPMV_OK;
     if (!row_ptr || !x || !y || (nnz > 0 && (!col_idx || !vals))) fail(SPMV_EINVAL, "NULL device pointer");
     const uintptr_t mis = reinterpret_cast<uintptr_t>(row_ptr) | reinterpret_cast<uintptr_t>(col_idx) |
@@ -1190,12 +1189,9 @@ int spmv_csr_merge(int64_t n, int64_t nnz, const int32_t* row_ptr, const int32_t
     int dev = 0, sms = 0;
     check_cuda(cudaGetDevice(&dev), "cudaGetDevice");
     check_cuda(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "SM count");
-    const int n_tiles = (int)((n + nnz + items - 1) / items);
     void* scratch = nullptr;
-    const size_t tile_bytes = (size_t)n_tiles * sizeof(spmvk::MergeTile);
-    check_cuda(cudaMallocAsync(&scratch, tile_bytes + (size_t)n_tiles * sizeof(spmvk::Carry), s), "cudaMallocAsync");
-    spmvk::MergeTile* tiles = static_cast<spmvk::MergeTile*>(scratch);
-    spmvk::Carry* carries = reinterpret_cast<spmvk::Carry*>(static_cast<char*>(scratch) + tile_bytes);
+    check_cuda(cudaMallocAsync(&scratch, (size_t)spmvk::merge_free_ranges(n + nnz) * sizeof(spmvk::Carry), s),
+               "cudaMallocAsync");
     spmvk::CsrArgs a{};
     a.ptr = row_ptr;
     a.col = col_idx;
@@ -1209,8 +1205,7 @@ int spmv_csr_merge(int64_t n, int64_t nnz, const int32_t* row_ptr, const int32_t
     a.guarded = 1;
     a.err = nullptr;
     a.abort_tile = g_merge_abort_tile.load();
-    cudaError_t e = spmvk::launch_merge_partition(row_ptr, 0, (int)n, 0, tiles, n_tiles, s);
-    if (e == cudaSuccess) e = spmvk::launch_merge(a, tiles, 0, n_tiles, carries, sms, s);
+    cudaError_t e = spmvk::launch_merge_free(a, static_cast<spmvk::Carry*>(scratch), sms, s);
     cudaError_t ef = cudaFreeAsync(scratch, s);
     check_cuda(e, "merge product");
     check_cuda(ef, "cudaFreeAsync");

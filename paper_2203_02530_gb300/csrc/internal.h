@@ -33,7 +33,7 @@ struct TileGeom {
     int rows() const { return threads / lanes; }
 };
 
-// Merge-path tile: merge items [d0, d1) of the (row ends, entries) merge of
+// Merge-path range: merge items [d0, d1) of the (row ends, entries) merge of
 // one rank's CSR; (r0, k0) is the path coordinate at d0, (r1, k1) at d1.
 struct MergeTile {
     int32_t r0, r1, k0, k1;
@@ -41,7 +41,7 @@ struct MergeTile {
 };
 static_assert(sizeof(MergeTile) == 32, "merge tile descriptor is two int4");
 
-// Carry of a row cut by a merge tile boundary.
+// Carry of a row cut by a merge range boundary.
 struct Carry {
     int32_t row;   // row index (in the CSR's row space), -1 when none
     int32_t pad;
@@ -103,8 +103,7 @@ struct CsrArgs {
     int guarded;            // 1: arrays are not padded past their ends
     int* err;               // device error word
     int abort_tile;         // test hook of the merge-path kernel: k > 0 makes
-                            // tiles k-1 and later take the path of a wait that
-                            // ran out (after their copies landed); 0 = never
+                            // ranges k-1 and later give up; 0 = never
     int pdl;                // programmatic-launch flags of the launch
                             // (kPdlNoWait, kPdlEarly; 0 = wait, no early release)
 };
@@ -132,7 +131,10 @@ cudaError_t launch_merge(const CsrArgs& a, const MergeTile* tiles, int tile_begi
                          int tile_end, Carry* carries, int num_sms, cudaStream_t s);
 cudaError_t launch_merge_partition(const int32_t* ptr, int row_begin, int row_end, int32_t xoff,
                                    MergeTile* tiles, int n_tiles, cudaStream_t s);
-int merge_items_per_tile();
+int merge_items_per_tile();   // of a plan's ranges
+// Plan-free merge product: its ranges (one carry each) and its launch.
+int64_t merge_free_ranges(int64_t items);
+cudaError_t launch_merge_free(const CsrArgs& a, Carry* carries, int num_sms, cudaStream_t s);
 cudaError_t read_clear_csr_error(int* out);
 int64_t noalloc_max_items();
 cudaError_t launch_merge_noalloc(const CsrArgs& a, int num_sms, cudaStream_t s);
