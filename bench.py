@@ -563,7 +563,7 @@ def run_ours(args, world, rank, local, fp64=None):
     achieved = alg_local / t_local / 1e9
     kname = {spmv.VARIANT_TILE: "csr_tile_kernel", spmv.VARIANT_VECTOR: "csr_vector_kernel",
              spmv.VARIANT_MERGE: "merge_kernel", spmv.VARIANT_PAIRS: "csr_pair_kernel",
-             spmv.VARIANT_WARP: "csr_warp_kernel", spmv.VARIANT_SELL: "csr_sell_kernel",
+             spmv.VARIANT_WARP: "csr_tile_kernel", spmv.VARIANT_SELL: "csr_sell_kernel",
              spmv.VARIANT_SELL16: "csr_sell_kernel"}[variant]
     traffic = profiled_traffic(args.workload, "%s/%d/%d" % (kname, variant, vparam))
 

@@ -134,7 +134,7 @@ enum {
     SPMV_Q_LAST_WAITS = 15,       /* stream waits issued for DAG edges by the last issue */
     SPMV_Q_ERROR = 16,            /* device error word (0 = none); synchronises */
     SPMV_Q_LOCAL_VARIANT = 17,
-    SPMV_Q_N_LOCAL_TILES = 18,
+    SPMV_Q_N_LOCAL_TILES = 18,    /* 32-row tiles of the LOCAL product */
     SPMV_Q_LAST_LAUNCHES = 19,    /* kernels launched by the last issue */
     SPMV_Q_REMOTE_VARIANT = 20,   /* 100 * variant + param of the REMOTE product
                                      (SPMV_Q_LOCAL_VARIANT: of the LOCAL one) */
@@ -180,17 +180,20 @@ int spmv_part_dag(const spmv_part* part, int32_t* edges_host, int64_t cap_pairs,
 
 /* Kernel variant of the LOCAL and REMOTE products (every variant gives the
  * same y within the FP64 bound; each is deterministic on its own).
- *   TILE   param = geometry 0..4: rows staged in shared memory by bulk
- *          copies, 1 or 2 threads per row (the geometry fixes which)
+ *   TILE   param = geometry 0..4 (8, 14, 4, 7 or 16 x gathers in flight per
+ *          lane): tiles of 32 rows staged in shared memory by bulk copies,
+ *          each by one warp, one thread per row, one DFMA per entry into
+ *          two sums, of the entries at even and at odd places, that are
+ *          added at the end (geometry 3: one sum); rows longer than 64
+ *          entries (and, in a tile with such a row, those longer than 32)
+ *          by the whole warp
  *   VECTOR param = lanes per row (2..32), 4 entries per lane per step with
  *          128-bit loads
  *   PAIRS  param = lanes per row (1, 2, 4, 8), one aligned pair of entries per
  *          lane per step, FMA count = the warp's longest share; 102 / 104:
  *          2 / 4 lanes with fewer pairs in flight and 8 CTAs per SM
  *   MERGE  merge-path split with deterministic carries (param ignored)
- *   WARP   param = geometry 0..4: warp-private shared-memory pipelines of
- *          32-row tiles (bulk copies per warp, no block-wide barrier), one
- *          thread per row, one DFMA per entry
+ *   WARP   param = geometry 0..4 (9, 14, 4, 7 or 16 gathers): as TILE, one sum
  *   SELL   param = 4, 8, 9 (entries per lane per step; 8, 4 and 4 CTAs per
  *          SM) or 104 / 105 / 106 / 107 (4 at 6, 8 at 5, 8 at 6, 9 at 5 CTAs
  *          per SM, in fewer registers), each + 2000 (2004, ..., 2107) for the same

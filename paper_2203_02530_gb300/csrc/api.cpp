@@ -170,15 +170,6 @@ int launch_product(spmv_part* pt, const spmvk::CsrArgs& a, bool remote, int p, c
                    "merge product");
         return me > mb ? 2 : 0;
     }
-    if (var == SPMV_VARIANT_WARP) {
-        const std::vector<int64_t>& wo = remote ? pt->rwtile_off : pt->lwtile_off;
-        const int wb = (int)(p < 0 ? 0 : wo[p]);
-        const int we = (int)(p < 0 ? wo[pt->P] : wo[p + 1]);
-        if (pt->dry_run) return we > wb;
-        check_cuda(spmvk::launch_warp(a, remote ? pt->rwtiles : pt->lwtiles, wb, we, param, pt->num_sms, s),
-                   "warp product");
-        return we > wb;
-    }
     if (var == SPMV_VARIANT_SELL || var == SPMV_VARIANT_SELL16) {
         const spmv_part::SellPart& sp = pt->sell[remote ? 1 : 0];
         spmvk::SellArgs sa{sp.slices, sp.longs, sp.val,  sp.col,         sp.col16,     sp.len, sp.perm,
@@ -219,7 +210,9 @@ int launch_product(spmv_part* pt, const spmvk::CsrArgs& a, bool remote, int p, c
         return be > bb;
     } else {
         if (pt->dry_run) return te > tb;
-        check_cuda(spmvk::launch_tile(a, tiles, tb, te, pt->geom, pt->num_sms, s), "tile product");
+        check_cuda(spmvk::launch_tile(a, tiles, tb, te, var == SPMV_VARIANT_WARP, param, pt->tile_cap[remote ? 1 : 0],
+                                      pt->num_sms, s),
+                   "tile product");
     }
     return te > tb;
 }
@@ -524,7 +517,7 @@ int spmv_part_create(int64_t n, const int64_t* row_ptr, const int32_t* col_idx, 
     check_cuda(cudaGetDevice(&pt->device), "cudaGetDevice");
     check_cuda(cudaDeviceGetAttribute(&pt->num_sms, cudaDevAttrMultiProcessorCount, pt->device), "SM count");
     spmvk::build_plan(pt, n, row_ptr, col_idx, vals);
-    spmvk::build_tiles(pt, spmvk::default_tile_geom());
+    spmvk::build_tiles(pt);
     build_dag(pt);
     *out = pt;
     pt = nullptr;
@@ -767,31 +760,15 @@ static void prepare_variant(spmv_part* pt, int variant, int param, int op_kind) 
     if (pt->csr_released && (variant != SPMV_VARIANT_SELL16 || op_kind != SPMV_OP_LOCAL) &&
         (variant != SPMV_VARIANT_SELL || (op_kind != SPMV_OP_REMOTE && !pt->sell[0].col)))
         spmvk::restore_csr(pt);
-    if (variant == SPMV_VARIANT_TILE) {
-        static const spmvk::TileGeom geoms[] = {{256, 3456, 2, 16, 2},
-                                                {512, 6912, 2, 16, 2},
-                                                {256, 3456, 3, 16, 2},
-                                                {128, 3456, 2, 32, 1},
-                                                {256, 2048, 3, 8, 2}};
-        const int ng = (int)(sizeof geoms / sizeof geoms[0]);
-        if (param < 0 || param >= ng) fail(SPMV_EINVAL, "tile geometry %d not in [0, %d)", param, ng);
-        const spmvk::TileGeom g = geoms[param];
-        if (!spmvk::tile_geom_supported(g)) fail(SPMV_EINVAL, "tile geometry not compiled");
-        check_cuda(cudaDeviceSynchronize(), "synchronize");
-        if (g.rows() != pt->geom.rows() || g.nnz_cap != pt->geom.nnz_cap)
-            spmvk::build_tiles(pt, g);
-        pt->geom = g;
+    if (variant == SPMV_VARIANT_TILE || variant == SPMV_VARIANT_WARP) {
+        if (!spmvk::tile_param_supported(param))
+            fail(SPMV_EINVAL, "%s geometry %d not in [0, 5)", variant == SPMV_VARIANT_TILE ? "tile" : "warp", param);
     } else if (variant == SPMV_VARIANT_VECTOR) {
         if (param != 2 && param != 4 && param != 8 && param != 16 && param != 32)
             fail(SPMV_EINVAL, "vector width %d not in {2,4,8,16,32}", param);
     } else if (variant == SPMV_VARIANT_PAIRS) {
         if (param != 1 && param != 2 && param != 4 && param != 8 && param != 102 && param != 104)
             fail(SPMV_EINVAL, "pair variant %d not in {1,2,4,8,102,104}", param);
-    } else if (variant == SPMV_VARIANT_WARP) {
-        const int cap = spmvk::warp_tile_cap(param);
-        if (cap < 0) fail(SPMV_EINVAL, "warp geometry %d not in [0, 5)", param);
-        check_cuda(cudaDeviceSynchronize(), "synchronize");
-        if (!pt->lwtiles || pt->wtile_cap != cap) spmvk::build_warp_tiles(pt, cap);
     } else if (variant == SPMV_VARIANT_MERGE) {
         check_cuda(cudaDeviceSynchronize(), "synchronize");
         if (!pt->lmtiles) spmvk::build_merge_tiles(pt);

@@ -11,27 +11,17 @@
 
 namespace spmvk {
 
-// Tile of rows processed by one CTA iteration: rows [r0, r1) of a CSR whose
-// entries [k0, k1) are staged in shared memory.  xoff is added to every
-// column index before x is read.  flags: TILE_LONG marks a single row longer
-// than the stage capacity, summed by the whole CTA straight from global
-// memory.
+// Tile of rows [r0, r1) of a CSR with entries [k0, k1); xoff is added to every
+// column index before x is read.  flags (tiles of the staged kernel): TILE_LONG
+// a row longer than kSellLong entries, TILE_WIDE more entries than the stage.
 struct Tile {
     int32_t r0, r1, k0, k1;
     int32_t xoff, flags, pad0, pad1;
 };
 static_assert(sizeof(Tile) == 32, "tile descriptor is two int4");
-enum { TILE_LONG = 1 };
-
-// Geometry of the thread-per-row tile kernel.
-struct TileGeom {
-    int threads;   // threads per CTA
-    int nnz_cap;   // entries per tile stage
-    int stages;    // shared-memory ring depth
-    int chunk;     // x gathers issued together per thread
-    int lanes;     // threads per row; a tile holds threads / lanes rows
-    int rows() const { return threads / lanes; }
-};
+enum { TILE_LONG = 1, TILE_WIDE = 2 };
+constexpr int kTileRows = 32;
+constexpr int kTileMaxEntries = 1792;   // 21.5 KB of stage per warp, 10 warps per SM
 
 // Merge-path range: merge items [d0, d1) of the (row ends, entries) merge of
 // one rank's CSR; (r0, k0) is the path coordinate at d0, (r1, k1) at d1.
@@ -113,13 +103,12 @@ cudaError_t launch_gather(const double* x, const int32_t* idx, const int32_t* po
                           double* dst, int64_t count, int num_sms, cudaStream_t s, int pdl = 0);
 cudaError_t launch_copy(const double* src, double* dst, int64_t count, int num_sms,
                         cudaStream_t s, int pdl = 0);
-cudaError_t launch_tile(const CsrArgs& a, const Tile* tiles, int tile_begin,
-                        int tile_end, const TileGeom& g, int num_sms, cudaStream_t s);
+cudaError_t launch_tile(const CsrArgs& a, const Tile* tiles, int tile_begin, int tile_end, bool one_sum, int param,
+                        int cap, int num_sms, cudaStream_t s);
+bool tile_param_supported(int param);
+int tile_stage_cap(int entries);   // stage size (entries) for tiles of up to `entries`
 cudaError_t launch_vector(const CsrArgs& a, const Tile* tiles, int tile_begin, int tile_end,
                           int lanes, int num_sms, cudaStream_t s);
-cudaError_t launch_warp(const CsrArgs& a, const Tile* tiles, int tile_begin, int tile_end,
-                        int param, int num_sms, cudaStream_t s);
-int warp_tile_cap(int param);
 cudaError_t selftest_wait_timeout(uint64_t limit_ns, int* status_host);
 int probe_threads();
 cudaError_t launch_dfma_probe(int64_t iters, int grid, int lanes, double* out, int64_t* dfma, cudaStream_t s);
@@ -170,8 +159,5 @@ cudaError_t launch_check_sell(const SellSlice* slices, int n_slices, const uint8
 inline bool sell_param_balanced(int param) { return param >= 2000; }
 // CTAs of a sliced launch of `units` work units.
 int sell_grid(int param, int units, int num_sms);
-int tile_ctas_per_sm(const TileGeom& g);
-bool tile_geom_supported(const TileGeom& g);
-TileGeom default_tile_geom();
 
 }  // namespace spmvk

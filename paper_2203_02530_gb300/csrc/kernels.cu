@@ -3,7 +3,7 @@
 // products y_L = A_L x_L and y += A_R x_R.
 //
 // Design for sm_103a: FP64 FMA issues at 2 lanes/clk/SM on this part, so a
-// CSR product with HBM at full speed is nearly FP64-bound.  Every product
+// CSR product with HBM at full speed is nearly FP64-bound.  Every staged product
 // kernel therefore spends exactly one DFMA per stored entry on the main path
 // (one thread walks a row), and gets coalescing from bulk copies
 // (cp.async.bulk, the TMA engine) of whole tiles into a shared-memory ring
@@ -61,17 +61,9 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
     }
     return true;
 }
-// Bulk copy global -> shared (16-byte aligned addresses, size % 16 == 0),
-// completion reported to an mbarrier as transaction bytes.
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes,
-                                         uint32_t bar) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-            dst),
-        "l"(src), "r"(bytes), "r"(bar)
-        : "memory");
-}
-// Bulk copy with an L2 eviction policy (evict-first for data read once).
+// Bulk copy global -> shared (16-byte aligned addresses, size % 16 == 0) with an
+// L2 eviction policy (evict-first for data read once), completion reported to
+// an mbarrier as transaction bytes.
 __device__ __forceinline__ void bulk_g2s_hint(uint32_t dst, const void* src, uint32_t bytes,
                                               uint32_t bar, uint64_t policy) {
     asm volatile(
@@ -198,252 +190,226 @@ cudaError_t launch_copy(const double* src, double* dst, int64_t count, int num_s
 }
 
 // ------------------------------------------------------------------------
-// Thread-per-row CSR product over bulk-copied tiles.
+// Thread-per-row CSR product over bulk-copied tiles (variants TILE and WARP).
 //
-// Persistent CTAs walk tiles tile_begin + blockIdx.x + j * gridDim.x.  One
-// elected thread copies each tile's values, columns and row pointers into a
-// ring of ST shared-memory stages with cp.async.bulk (start addresses rounded
-// down to 16 bytes, sizes rounded up; the device arrays are padded so the
-// rounded reads stay in bounds).  Thread i of the CTA sums row r0 + i of the
-// tile in storage order with one DFMA per entry.
+// A tile is up to 32 consecutive rows of one rank and belongs to one warp,
+// which copies the tile's values and columns (contiguous in the CSR) into its
+// own stage of shared memory with two bulk copies against its own mbarrier
+// (start addresses rounded down to 16 bytes, sizes rounded up; the device
+// arrays are padded so the rounded reads stay in bounds).  Lane i sums row
+// r0 + i in storage order with one DFMA per entry, U gathers of x in flight,
+// into S sums: 1, or 2 (the entries at even and at odd places of the row, added
+// at the end: half the chain of dependent FMAs, and a smaller rounding error).
+// Warps never wait for each other.
+//
+// A tile whose entries do not fit the stage (TILE_WIDE) is summed the same
+// way straight from global memory.  In a tile with a row longer than kSellLong
+// entries (TILE_LONG) every row longer than kTileWarpRow is summed by the
+// whole warp instead (lane l takes entries l, l+32, ..., then a fixed
+// butterfly), so a long row costs its 32nd part.  Each row is summed in a
+// fixed order whatever the grid, the stream or the schedule.
+//
+// What bounds it: HBM and the FP64 pipe once enough warps are resident, and
+// the stages decide how many: one stage per warp, as large as 98 % of the
+// plan's tiles need (27-point stencil: 864 entries, 10.4 KB, 20 warps per SM),
+// where two stages of half as many warps or block-wide tiles of 128 rows took
+// longer.  LOCAL products: 27-point 91^3 (19.9 M entries) 51 us against 77 us
+// with block-wide double-buffered tiles and 71 us with two stages per warp;
+// 7-point 120^3 34 us against 93 us; power-law 1 M rows 126 us against 2600 us
+// (long rows one per thread); 27-point 20^3 4.5 us against 5.0 us.
 // ------------------------------------------------------------------------
-template <int ROWS, int CAP>
-struct TileLayout {
-    static constexpr int VAL_N = CAP + 2;    // doubles: k0 rounded down to even, k1 up
-    static constexpr int COL_N = CAP + 8;    // ints: rounded to multiples of 4
-    static constexpr int PTR_N = ROWS + 8;   // ints: rows r0..r1 inclusive, rounded
-    static constexpr int VAL_OFF = 0;
-    static constexpr int COL_OFF = VAL_N * 8;
-    static constexpr int PTR_OFF = COL_OFF + COL_N * 4;
-    static constexpr int BYTES = PTR_OFF + PTR_N * 4;
-    static_assert(CAP % 4 == 0 && ROWS % 4 == 0, "16-byte aligned stage parts");
-    static_assert(BYTES % 16 == 0, "stage size keeps 16-byte alignment");
+constexpr int kTileWarps = 4;      // warps per CTA
+constexpr int kTileWarpRow = 32;   // in a TILE_LONG tile, longer rows go to the whole warp
+
+struct StageLayout {   // of one warp's stage for up to `cap` entries (a multiple of 32)
+    int col_off, bytes;
+    __host__ __device__ explicit StageLayout(int cap)
+        : col_off((cap + 2) * 8), bytes((cap + 2) * 8 + (cap + 8) * 4) {}
 };
 
-template <int NT, int CAP, int ST, int CH, int LANES>
-__global__ void __launch_bounds__(NT, 1) csr_tile_kernel(CsrArgs a, const Tile* __restrict__ tiles,
-                                                      int tile_begin, int tile_end) {
+template <int U, int S>
+__global__ void __launch_bounds__(kTileWarps * 32, U > 9 ? 8 : 10) csr_tile_kernel(CsrArgs a,
+                                                                                    const Tile* __restrict__ tiles,
+                                                                                    int tile_begin, int tile_end,
+                                                                                    int cap) {
     pdl_begin(a.pdl);  // the previous kernel of this stream is done (unless independent)
-    static_assert(LANES == 1 || LANES == 2 || LANES == 4, "lanes per row");
-    using L = TileLayout<NT / LANES, CAP>;
+    extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ __align__(8) uint64_t bars[kTileWarps];
     const uint64_t pol_stream = policy_evict_first();
     const uint64_t pol_keep = policy_evict_last();
-    extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ __align__(8) uint64_t bars[ST];
-    __shared__ double red[NT];
-
-    const int tid = threadIdx.x;
-    const int first = tile_begin + (int)blockIdx.x;
-    const int stride = (int)gridDim.x;
-
-    if (tid == 0) {
-        for (int s = 0; s < ST; ++s) mbar_init(smem_u32(&bars[s]), 1);
+    const int lane = threadIdx.x & 31;
+    const int w = threadIdx.x >> 5;
+    const StageLayout lay(cap);
+    unsigned char* stage = smem + (size_t)w * lay.bytes;
+    const double* vs = reinterpret_cast<const double*>(stage);
+    const int32_t* cs = reinterpret_cast<const int32_t*>(stage + lay.col_off);
+    const uint32_t bar = smem_u32(&bars[w]);
+    if (lane == 0) {
+        mbar_init(bar, 1);
         mbar_fence_init();
     }
-    __syncthreads();
-
-    // Producer: thread 0 issues the copies of the j-th tile of this CTA.
-    auto issue = [&](int j) {
-        const int t = first + j * stride;
-        if (t >= tile_end) return;
-        const int s = j % ST;
+    __syncwarp();
+    uint32_t parity = 0;
+    for (int t = tile_begin + (int)blockIdx.x * kTileWarps + w; t < tile_end; t += (int)gridDim.x * kTileWarps) {
         const Tile d = tiles[t];
-        const uint32_t bar = smem_u32(&bars[s]);
-        if (d.flags & TILE_LONG) {
-            mbar_arrive_expect_tx(bar, 0);
-            return;
+        const bool staged = d.flags == 0;
+        const int va = d.k0 & ~1, ca = d.k0 & ~3;
+        if (staged && lane == 0) {
+            fence_proxy_async_smem();   // the stage was read by the warp before
+            const uint32_t vbytes = (uint32_t)(((d.k1 + 1) & ~1) - va) * 8u;
+            const uint32_t cbytes = (uint32_t)(((d.k1 + 3) & ~3) - ca) * 4u;
+            mbar_arrive_expect_tx(bar, vbytes + cbytes);
+            if (vbytes) bulk_g2s_hint(smem_u32(stage), a.val + va, vbytes, bar, pol_stream);
+            if (cbytes) bulk_g2s_hint(smem_u32(stage + lay.col_off), a.col + ca, cbytes, bar, pol_stream);
         }
-        const int va = d.k0 & ~1, vb = (d.k1 + 1) & ~1;
-        const int ca = d.k0 & ~3, cb = (d.k1 + 3) & ~3;
-        const int pa = d.r0 & ~3, pb = (d.r1 + 4) & ~3;
-        const uint32_t vbytes = (uint32_t)(vb - va) * 8u;
-        const uint32_t cbytes = (uint32_t)(cb - ca) * 4u;
-        const uint32_t pbytes = (uint32_t)(pb - pa) * 4u;
-        unsigned char* st = smem + (size_t)s * L::BYTES;
-        mbar_arrive_expect_tx(bar, vbytes + cbytes + pbytes);
-        if (vbytes) bulk_g2s_hint(smem_u32(st + L::VAL_OFF), a.val + va, vbytes, bar, pol_stream);
-        if (cbytes) bulk_g2s_hint(smem_u32(st + L::COL_OFF), a.col + ca, cbytes, bar, pol_stream);
-        bulk_g2s_hint(smem_u32(st + L::PTR_OFF), a.ptr + pa, pbytes, bar, pol_stream);
-    };
-
-    if (tid == 0) {
-        for (int j = 0; j < ST - 1; ++j) issue(j);
-    }
-
-    int j = 0;
-    bool aborted = false;
-    for (;; ++j) {
-        const int t = first + j * stride;
-        if (t >= tile_end) break;
-        if (tid == 0) {
-            // stage (j-1) % ST was released by the barrier that ended j-1
-            fence_proxy_async_smem();
-            issue(j + ST - 1);
-        }
-        const int s = j % ST;
-        const bool ok = mbar_wait_bounded(smem_u32(&bars[s]), (uint32_t)((j / ST) & 1), kWaitLimitNs);
-        // every thread leaves together if any wait gave up
-        if (__syncthreads_or(!ok)) {
-            aborted = true;
-            break;
-        }
-        const Tile d = tiles[t];
-        {
-            if (d.flags & TILE_LONG) {
-                // one row longer than a stage: the CTA sums it from global
-                // memory with a fixed-order tree, so the result is still
-                // independent of the launch.
-                const double* xb = a.x + d.xoff;
-                double part = 0.0;
-                for (int k = d.k0 + tid; k < d.k1; k += NT)
-                    part = fma(__ldg(a.val + k), __ldg(xb + __ldg(a.col + k)), part);
-                red[tid] = part;
-                __syncthreads();
-                for (int w = NT / 2; w > 0; w >>= 1) {
-                    if (tid < w) red[tid] += red[tid + w];
-                    __syncthreads();
+        const int row = d.r0 + lane;
+        const bool live = row < d.r1;
+        const int kb = live ? __ldg(a.ptr + row) : 0;
+        const int len = live ? __ldg(a.ptr + row + 1) - kb : 0;
+        const double* xb = a.x + d.xoff;
+        const int warp_row = d.flags & TILE_LONG ? kTileWarpRow : INT32_MAX;
+        const bool mine = len <= warp_row;
+        const int cnt = mine ? len : 0;
+        const int wmax = __reduce_max_sync(0xffffffffu, cnt);
+        double sum[2] = {0.0, 0.0};
+        if (staged) {
+            const bool ok = mbar_wait_bounded(bar, parity, kWaitLimitNs);
+            if (__any_sync(0xffffffffu, !ok)) {
+                if (lane == 0) {   // let the copies still in flight land before the warp leaves
+                    atomicExch(a.err, kErrTimeout);
+                    mbar_wait_bounded(bar, parity, kDrainLimitNs);
                 }
-                if (tid == 0) store_row(a, d.r0, red[0]);
-            } else {
-                // LANES threads share a row: thread h takes entries
-                // kb + h, kb + h + LANES, ...; the FMA loop runs as many
-                // times as the warp's longest share, and the LANES partial
-                // sums meet in a fixed xor-butterfly
-                const int row = d.r0 + tid / LANES;
-                const int h = tid % LANES;
-                const unsigned char* st = smem + (size_t)s * L::BYTES;
-                const double* vs = reinterpret_cast<const double*>(st + L::VAL_OFF);
-                const int32_t* cs = reinterpret_cast<const int32_t*>(st + L::COL_OFF);
-                const int32_t* ps = reinterpret_cast<const int32_t*>(st + L::PTR_OFF);
-                const int va = d.k0 & ~1, ca = d.k0 & ~3, pa = d.r0 & ~3;
-                const int dc = va - ca;   // column slot of value slot 0
-                int kb = 0, cnt = 0;
-                if (row < d.r1) {
-                    kb = ps[row - pa] - va + h;
-                    const int ke = ps[row + 1 - pa] - va;
-                    cnt = ke > kb ? (ke - kb + LANES - 1) / LANES : 0;
-                }
-                const int wmax = __reduce_max_sync(0xffffffffu, cnt);
-                const double* xb = a.x + d.xoff;
-                double sum = 0.0;
-                for (int base = 0; base < wmax; base += CH) {
-                    // CH gathers in flight before their FMAs; slots past
-                    // the share read x[xoff] (a valid address) so every
-                    // load is unconditional, and their FMA results are
-                    // discarded; FMAs still run in storage order
-                    double xv[CH], vv[CH];
+                break;
+            }
+            parity ^= 1;
+        }
+        // gathers in flight before their FMAs; slots past the row read x[xoff]
+        // (a valid address), and their FMA results are discarded; FMAs run in
+        // storage order
+        if (staged) {
+            const double* vr = vs + (kb - va);
+            const int32_t* cr = cs + (kb - ca);
+            for (int base = 0; base < wmax; base += U) {
+                double xv[U];
 #pragma unroll
-                    for (int u = 0; u < CH; ++u) {
-                        const bool m = base + u < cnt;
-                        const int k = kb + LANES * (base + u);
-                        const int c = m ? cs[k + dc] : 0;
-                        vv[u] = m ? vs[k] : 0.0;
-                        xv[u] = ldg_keep(xb + c, pol_keep);
-                    }
+                for (int u = 0; u < U; ++u) xv[u] = ldg_keep(xb + (base + u < cnt ? cr[base + u] : 0), pol_keep);
 #pragma unroll
-                    for (int u = 0; u < CH; ++u) {
-                        if (base + u >= wmax) break;   // warp-uniform
-                        const double t = fma(vv[u], xv[u], sum);
-                        sum = (base + u < cnt) ? t : sum;
+                for (int u0 = 0; u0 < U; u0 += 3) {   // values three at a time, ahead of the dependent FMAs
+                    double vv[3];
+#pragma unroll
+                    for (int i = 0; i < 3; ++i) vv[i] = u0 + i < U && base + u0 + i < cnt ? vr[base + u0 + i] : 0.0;
+#pragma unroll
+                    for (int i = 0; i < 3 && u0 + i < U; ++i) {
+                        if (base + u0 + i >= wmax) break;   // warp-uniform
+                        double& acc = sum[(u0 + i) % S];
+                        const double p = fma(vv[i], xv[u0 + i], acc);
+                        acc = base + u0 + i < cnt ? p : acc;
                     }
                 }
+                if (S == 2 && U % 2 == 1) {   // the next round begins at an odd place
+                    const double even = sum[0];
+                    sum[0] = sum[1];
+                    sum[1] = even;
+                }
+            }
+        } else {
+#pragma unroll 1
+            for (int base = 0; base < wmax; base += 4) {
+                double xv[4], vv[4];
 #pragma unroll
-                for (int off = LANES / 2; off > 0; off >>= 1)
-                    sum += __shfl_xor_sync(0xffffffffu, sum, off, LANES);
-                if (row < d.r1 && h == 0) store_row(a, row, sum);
+                for (int u = 0; u < 4; ++u) {
+                    const bool m = base + u < cnt;
+                    vv[u] = m ? __ldg(a.val + kb + base + u) : 0.0;
+                    xv[u] = ldg_keep(xb + (m ? __ldg(a.col + kb + base + u) : 0), pol_keep);
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    double& acc = sum[u % S];
+                    const double p = fma(vv[u], xv[u], acc);
+                    acc = base + u < cnt ? p : acc;
+                }
             }
         }
-        __syncthreads();   // stage s is free again
-    }
-    if (aborted && tid == 0) {
-        atomicExch(a.err, kErrTimeout);
-        // let the copies still in flight land before the CTA leaves
-        for (int jj = j + 1; jj < j + ST; ++jj) {
-            if (first + jj * stride >= tile_end) break;
-            mbar_wait_bounded(smem_u32(&bars[jj % ST]), (uint32_t)((jj / ST) & 1), kDrainLimitNs);
+        if (live && mine) store_row(a, row, S == 2 ? sum[0] + sum[1] : sum[0]);
+        for (unsigned todo = __ballot_sync(0xffffffffu, !mine); todo; todo &= todo - 1) {
+            const int src = __ffs(todo) - 1;
+            const int k0 = __shfl_sync(0xffffffffu, kb, src), k1 = k0 + __shfl_sync(0xffffffffu, len, src);
+            double part = 0.0;
+#pragma unroll 1
+            for (int k = k0; k < k1; k += 32 * 4) {
+                double xv[4], vv[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const bool m = k + 32 * u + lane < k1;
+                    vv[u] = m ? __ldg(a.val + k + 32 * u + lane) : 0.0;
+                    xv[u] = m ? ldg_keep(xb + __ldg(a.col + k + 32 * u + lane), pol_keep) : 0.0;
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    if (k + 32 * u >= k1) break;   // warp-uniform
+                    const double p = fma(vv[u], xv[u], part);
+                    part = k + 32 * u + lane < k1 ? p : part;
+                }
+            }
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
+            if (lane == 0) store_row(a, d.r0 + src, part);
         }
+        __syncwarp();   // the stage is free again
     }
 }
 
-template <int NT, int CAP, int ST, int CH, int LANES>
-static cudaError_t run_tile(const CsrArgs& a, const Tile* tiles, int tb, int te, int num_sms,
+int tile_stage_cap(int entries) {
+    const int cap = (entries + 31) / 32 * 32;
+    return cap < 64 ? 64 : cap > kTileMaxEntries ? kTileMaxEntries : cap;
+}
+
+template <int U, int S>
+static cudaError_t run_tile(const CsrArgs& a, const Tile* tiles, int tb, int te, int cap, int num_sms,
                             cudaStream_t s) {
-    using L = TileLayout<NT / LANES, CAP>;
-    const size_t smem = (size_t)ST * L::BYTES;
+    const size_t smem = (size_t)kTileWarps * StageLayout(cap).bytes;
     static std::atomic<unsigned long long> configured{0};   // one bit per device ordinal
     int dev = 0;
-    cudaError_t e0 = cudaGetDevice(&dev);
-    if (e0 != cudaSuccess) return e0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
     if (dev >= 64 || !(configured.load(std::memory_order_acquire) >> dev & 1ull)) {
-        cudaError_t e = cudaFuncSetAttribute(csr_tile_kernel<NT, CAP, ST, CH, LANES>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = cudaFuncSetAttribute(csr_tile_kernel<U, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 kTileWarps * StageLayout(kTileMaxEntries).bytes);
         if (e != cudaSuccess) return e;
         if (dev < 64) configured.fetch_or(1ull << dev, std::memory_order_acq_rel);
     }
     int occ = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, csr_tile_kernel<NT, CAP, ST, CH, LANES>,
-                                                                  NT, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, csr_tile_kernel<U, S>, kTileWarps * 32, smem);
     if (e != cudaSuccess) return e;
     if (occ < 1) return cudaErrorInvalidConfiguration;
-    const int n_tiles = te - tb;
     int grid = num_sms * occ;
-    if (grid > n_tiles) grid = n_tiles;
-    return launch_pdl(csr_tile_kernel<NT, CAP, ST, CH, LANES>, dim3(grid), dim3(NT), smem, s, a, tiles, tb, te);
+    const int need = (te - tb + kTileWarps - 1) / kTileWarps;
+    if (grid > need) grid = need;
+    return launch_pdl(csr_tile_kernel<U, S>, dim3(grid), dim3(kTileWarps * 32), smem, s, a, tiles, tb, te, cap);
 }
 
-template <int NT, int CAP, int ST, int CH, int LANES>
-static int ctas_per_sm_of() {
-    using L = TileLayout<NT / LANES, CAP>;
-    const size_t smem = (size_t)ST * L::BYTES;
-    cudaFuncSetAttribute(csr_tile_kernel<NT, CAP, ST, CH, LANES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
-    int occ = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, csr_tile_kernel<NT, CAP, ST, CH, LANES>, NT, smem) !=
-        cudaSuccess)
-        return 0;
-    return occ;
-}
+bool tile_param_supported(int param) { return param >= 0 && param < 5; }
 
-// The geometries compiled into the library (threads, entries per stage,
-// stages).  The plan builds its tiles for one of them.
-// (threads, entries per stage, stages, gathers per chunk, threads per row)
-#define SPMV_TILE_GEOMS(X)      \
-    X(256, 3456, 2, 16, 2)      \
-    X(512, 6912, 2, 16, 2)      \
-    X(256, 3456, 3, 16, 2)      \
-    X(128, 3456, 2, 32, 1)      \
-    X(256, 2048, 3, 8, 2)
-
-TileGeom default_tile_geom() { return TileGeom{256, 3456, 2, 16, 2}; }
-
-#define GEOM_IS(nt, cap, st, ch, ln) \
-    (g.threads == nt && g.nnz_cap == cap && g.stages == st && g.chunk == ch && g.lanes == ln)
-
-bool tile_geom_supported(const TileGeom& g) {
-#define X(nt, cap, st, ch, ln) \
-    if (GEOM_IS(nt, cap, st, ch, ln)) return true;
-    SPMV_TILE_GEOMS(X)
-#undef X
-    return false;
-}
-
-int tile_ctas_per_sm(const TileGeom& g) {
-#define X(nt, cap, st, ch, ln) \
-    if (GEOM_IS(nt, cap, st, ch, ln)) return ctas_per_sm_of<nt, cap, st, ch, ln>();
-    SPMV_TILE_GEOMS(X)
-#undef X
-    return 0;
-}
-
-cudaError_t launch_tile(const CsrArgs& a, const Tile* tiles, int tile_begin, int tile_end,
-                        const TileGeom& g, int num_sms, cudaStream_t s) {
+// Geometries: gathers in flight per lane.  TILE keeps two sums a row (geometry
+// 3: one), WARP one.
+cudaError_t launch_tile(const CsrArgs& a, const Tile* tiles, int tile_begin, int tile_end, bool one_sum, int param,
+                        int cap, int num_sms, cudaStream_t s) {
     if (tile_end <= tile_begin) return cudaSuccess;
-#define X(nt, cap, st, ch, ln) \
-    if (GEOM_IS(nt, cap, st, ch, ln)) \
-        return run_tile<nt, cap, st, ch, ln>(a, tiles, tile_begin, tile_end, num_sms, s);
-    SPMV_TILE_GEOMS(X)
-#undef X
-    return cudaErrorInvalidValue;
+#define TILE_RUN(u, sums) return run_tile<u, sums>(a, tiles, tile_begin, tile_end, cap, num_sms, s)
+    switch (one_sum ? param + 5 : param) {
+        case 0: TILE_RUN(8, 2);
+        case 1: TILE_RUN(14, 2);
+        case 2: TILE_RUN(4, 2);
+        case 4: TILE_RUN(16, 2);
+        case 5: TILE_RUN(9, 1);
+        case 6: TILE_RUN(14, 1);
+        case 7: TILE_RUN(4, 1);
+        case 3:
+        case 8: TILE_RUN(7, 1);
+        case 9: TILE_RUN(16, 1);
+        default: return cudaErrorInvalidValue;
+    }
+#undef TILE_RUN
 }
 
 // ------------------------------------------------------------------------
@@ -492,179 +458,6 @@ __global__ void __launch_bounds__(256) csr_vector_kernel(CsrArgs a, const Tile* 
             for (int off = V / 2; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off, V);
             if (row < d.r1 && lane == 0) store_row(a, row, sum);
         }
-    }
-}
-
-// ------------------------------------------------------------------------
-// Warp-private pipelines: every warp owns an ST-stage ring of 32-row tiles
-// (values, columns, row pointers) in shared memory, filled by bulk copies its
-// lane 0 issues against the warp's own mbarriers.  There is no block-wide
-// barrier after set-up, so warps never wait for each other.  One thread per
-// row, exactly one DFMA per entry in storage order (the FMA loop runs the
-// warp's longest row), CH gathers of x in flight per chunk.  A row longer
-// than a stage (TILE_LONG) is summed by the 32 lanes from global memory with
-// a fixed butterfly.
-// ------------------------------------------------------------------------
-template <int WARPS, int CAP, int ST, int CH>
-__global__ void __launch_bounds__(WARPS * 32, 1) csr_warp_kernel(CsrArgs a, const Tile* __restrict__ tiles,
-                                                                int tile_begin, int tile_end) {
-    pdl_begin(a.pdl);  // the previous kernel of this stream is done (unless independent)
-    using L = TileLayout<32, CAP>;
-    extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ __align__(8) uint64_t bars[WARPS][ST];
-    const uint64_t pol_stream = policy_evict_first();
-    const uint64_t pol_keep = policy_evict_last();
-    const int lane = threadIdx.x & 31;
-    const int w = threadIdx.x >> 5;
-    unsigned char* ring = smem + (size_t)w * ST * L::BYTES;
-    const int first = tile_begin + (int)blockIdx.x * WARPS + w;
-    const int stride = (int)gridDim.x * WARPS;
-    if (lane == 0) {
-        for (int s = 0; s < ST; ++s) mbar_init(smem_u32(&bars[w][s]), 1);
-        mbar_fence_init();
-    }
-    __syncwarp();
-
-    auto issue = [&](int j) {   // lane 0 only
-        const int t = first + j * stride;
-        if (t >= tile_end) return;
-        const int s = j % ST;
-        const Tile d = tiles[t];
-        const uint32_t bar = smem_u32(&bars[w][s]);
-        if (d.flags & TILE_LONG) {
-            mbar_arrive_expect_tx(bar, 0);
-            return;
-        }
-        const int va = d.k0 & ~1, vb = (d.k1 + 1) & ~1;
-        const int ca = d.k0 & ~3, cb = (d.k1 + 3) & ~3;
-        const int pa = d.r0 & ~3, pb = (d.r1 + 4) & ~3;
-        const uint32_t vbytes = (uint32_t)(vb - va) * 8u;
-        const uint32_t cbytes = (uint32_t)(cb - ca) * 4u;
-        const uint32_t pbytes = (uint32_t)(pb - pa) * 4u;
-        unsigned char* st = ring + (size_t)s * L::BYTES;
-        mbar_arrive_expect_tx(bar, vbytes + cbytes + pbytes);
-        if (vbytes) bulk_g2s_hint(smem_u32(st + L::VAL_OFF), a.val + va, vbytes, bar, pol_stream);
-        if (cbytes) bulk_g2s_hint(smem_u32(st + L::COL_OFF), a.col + ca, cbytes, bar, pol_stream);
-        bulk_g2s_hint(smem_u32(st + L::PTR_OFF), a.ptr + pa, pbytes, bar, pol_stream);
-    };
-
-    if (lane == 0)
-        for (int j = 0; j < ST - 1; ++j) issue(j);
-    int j = 0;
-    bool aborted = false;
-    for (;; ++j) {
-        const int t = first + j * stride;
-        if (t >= tile_end) break;
-        if (lane == 0) {
-            fence_proxy_async_smem();   // stage (j-1) % ST was released by the warp
-            issue(j + ST - 1);
-        }
-        const int s = j % ST;
-        const bool ok = mbar_wait_bounded(smem_u32(&bars[w][s]), (uint32_t)((j / ST) & 1), kWaitLimitNs);
-        if (__any_sync(0xffffffffu, !ok)) {
-            aborted = true;
-            break;
-        }
-        const Tile d = tiles[t];
-        const double* xb = a.x + d.xoff;
-        if (d.flags & TILE_LONG) {
-            double part = 0.0;
-            for (int k = d.k0 + lane; k < d.k1; k += 32)
-                part = fma(__ldg(a.val + k), ldg_keep(xb + __ldg(a.col + k), pol_keep), part);
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
-            if (lane == 0) store_row(a, d.r0, part);
-        } else {
-            const unsigned char* st = ring + (size_t)s * L::BYTES;
-            const double* vs = reinterpret_cast<const double*>(st + L::VAL_OFF);
-            const int32_t* cs = reinterpret_cast<const int32_t*>(st + L::COL_OFF);
-            const int32_t* ps = reinterpret_cast<const int32_t*>(st + L::PTR_OFF);
-            const int va = d.k0 & ~1, ca = d.k0 & ~3, pa = d.r0 & ~3;
-            const int dc = va - ca;
-            const int row = d.r0 + lane;
-            int kb = 0, cnt = 0;
-            if (row < d.r1) {
-                kb = ps[row - pa] - va;
-                cnt = ps[row + 1 - pa] - va - kb;
-            }
-            const int wmax = __reduce_max_sync(0xffffffffu, cnt);
-            double sum = 0.0;
-            for (int base = 0; base < wmax; base += CH) {
-                double xv[CH], vv[CH];
-#pragma unroll
-                for (int u = 0; u < CH; ++u) {
-                    const bool m = base + u < cnt;
-                    const int k = kb + base + u;
-                    const int c = m ? cs[k + dc] : 0;
-                    vv[u] = m ? vs[k] : 0.0;
-                    xv[u] = ldg_keep(xb + c, pol_keep);
-                }
-#pragma unroll
-                for (int u = 0; u < CH; ++u) {
-                    if (base + u >= wmax) break;   // warp-uniform
-                    const double t0 = fma(vv[u], xv[u], sum);
-                    sum = (base + u < cnt) ? t0 : sum;
-                }
-            }
-            if (row < d.r1) store_row(a, row, sum);
-        }
-        __syncwarp();   // stage s is free again
-    }
-    if (aborted && lane == 0) {
-        atomicExch(a.err, kErrTimeout);
-        for (int jj = j + 1; jj < j + ST; ++jj) {
-            if (first + jj * stride >= tile_end) break;
-            mbar_wait_bounded(smem_u32(&bars[w][jj % ST]), (uint32_t)((jj / ST) & 1), kDrainLimitNs);
-        }
-    }
-}
-
-template <int WARPS, int CAP, int ST, int CH>
-static cudaError_t run_warp(const CsrArgs& a, const Tile* tiles, int tb, int te, int num_sms, cudaStream_t s) {
-    using L = TileLayout<32, CAP>;
-    const size_t smem = (size_t)WARPS * ST * L::BYTES;
-    static std::atomic<unsigned long long> configured{0};   // one bit per device ordinal
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev >= 64 || !(configured.load(std::memory_order_acquire) >> dev & 1ull)) {
-        e = cudaFuncSetAttribute(csr_warp_kernel<WARPS, CAP, ST, CH>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        if (dev < 64) configured.fetch_or(1ull << dev, std::memory_order_acq_rel);
-    }
-    int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, csr_warp_kernel<WARPS, CAP, ST, CH>, WARPS * 32, smem);
-    if (e != cudaSuccess) return e;
-    if (occ < 1) return cudaErrorInvalidConfiguration;
-    int grid = num_sms * occ;
-    const int need = (te - tb + WARPS - 1) / WARPS;
-    if (grid > need) grid = need;
-    return launch_pdl(csr_warp_kernel<WARPS, CAP, ST, CH>, dim3(grid), dim3(WARPS * 32), smem, s, a, tiles, tb, te);
-}
-
-// Warp-tile geometries: (warps per CTA, entries per stage, stages, gathers per chunk).
-int warp_tile_cap(int param) {
-    switch (param) {
-        case 0: return 896;    // 32 rows x 28 entries
-        case 1: return 896;
-        case 2: return 896;
-        case 3: return 1792;   // rows up to 56 entries
-        case 4: return 896;
-        default: return -1;
-    }
-}
-
-cudaError_t launch_warp(const CsrArgs& a, const Tile* tiles, int tb, int te, int param, int num_sms,
-                        cudaStream_t s) {
-    if (te <= tb) return cudaSuccess;
-    switch (param) {
-        case 0: return run_warp<8, 896, 2, 16>(a, tiles, tb, te, num_sms, s);    // 175 KB, 1 CTA
-        case 1: return run_warp<4, 896, 2, 16>(a, tiles, tb, te, num_sms, s);    // 88 KB, 2 CTAs
-        case 2: return run_warp<10, 896, 2, 16>(a, tiles, tb, te, num_sms, s);   // 219 KB, 1 CTA
-        case 3: return run_warp<4, 1792, 2, 16>(a, tiles, tb, te, num_sms, s);   // 174 KB, 1 CTA
-        case 4: return run_warp<10, 896, 2, 32>(a, tiles, tb, te, num_sms, s);   // 219 KB, 32 gathers in flight
-        default: return cudaErrorInvalidValue;
     }
 }
 

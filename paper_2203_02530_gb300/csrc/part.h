@@ -86,24 +86,17 @@ struct spmv_part {
     // after the rank's LOCAL product; the host path copies it out early)
     std::vector<std::pair<int64_t, int64_t>> io_free;
 
-    // tiles (thread-per-row and vector kernels)
-    spmvk::TileGeom geom{};
+    // 32-row tiles of the staged kernel and its stage size, LOCAL and REMOTE
     spmvk::Tile* ltiles = nullptr;
     spmvk::Tile* rtiles = nullptr;
+    int tile_cap[2] = {0, 0};
     std::vector<int64_t> ltile_off;   // P+1
     std::vector<int64_t> rtile_off;   // P+1
-    // fixed 256-row blocks (vector and pair kernels): independent of the
-    // tile geometry so their passes of 256 / lanes rows are always full
+    // fixed 256-row blocks (vector and pair kernels)
     spmvk::Tile* lblocks = nullptr;
     spmvk::Tile* rblocks = nullptr;
     std::vector<int64_t> lblock_off;  // P+1
     std::vector<int64_t> rblock_off;  // P+1
-    // 32-row tiles of the warp-pipeline kernel (built on first use)
-    spmvk::Tile* lwtiles = nullptr;
-    spmvk::Tile* rwtiles = nullptr;
-    std::vector<int64_t> lwtile_off;  // P+1
-    std::vector<int64_t> rwtile_off;  // P+1
-    int wtile_cap = 0;
     // merge-path tiles (built on first use of the merge variant)
     spmvk::MergeTile* lmtiles = nullptr;
     spmvk::MergeTile* rmtiles = nullptr;
@@ -183,9 +176,8 @@ namespace spmvk {
 void validate_csr(int64_t n, const int64_t* row_ptr, const int32_t* col_idx, const double* vals, int P);
 void build_plan(spmv_part* pt, int64_t n, const int64_t* row_ptr, const int32_t* col_idx,
                 const double* vals);
-void build_tiles(spmv_part* pt, const TileGeom& g);
+void build_tiles(spmv_part* pt);
 void build_merge_tiles(spmv_part* pt);
-void build_warp_tiles(spmv_part* pt, int cap);
 void build_sell(spmv_part* pt);
 bool build_sell_delta16(spmv_part* pt);
 void build_sell_split(spmv_part* pt, int part_idx, int param);

@@ -237,30 +237,34 @@ void build_plan(spmv_part* pt, int64_t n, const int64_t* rp, const int32_t* ci,
     pt->err = static_cast<int*>(dev_alloc(pt, sizeof(int)));
 }
 
-// Greedy row tiles of one CSR row range: consecutive rows while the tile
-// holds at most g.rows() rows and g.nnz_cap entries; a row longer than the
-// capacity gets a tile of its own marked TILE_LONG.
+// 32-row tiles of one CSR row range.
 static void tile_range(const std::vector<int32_t>& ptr, int64_t rb, int64_t re, int32_t xoff,
-                       const TileGeom& g, std::vector<Tile>& out) {
-    int64_t r = rb;
-    while (r < re) {
-        const int64_t len = (int64_t)ptr[(size_t)r + 1] - ptr[(size_t)r];
-        if (len > g.nnz_cap) {
-            out.push_back(Tile{(int32_t)r, (int32_t)(r + 1), ptr[(size_t)r], ptr[(size_t)r + 1], xoff,
-                               TILE_LONG, 0, 0});
-            ++r;
-            continue;
-        }
-        const int64_t start = r;
-        int64_t cnt = 0;
-        while (r < re && r - start < g.rows()) {
-            const int64_t l = (int64_t)ptr[(size_t)r + 1] - ptr[(size_t)r];
-            if (l > g.nnz_cap || cnt + l > g.nnz_cap) break;
-            cnt += l;
-            ++r;
-        }
-        out.push_back(Tile{(int32_t)start, (int32_t)r, ptr[(size_t)start], ptr[(size_t)r], xoff, 0, 0, 0});
+                       std::vector<Tile>& out) {
+    for (int64_t r = rb; r < re; r += kTileRows) {
+        const int64_t e = std::min<int64_t>(re, r + kTileRows);
+        int32_t flags = 0;
+        for (int64_t i = r; i < e; ++i)
+            if (ptr[(size_t)i + 1] - ptr[(size_t)i] > kSellLong) flags = TILE_LONG;
+        out.push_back(Tile{(int32_t)r, (int32_t)e, ptr[(size_t)r], ptr[(size_t)e], xoff, flags, 0, 0});
     }
+}
+
+// Stage size for a product's tiles: what 98 % of those without long rows need
+// (a few wide tiles then do not cost every warp its shared memory); the
+// others are marked TILE_WIDE.
+static int tile_stage(std::vector<Tile>& tiles) {
+    std::vector<int32_t> n;
+    for (const Tile& t : tiles)
+        if (!t.flags) n.push_back(t.k1 - t.k0);
+    int cap = tile_stage_cap(0);
+    if (!n.empty()) {
+        const size_t at = (n.size() - 1) - (n.size() - 1) / 50;
+        std::nth_element(n.begin(), n.begin() + (long)at, n.end());
+        cap = tile_stage_cap(n[at]);
+    }
+    for (Tile& t : tiles)
+        if (t.k1 - t.k0 > cap) t.flags |= TILE_WIDE;
+    return cap;
 }
 
 template <class T>
@@ -270,7 +274,7 @@ static std::vector<T> download(const T* d, size_t count) {
     return h;
 }
 
-void build_tiles(spmv_part* pt, const TileGeom& g) {
+void build_tiles(spmv_part* pt) {
     const int P = pt->P;
     const std::vector<int32_t> l_ptr = download(pt->l_ptr, (size_t)pt->n + 1);
     const std::vector<int32_t> rr_ptr = download(pt->rr_ptr, (size_t)pt->n_rr + 1);
@@ -279,18 +283,17 @@ void build_tiles(spmv_part* pt, const TileGeom& g) {
     pt->rtile_off.assign(P + 1, 0);
     for (int p = 0; p < P; ++p) {
         pt->ltile_off[p] = (int64_t)lt.size();
-        tile_range(l_ptr, pt->bounds[p], pt->bounds[p + 1], (int32_t)pt->bounds[p], g, lt);
+        tile_range(l_ptr, pt->bounds[p], pt->bounds[p + 1], (int32_t)pt->bounds[p], lt);
         pt->rtile_off[p] = (int64_t)rt.size();
-        tile_range(rr_ptr, pt->rr_off[p], pt->rr_off[p + 1], 0, g, rt);
+        tile_range(rr_ptr, pt->rr_off[p], pt->rr_off[p + 1], 0, rt);
     }
     pt->ltile_off[P] = (int64_t)lt.size();
     pt->rtile_off[P] = (int64_t)rt.size();
-    free_one(pt, pt->ltiles);
-    free_one(pt, pt->rtiles);
+    pt->tile_cap[0] = tile_stage(lt);
+    pt->tile_cap[1] = tile_stage(rt);
     pt->ltiles = upload(pt, lt);
     pt->rtiles = upload(pt, rt);
-    pt->geom = g;
-    if (!pt->lblocks) {
+    {
         std::vector<Tile> lb, rb;
         pt->lblock_off.assign(P + 1, 0);
         pt->rblock_off.assign(P + 1, 0);
@@ -352,30 +355,6 @@ void build_merge_tiles(spmv_part* pt) {
                    "merge partition");
     }
     check_cuda(cudaDeviceSynchronize(), "merge partition");
-}
-
-// Tiles of at most 32 rows and `cap` entries (one warp each).
-void build_warp_tiles(spmv_part* pt, int cap) {
-    const int P = pt->P;
-    const std::vector<int32_t> l_ptr = download(pt->l_ptr, (size_t)pt->n + 1);
-    const std::vector<int32_t> rr_ptr = download(pt->rr_ptr, (size_t)pt->n_rr + 1);
-    const TileGeom g{32, cap, 2, 16, 1};
-    std::vector<Tile> lt, rt;
-    pt->lwtile_off.assign(P + 1, 0);
-    pt->rwtile_off.assign(P + 1, 0);
-    for (int p = 0; p < P; ++p) {
-        pt->lwtile_off[p] = (int64_t)lt.size();
-        tile_range(l_ptr, pt->bounds[p], pt->bounds[p + 1], (int32_t)pt->bounds[p], g, lt);
-        pt->rwtile_off[p] = (int64_t)rt.size();
-        tile_range(rr_ptr, pt->rr_off[p], pt->rr_off[p + 1], 0, g, rt);
-    }
-    pt->lwtile_off[P] = (int64_t)lt.size();
-    pt->rwtile_off[P] = (int64_t)rt.size();
-    free_one(pt, pt->lwtiles);
-    free_one(pt, pt->rwtiles);
-    pt->lwtiles = upload(pt, lt);
-    pt->rwtiles = upload(pt, rt);
-    pt->wtile_cap = cap;
 }
 
 // Sliced layout of one CSR (row pointer `ptr` over rows [0, rows)), rank p
