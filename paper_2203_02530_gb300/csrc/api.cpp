@@ -175,8 +175,12 @@ int launch_product(spmv_part* pt, const spmvk::CsrArgs& a, bool remote, int p, c
         spmvk::SellArgs sa{sp.slices, sp.longs, sp.val,  sp.col,         sp.col16,     sp.len, sp.perm,
                            0,         0,        0,       0,       sp.long_part, sp.long_cnt, nullptr};
         sa.ypos = sp.ypos;
-        sa.slice_begin = (int)(p < 0 ? 0 : sp.slice_off[p]);
-        sa.slice_end = (int)(p < 0 ? sp.slice_off[pt->P] : sp.slice_off[p + 1]);
+        const bool grouped =
+            var == SPMV_VARIANT_SELL && spmvk::sell_grouped(pt, remote ? 1 : 0, p < 0 ? pt->P : p, param);
+        if (grouped) sa.groups = sp.groups;
+        const std::vector<int64_t>& so = grouped ? sp.group_off : sp.slice_off;
+        sa.slice_begin = (int)(p < 0 ? 0 : so[p]);
+        sa.slice_end = (int)(p < 0 ? so[pt->P] : so[p + 1]);
         sa.long_begin = (int)(p < 0 ? 0 : sp.long_off[p]);
         sa.long_end = (int)(p < 0 ? sp.long_off[pt->P] : sp.long_off[p + 1]);
         if (pt->dry_run) return (sa.slice_end > sa.slice_begin || sa.long_end > sa.long_begin) ? 1 : 0;
@@ -184,7 +188,7 @@ int launch_product(spmv_part* pt, const spmvk::CsrArgs& a, bool remote, int p, c
             const int units = (sa.slice_end - sa.slice_begin) + (sa.long_end - sa.long_begin);
             const int grid = spmvk::sell_grid(param, units, pt->num_sms);
             if (grid > 0) {
-                sa.cta_off = spmvk::sell_split(pt, remote ? 1 : 0, p < 0 ? pt->P : p, grid);
+                sa.cta_off = spmvk::sell_split(pt, remote ? 1 : 0, grouped, p < 0 ? pt->P : p, grid);
                 if (!sa.cta_off) fail(SPMV_EINVAL, "balanced sliced ranges not prepared");
             }
         }
@@ -782,8 +786,8 @@ static void prepare_variant(spmv_part* pt, int variant, int param, int op_kind) 
         if (variant == SPMV_VARIANT_SELL16 && !spmvk::build_sell_delta16(pt))
             fail(SPMV_EINVAL, "a LOCAL column lies more than 32767 rows from its row: no 16-bit deltas");
         if (spmvk::sell_param_balanced(param)) {
-            if (op_kind != SPMV_OP_REMOTE) spmvk::build_sell_split(pt, 0, param);
-            if (op_kind != SPMV_OP_LOCAL) spmvk::build_sell_split(pt, 1, param);
+            if (op_kind != SPMV_OP_REMOTE) spmvk::build_sell_split(pt, 0, param, variant == SPMV_VARIANT_SELL16);
+            if (op_kind != SPMV_OP_LOCAL) spmvk::build_sell_split(pt, 1, param, false);
         }
     } else {
         fail(SPMV_EINVAL, "unknown variant %d", variant);

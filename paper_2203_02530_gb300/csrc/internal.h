@@ -43,9 +43,17 @@ struct Carry {
 // at off + 32 j + r.
 struct SellSlice {
     int32_t p0, rows, len, xoff;
-    int32_t off, pad0, pad1, pad2;
+    int32_t off, group, pad1, pad2;   // group: slices in the group this descriptor starts (1: the slice alone)
 };
 static_assert(sizeof(SellSlice) == 32, "slice descriptor is two int4");
+
+// A group of a sorted layout: kSellGroup[len] slices that follow each other,
+// every row of them len entries long, taken by a warp at once (a SellSlice for
+// the first with group > 1; the others' slots and positions follow it).  At
+// most 8 slots a lane, so that a group fits the registers of the sliced kernels
+// with 8 or 9 entries per lane and step; those with 4 take slices.
+constexpr int kSellGroupLen = 5;
+constexpr int kSellGroup[kSellGroupLen] = {4, 4, 4, 2, 2};
 
 // A piece of a row longer than kSellLong entries: entries [k0, k1) of the
 // CSR row, summed by a whole warp.  A row longer than kSellChunk entries is
@@ -77,6 +85,8 @@ struct SellArgs {
                              // CTA b takes units [cta_off[b], cta_off[b + 1])
     const int32_t* ypos;     // per position: its y row (row order and row map
                              // composed; sorted remote layouts), or nullptr
+    const SellSlice* groups; // the launch takes groups [slice_begin, slice_end)
+                             // of a sorted layout, or nullptr: slices
 };
 
 // Operands of one CSR product launch.
@@ -135,6 +145,7 @@ cudaError_t launch_sell(const CsrArgs& a, const SellArgs& s, int param, bool del
 cudaError_t launch_sell_delta(const SellSlice* slices, int n_slices, const uint8_t* len, const int32_t* perm,
                               const int32_t* scol, int16_t* scol16, int* bad, int num_sms, cudaStream_t s);
 bool sell_param_supported(int param);
+bool sell_param_grouped(int param);   // launches take groups where the layout has them
 cudaError_t launch_segment_copy(const int32_t* tab, int n_seg, const double* sv, const int32_t* sc, double* dv,
                                 int32_t* dc, int num_sms, cudaStream_t s);
 cudaError_t launch_sell_unfill(const int32_t* ptr, const SellSlice* slices, int n_slices, const uint8_t* len,

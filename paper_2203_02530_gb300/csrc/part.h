@@ -118,10 +118,13 @@ struct spmv_part {
         int16_t* col16 = nullptr;         // column - row deltas (LOCAL only), once built
         double* long_part = nullptr;      // partial sums of cut long rows
         int* long_cnt = nullptr;          // pieces done per cut long row
+        spmvk::SellSlice* groups = nullptr;   // sorted layouts: the slices in groups (kSellGroup)
+        std::vector<int64_t> group_off;   // P+1
         std::vector<int32_t> h_slice_len; // per slice: its longest row's entries
+        std::vector<int32_t> h_group_len; // per group: its slots per lane
         std::vector<int32_t> h_long_len;  // per long-row piece: its entries
         // balanced CTA ranges per launch site (rank p, or P for all ranks)
-        // and grid: key site << 32 | grid
+        // and grid: key grouped << 62 | site << 32 | grid
         std::map<int64_t, int32_t*> cta_split;
         int delta_state = 0;              // 0 not checked, 1 built, -1 some delta needs > 16 bits
         // with the CSR released: the long rows' entries, piece after piece
@@ -180,10 +183,13 @@ void build_tiles(spmv_part* pt);
 void build_merge_tiles(spmv_part* pt);
 void build_sell(spmv_part* pt);
 bool build_sell_delta16(spmv_part* pt);
-void build_sell_split(spmv_part* pt, int part_idx, int param);
+void build_sell_split(spmv_part* pt, int part_idx, int param, bool delta16);
 void release_csr(spmv_part* pt);
 void restore_csr(spmv_part* pt);
-const int32_t* sell_split(const spmv_part* pt, int part_idx, int site, int grid);
+// Whether a launch of part_idx's 32-bit sliced product at `site` (rank, or P for
+// all ranks) takes the layout's groups.
+bool sell_grouped(const spmv_part* pt, int part_idx, int site, int param);
+const int32_t* sell_split(const spmv_part* pt, int part_idx, bool grouped, int site, int grid);
 void* dev_alloc(spmv_part* pt, size_t bytes);
 void free_plan(spmv_part* pt);
 }  // namespace spmvk

@@ -433,12 +433,41 @@ static int64_t build_sell_part(spmv_part* pt, spmv_part::SellPart& sp, const std
             for (int64_t i = q; i < e; ++i)
                 if (len[(size_t)i] != kSellLenLong) mx = std::max<int32_t>(mx, len[(size_t)i]);
             if (off + 32 * (int64_t)mx > INT32_MAX - 64) fail(SPMV_EBOUNDS, "sliced layout exceeds 2^31 entries");
-            slices.push_back(SellSlice{(int32_t)q, (int32_t)(e - q), mx, xo[p], (int32_t)off, 0, 0, 0});
+            slices.push_back(SellSlice{(int32_t)q, (int32_t)(e - q), mx, xo[p], (int32_t)off, 1, 0, 0});
             off += 32 * (int64_t)mx;
         }
     }
     sp.slice_off[P] = (int64_t)slices.size();
     sp.long_off[P] = (int64_t)longs.size();
+    if (any_sorted) {
+        // groups of full slices: 32 rows, all as long as the slice
+        auto full = [&](const SellSlice& sl) {
+            if (sl.rows != 32) return false;
+            for (int i = 0; i < 32; ++i)
+                if (len[(size_t)sl.p0 + i] != sl.len) return false;
+            return true;
+        };
+        std::vector<SellSlice> groups;
+        sp.group_off.assign(P + 1, 0);
+        for (int p = 0; p < P; ++p) {
+            sp.group_off[p] = (int64_t)groups.size();
+            for (int64_t i = sp.slice_off[p]; i < sp.slice_off[p + 1];) {
+                const int32_t L = slices[(size_t)i].len;
+                const int want = L < kSellGroupLen ? kSellGroup[L] : 1;
+                int got = 0;
+                while (got < want && i + got < sp.slice_off[p + 1] && slices[(size_t)(i + got)].len == L &&
+                       full(slices[(size_t)(i + got)]))
+                    ++got;
+                groups.push_back(slices[(size_t)i]);
+                groups.back().group = got == want ? want : 1;
+                i += got == want ? want : 1;
+            }
+        }
+        sp.group_off[P] = (int64_t)groups.size();
+        sp.h_group_len.resize(groups.size());
+        for (size_t i = 0; i < groups.size(); ++i) sp.h_group_len[i] = groups[i].len * groups[i].group;
+        sp.groups = upload(pt, groups);
+    }
     sp.h_slice_len.resize(slices.size());
     for (size_t i = 0; i < slices.size(); ++i) sp.h_slice_len[i] = slices[i].len;
     sp.h_long_len.resize(longs.size());
@@ -490,7 +519,7 @@ void build_sell(spmv_part* pt) {
 // (and so each SM, which holds several) gets the same work and keeps the
 // neighbouring slices of the round-robin split together.  A unit's cost is
 // its entries per lane (a slice's longest row; a piece's entries over 32,
-// rounded up) plus 3 for its descriptor, row and store.
+// rounded up; a group's slots per lane) plus 3 for its descriptor, row and store.
 // Estimated time of one work unit of a sliced launch: a fixed part (the
 // unit's descriptor, lengths and row-map loads and its stores) plus one per
 // entry of a lane (slots of a slice lane; a long-row piece's entries over
@@ -502,21 +531,39 @@ double sell_unit_cost(bool long_piece, int64_t len) {
     return 3.0 + (double)per_lane;
 }
 
-void build_sell_split(spmv_part* pt, int part_idx, int param) {
+// A launch over all ranks takes groups, one over a rank from 10 slices per SM
+// on: below, its warps outnumber its units, and a group only lengthens a warp's
+// chain (power-law, 8 ranks, 4 streams: 390 slices per launch 38.7 us with
+// slices, 39.8 us with groups; 2300: 78.2 and 75.1 us; 4700: 141.5 and 131.4 us;
+// 7800: 228 and 215 us; over all ranks 3100 slices 18.0 and 15.5 us).
+bool sell_grouped(const spmv_part* pt, int part_idx, int site, int param) {
+    const spmv_part::SellPart& sp = pt->sell[part_idx];
+    if (!sp.groups || !sell_param_grouped(param)) return false;
+    return site == pt->P || sp.slice_off[site + 1] - sp.slice_off[site] >= (int64_t)pt->num_sms * 10;
+}
+
+static int64_t sell_split_key(bool grouped, int site, int grid) {
+    return ((int64_t)(grouped ? 1 : 0) << 62) | ((int64_t)site << 32) | grid;
+}
+
+void build_sell_split(spmv_part* pt, int part_idx, int param, bool delta16) {
     spmv_part::SellPart& sp = pt->sell[part_idx];
     const int P = pt->P;
     for (int site = 0; site <= P; ++site) {
         const int64_t lb = site < P ? sp.long_off[site] : 0, le = site < P ? sp.long_off[site + 1] : sp.long_off[P];
-        const int64_t sb = site < P ? sp.slice_off[site] : 0, se = site < P ? sp.slice_off[site + 1] : sp.slice_off[P];
+        const bool grouped = !delta16 && sell_grouped(pt, part_idx, site, param);
+        const std::vector<int64_t>& so = grouped ? sp.group_off : sp.slice_off;
+        const std::vector<int32_t>& sl = grouped ? sp.h_group_len : sp.h_slice_len;
+        const int64_t sb = site < P ? so[site] : 0, se = site < P ? so[site + 1] : so[P];
         const int units = (int)((le - lb) + (se - sb));
         const int grid = sell_grid(param, units, pt->num_sms);
         if (grid <= 0) continue;
-        const int64_t key = ((int64_t)site << 32) | grid;
+        const int64_t key = sell_split_key(grouped, site, grid);
         if (sp.cta_split.count(key)) continue;
         std::vector<double> prefix((size_t)units + 1, 0.0);
         for (int u = 0; u < units; ++u) {
             const bool lng = u < le - lb;
-            const int64_t len = lng ? sp.h_long_len[(size_t)(lb + u)] : sp.h_slice_len[(size_t)(sb + u - (le - lb))];
+            const int64_t len = lng ? sp.h_long_len[(size_t)(lb + u)] : sl[(size_t)(sb + u - (le - lb))];
             prefix[(size_t)u + 1] = prefix[(size_t)u] + sell_unit_cost(lng, len);
         }
         std::vector<int32_t> off((size_t)grid + 1);
@@ -532,9 +579,9 @@ void build_sell_split(spmv_part* pt, int part_idx, int param) {
     }
 }
 
-const int32_t* sell_split(const spmv_part* pt, int part_idx, int site, int grid) {
+const int32_t* sell_split(const spmv_part* pt, int part_idx, bool grouped, int site, int grid) {
     const spmv_part::SellPart& sp = pt->sell[part_idx];
-    auto it = sp.cta_split.find(((int64_t)site << 32) | grid);
+    auto it = sp.cta_split.find(sell_split_key(grouped, site, grid));
     return it == sp.cta_split.end() ? nullptr : it->second;
 }
 

@@ -111,6 +111,57 @@ __device__ __forceinline__ void sell_tail(int r, const CT* cp, const double* vp,
     }
 }
 
+// A group of C slices that follow each other in a sorted layout, every row of
+// them L entries long: slot j of the group's slice i is slot i L + j of one
+// run, so the warp has the loads of all its rows, then all its gathers, in
+// flight at once.  The short rows that make up most of a skewed matrix
+// otherwise cost a chain of dependent loads (descriptor, columns, gather, row
+// number, store) for 1 to 4 gathers a lane.  Power-law 2 M rows, 8 ranks: 215
+// against 228 us per step in per-rank launches, 197 against 214 us with one
+// launch over all ranks; the x gathers (37 M, 130 us) bound both.
+template <int C, int L, bool YP>
+__device__ __forceinline__ void sell_group(const CsrArgs& a, const SellArgs& sa, const SellSlice& d, int lane,
+                                           uint64_t pol_stream, uint64_t pol_keep, bool& pending) {
+    const int pos = d.p0 + lane;
+    int row[C];
+#pragma unroll
+    for (int i = 0; i < C; ++i) row[i] = __ldg((YP ? sa.ypos : sa.perm) + pos + 32 * i);
+    double sum[C];
+#pragma unroll
+    for (int i = 0; i < C; ++i) sum[i] = 0.0;
+    if (L > 0) {
+        const double* vp = sa.val + (int64_t)d.off + lane;
+        const int32_t* cp = sa.col + (int64_t)d.off + lane;
+        const double* xb = a.x + d.xoff;
+        int32_t c[C * L + 1];
+        double v[C * L + 1], xv[C * L + 1];
+#pragma unroll
+        for (int q = 0; q < C * L; ++q) {
+            c[q] = ld_stream(cp + 32 * q, pol_stream);
+            v[q] = ld_stream(vp + 32 * q, pol_stream);
+        }
+#pragma unroll
+        for (int q = 0; q < C * L; ++q) xv[q] = ld_keep(xb + c[q], pol_keep);
+#pragma unroll
+        for (int q = 0; q < C * L; ++q) sum[q / (L > 0 ? L : 1)] = fma(v[q], xv[q], sum[q / (L > 0 ? L : 1)]);
+    }
+    pdl_settle(pending);
+    if (!YP && a.rowmap) {
+#pragma unroll
+        for (int i = 0; i < C; ++i) row[i] = __ldg(a.rowmap + row[i]);
+    }
+    if (a.accumulate) {
+        double y[C];
+#pragma unroll
+        for (int i = 0; i < C; ++i) y[i] = a.y[row[i]];
+#pragma unroll
+        for (int i = 0; i < C; ++i) a.y[row[i]] = y[i] + sum[i];
+    } else {
+#pragma unroll
+        for (int i = 0; i < C; ++i) a.y[row[i]] = sum[i];
+    }
+}
+
 // Entries [k, ke) of a long row taken by one lane in steps of 32 (k = the
 // lane's first), R at a time: R value and R column loads, then R gathers,
 // then R FMAs in entry order; in the last round the entries at or past ke
@@ -149,7 +200,9 @@ __device__ __forceinline__ void long_round(const CsrArgs& a, const double* xb, i
 // CT = int16_t: slot columns are deltas to the row (x index = row + delta),
 // half the index bytes where every |column - row| fits in 16 bits.
 // YP: the layout has a y row per position (sa.ypos; sorted remote layouts).
-template <int U, int MINB, typename CT, bool YP = false>
+// GRP: the units after the long rows are the sorted layout's groups
+// (sell_group) instead of its slices; a group of one slice is that slice.
+template <int U, int MINB, typename CT, bool YP = false, bool GRP = false>
 __global__ void __launch_bounds__(256, MINB) csr_sell_kernel(CsrArgs a, SellArgs sa) {
     // the previous kernel of this stream is done (unless independent, or
     // the wait is deferred to the first access to y)
@@ -226,7 +279,17 @@ __global__ void __launch_bounds__(256, MINB) csr_sell_kernel(CsrArgs a, SellArgs
             }
             continue;
         }
-        const SellSlice d = sa.slices[sa.slice_begin + u0 - n_long];
+        const SellSlice d = (GRP ? sa.groups : sa.slices)[sa.slice_begin + u0 - n_long];
+        if (GRP && d.group > 1) {
+            switch (d.len) {
+                case 0: sell_group<kSellGroup[0], 0, YP>(a, sa, d, lane, pol_stream, pol_keep, pending); break;
+                case 1: sell_group<kSellGroup[1], 1, YP>(a, sa, d, lane, pol_stream, pol_keep, pending); break;
+                case 2: sell_group<kSellGroup[2], 2, YP>(a, sa, d, lane, pol_stream, pol_keep, pending); break;
+                case 3: sell_group<kSellGroup[3], 3, YP>(a, sa, d, lane, pol_stream, pol_keep, pending); break;
+                default: sell_group<kSellGroup[4], 4, YP>(a, sa, d, lane, pol_stream, pol_keep, pending); break;
+            }
+            continue;
+        }
         const int pos = d.p0 + lane;
         int len = 0;
         bool store = false;
@@ -439,6 +502,8 @@ cudaError_t launch_sell_col32(const SellSlice* slices, int n_slices, const uint8
     return cudaGetLastError();
 }
 
+bool sell_param_grouped(int param) { return param % 1000 != 4 && param % 1000 != 104; }
+
 bool sell_param_supported(int param) {
     const int base = param >= 2000 ? param - 2000 : param;
     return base == 4 || base == 8 || base == 9 || (base >= 104 && base <= 107);
@@ -470,7 +535,11 @@ cudaError_t launch_sell(const CsrArgs& a, const SellArgs& sa, int param, bool de
     if (grid <= 0) return cudaErrorInvalidValue;
     if (sell_param_balanced(param) != (sa.cta_off != nullptr)) return cudaErrorInvalidValue;
 #define SELL_LAUNCH(u, b)                                                                        \
-    e = delta16 ? launch_pdl(csr_sell_kernel<u, b, int16_t>, dim3(grid), dim3(256), 0, st, a, sa)      \
+    e = sa.groups && sa.ypos                                                                             \
+            ? launch_pdl(csr_sell_kernel<u, b, int32_t, true, (u >= 8)>, dim3(grid), dim3(256), 0, st, a, sa) \
+        : sa.groups                                                                                            \
+            ? launch_pdl(csr_sell_kernel<u, b, int32_t, false, (u >= 8)>, dim3(grid), dim3(256), 0, st, a, sa) \
+        : delta16 ? launch_pdl(csr_sell_kernel<u, b, int16_t>, dim3(grid), dim3(256), 0, st, a, sa)      \
         : sa.ypos ? launch_pdl(csr_sell_kernel<u, b, int32_t, true>, dim3(grid), dim3(256), 0, st, a, sa) \
                   : launch_pdl(csr_sell_kernel<u, b, int32_t>, dim3(grid), dim3(256), 0, st, a, sa)
     cudaError_t e = cudaSuccess;
