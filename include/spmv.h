@@ -532,8 +532,9 @@ int spmv_batch_run_separate(spmv_batch* batch, int m, const double* x_dev, doubl
  * around its SpMV.
  * spmv_serve_create: n_streams (1..64) stream slots, one block in flight per
  *   slot; budget_bytes covers the resident matrices plus a pool from which
- *   every in-flight block of total width w takes 16 n w bytes (X and Y,
- *   n x w doubles each, row-major); SPMV_ENOMEM when the budget is below the
+ *   every in-flight block of total width w takes 8 n (w + w') bytes (X,
+ *   n x w' doubles, and Y, n x w, row-major; w' = w, in the sliced layout
+ *   rounded up to 4 or 8 above 2); SPMV_ENOMEM when the budget is below the
  *   resident matrices, SPMV_EBOUNDS for a matrix with n >= 2^28.
  * spmv_serve_run: runs n_req requests open loop against their arrival times
  *   (seconds from the call, non-decreasing), on the host thread, until all
@@ -545,7 +546,7 @@ int spmv_batch_run_separate(spmv_batch* batch, int m, const double* x_dev, doubl
  *   sliced layout, BATCHED goes further: a free slot takes ceil(blocks /
  *   slots) of the blocks the queues would form (at most the group size,
  *   spmv_serve_set_group_max) and runs more than one, across matrices, as one
- *   group with one launch per kernel kind (X generation, slices, long rows);
+ *   group with one launch that draws X and one that multiplies;
  *   while no more blocks wait than there are slots every block thus gets a
  *   slot of its own, and groups grow only with a longer queue.
  *   PLAIN launches every request alone (one block per request).  Outputs:

@@ -748,26 +748,33 @@ void upload_items(spmv_batch* b) {
     // spread the gathers over all of them); within a matrix its heaviest
     // units (the long rows) first, so they do not end up in the tail
     std::vector<Unit> units[2];   // sliced layout, CSR modes
+    units[0].reserve((size_t)(n_slices / slices_per) + all.size());
+    units[1].reserve((size_t)(csr_rows / rows_per) + all.size());
+    struct Run {   // an item (or a matrix's pieces): units of `per`, each of about `cost`
+        int kind, a, b, per;
+        int64_t cost;
+    };
+    std::vector<Run> runs;
     b->unit_off.assign(2 * (b->count + 1), 0);
     for (int m = 0, piece = 0; m < b->count; ++m) {
         const int part = b->mats[m].lanes == kSliced ? 0 : 1;
         std::vector<Unit>& u = units[part];
         b->unit_off[m] = (int)units[0].size();
         b->unit_off[b->count + 1 + m] = (int)units[1].size();
-        const size_t first = u.size();
-        for (size_t j = 0; j < b->pieces[m].size(); ++j, ++piece)
-            u.push_back(Unit{{m, 3, piece, piece + 1}, long_cost(b->piece_len, 1)});
+        runs.clear();
+        const int pieces = (int)b->pieces[m].size();
+        if (pieces > 0) runs.push_back(Run{3, piece, piece + pieces, 1, long_cost(b->piece_len, 1)});
+        piece += pieces;
         const auto& items = part == 0 ? b->sliced_items[m] : b->csr_items[m];
         const auto& cost = part == 0 ? b->sliced_cost[m] : b->csr_cost[m];
         for (size_t i = 0; i < items.size(); ++i) {
-            const BatchItem w = items[i];
-            const int per = w.kind == 0 ? rows_per : w.kind == 1 ? longs_per : slices_per;
-            for (int a = w.a; a < w.b; a += per) {
-                const int e = std::min(w.b, a + per);
-                u.push_back(Unit{{m, w.kind, a, e}, cost[i] * (e - a) / (w.b - w.a)});
-            }
+            const BatchItem& w = items[i];
+            const int per = std::min(w.b - w.a, w.kind == 0 ? rows_per : w.kind == 1 ? longs_per : slices_per);
+            runs.push_back(Run{w.kind, w.a, w.b, per, cost[i] * per / (w.b - w.a)});
         }
-        std::stable_sort(u.begin() + (long)first, u.end(), [](const Unit& p, const Unit& q) { return p.cost > q.cost; });
+        std::stable_sort(runs.begin(), runs.end(), [](const Run& p, const Run& q) { return p.cost > q.cost; });
+        for (const Run& r : runs)
+            for (int a = r.a; a < r.b; a += r.per) u.push_back(Unit{{m, r.kind, a, std::min(r.b, a + r.per)}, r.cost});
     }
     b->unit_off[b->count] = b->n_sliced_units = (int)units[0].size();
     b->unit_off[2 * b->count + 1] = (int)units[1].size();

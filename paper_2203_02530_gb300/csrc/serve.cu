@@ -16,6 +16,7 @@
 // alone and in any mix (checked through an order-independent 64-bit hash of
 // its bits).
 #include "batch.h"
+#include "pdl.cuh"
 
 #include <cuda_runtime.h>
 
@@ -28,6 +29,7 @@
 
 using spmvk::BatchMat;
 using spmvk::BSlice;
+using spmvk::launch_pdl;
 
 namespace {
 
@@ -81,18 +83,32 @@ struct BlockReq {
     int pad;
 };
 
+// A block's column: its request's width, its place among the request's columns
+// and the request's index (hash slot).
+struct BlockCol {
+    int width, off, index, pad;
+};
+
 struct BlockDesc {
     BlockReq req[kMaxW];
+    BlockCol col[kMaxW];
     int n_req;
     int width;
 };
 
-// X[i, c] for every column of every request of a block (row-major, ld W):
+// The column table of a block's requests.
+void set_columns(const BlockReq* req, int n_req, BlockCol* col) {
+    for (int r = 0; r < n_req; ++r)
+        for (int j = 0; j < req[r].width; ++j) col[req[r].col0 + j] = BlockCol{req[r].width, j, req[r].index, 0};
+}
+
+// X[i, c] for every column of every request of a block (row-major, leading
+// dimension ld):
 // request r's element (i, j) is U(seed_r, 8 i + j), columns of no request 0.
 // Thread `tid` of `nthreads` (nthreads >= W) owns column tid mod W and rows
 // tid / W, tid / W + R, ... with R = nthreads / W, so consecutive threads
 // write consecutive elements and the counter advances by a constant.
-__device__ __forceinline__ void gen_x(double* __restrict__ X, int n, int W, const BlockReq* req, int n_req,
+__device__ __forceinline__ void gen_x(double* __restrict__ X, int n, int W, int ld, const BlockReq* req, int n_req,
                                       int tid, int nthreads) {
     const int R = nthreads / W;
     if (tid >= R * W) return;
@@ -105,18 +121,18 @@ __device__ __forceinline__ void gen_x(double* __restrict__ X, int n, int W, cons
         if (c >= q.col0 && c < q.col0 + q.width) { seed = q.seed; j = c - q.col0; }
     }
     if (j < 0) {
-        for (; i < n; i += R) X[(int64_t)i * W + c] = 0.0;
+        for (; i < n; i += R) X[(int64_t)i * ld + c] = 0.0;
         return;
     }
     uint64_t z = seed + ((uint64_t)i * kMaxW + (uint64_t)j + 1) * kGolden;
     const uint64_t dz = (uint64_t)R * kMaxW * kGolden;
 #pragma unroll 4
     for (; i < n; i += R, z += dz)
-        X[(int64_t)i * W + c] = __longlong_as_double((long long)pm1_bits_from_u53(splitmix_out(z) >> 11));
+        X[(int64_t)i * ld + c] = __longlong_as_double((long long)pm1_bits_from_u53(splitmix_out(z) >> 11));
 }
 
-__global__ void gen_x_kernel(double* __restrict__ X, int n, BlockDesc b) {
-    gen_x(X, n, b.width, b.req, b.n_req, (int)(blockIdx.x * blockDim.x + threadIdx.x), (int)(gridDim.x * blockDim.x));
+__global__ void gen_x_kernel(double* __restrict__ X, int n, int ld, BlockDesc b) {
+    gen_x(X, n, b.width, ld, b.req, b.n_req, (int)(blockIdx.x * blockDim.x + threadIdx.x), (int)(gridDim.x * blockDim.x));
 }
 
 __device__ __forceinline__ uint64_t mix64(uint64_t z) {
@@ -125,11 +141,38 @@ __device__ __forceinline__ uint64_t mix64(uint64_t z) {
     return z ^ (z >> 33);
 }
 
-// A row of X (W values, leading dimension W): two per 16-byte load when W
-// is even (every row then starts 16-byte aligned), else one at a time.
-template <int W>
+// Columns of X in a block of the pool: the block's width, rounded up to 4 or 8
+// above 2, so that every row starts at a multiple of its size.
+__host__ __device__ constexpr int pow2_columns(int w) { return w > 4 ? 8 : w > 2 ? 4 : w; }
+
+// A row of X (W values).  PAD (leading dimension pow2_columns(W), X at a multiple
+// of 32 bytes): four per 32-byte load, the rest in one; else (leading dimension
+// W) two per 16-byte load when W is even, or one at a time.  Every load of a
+// warp costs the L1 a look-up per lane (the rows lie far apart): 8 columns in
+// four loads cost 128 cycles per entry of a slice, as many as its 8 warp FMAs
+// on the FP64 pipe, 7 columns in seven loads 224; in two loads they cost 64.
+template <int W, bool PAD>
 __device__ __forceinline__ void load_row(const double* xr, double (&xv)[W]) {
-    if (W % 2 == 0) {
+    if (PAD && W > 2) {
+#pragma unroll
+        for (int c = 0; c < W; c += 4) {
+            if (W - c >= 3) {
+                double t[4];
+                asm("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];"
+                    : "=d"(t[0]), "=d"(t[1]), "=d"(t[2]), "=d"(t[3])
+                    : "l"(xr + c));
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (c + i < W) xv[c + i < W ? c + i : 0] = t[i];
+            } else if (W - c == 2) {
+                const double2 t = __ldg(reinterpret_cast<const double2*>(xr + c));
+                xv[c] = t.x;
+                xv[c + 1 < W ? c + 1 : 0] = t.y;
+            } else {
+                xv[c] = __ldg(xr + c);
+            }
+        }
+    } else if (W % 2 == 0) {
 #pragma unroll
         for (int c = 0; c < W; c += 2) {
             const double2 t = __ldg(reinterpret_cast<const double2*>(xr + c));
@@ -142,34 +185,47 @@ __device__ __forceinline__ void load_row(const double* xr, double (&xv)[W]) {
     }
 }
 
-// Hash of row `row`'s W values into the per-request sums h (definition below).
-template <int W>
-__device__ __forceinline__ void hash_row(const BlockReq* req, int n_req, int row, const double (&acc)[W],
-                                         unsigned long long (&h)[kMaxW]) {
-#pragma unroll
-    for (int r = 0; r < kMaxW; ++r) {
-        if (r >= n_req) break;
-        const BlockReq q = req[r];
-#pragma unroll
-        for (int c = 0; c < W; ++c) {
-            if (c >= q.col0 && c < q.col0 + q.width) {
-                const uint64_t e = (uint64_t)row * q.width + (uint64_t)(c - q.col0);
-                h[r] += mix64((uint64_t)__double_as_longlong(acc[c]) + e * kGolden);
-            }
-        }
-    }
+// Hash term of element (row, column c) of Y (definition below).
+__device__ __forceinline__ unsigned long long hash_term(const BlockCol& q, int row, double y) {
+    const uint64_t e = (uint64_t)row * q.width + (uint64_t)q.off;
+    return mix64((uint64_t)__double_as_longlong(y) + e * kGolden);
 }
 
-__device__ __forceinline__ void flush_hash(const BlockReq* req, int n_req, unsigned long long (&h)[kMaxW],
-                                           unsigned long long* hashes) {
+// Terms of row `row`'s W values into the per-column sums h.
+template <int W>
+__device__ __forceinline__ void hash_row(const BlockCol* col, int row, const double (&acc)[W],
+                                         unsigned long long (&h)[kMaxW]) {
 #pragma unroll
-    for (int r = 0; r < kMaxW; ++r) {
-        if (r >= n_req) break;
-        unsigned long long v = h[r];
-        h[r] = 0;
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-        if ((threadIdx.x & 31) == 0 && v) atomicAdd(hashes + req[r].index, v);
+    for (int c = 0; c < W; ++c) h[c] += hash_term(col[c], row, acc[c]);
+}
+
+// Adds column sums (lane c < width: column c's) to their requests' hashes: the
+// columns of a request, which lie side by side, are added first, so that a
+// request gets one atomic.
+__device__ __forceinline__ void add_hashes(const BlockCol* col, int width, unsigned long long v,
+                                           unsigned long long* hashes) {
+    const int lane = threadIdx.x & 31;
+    const BlockCol q = lane < width ? col[lane] : BlockCol{0, 0, 0, 0};
+#pragma unroll
+    for (int d = 1; d < kMaxW; d *= 2) {
+        const unsigned long long next = __shfl_down_sync(0xffffffffu, v, d);
+        if (q.off + d < q.width) v += next;
     }
+    if (lane < width && q.off == 0 && v) atomicAdd(hashes + q.index, v);
+}
+
+// Adds the warp's per-column sums, spread over its lanes, to the hashes.
+__device__ __forceinline__ void flush_hash(const BlockCol* col, int width, unsigned long long (&h)[kMaxW],
+                                           unsigned long long* hashes) {
+    unsigned long long mine = 0;
+#pragma unroll
+    for (int c = 0; c < kMaxW; ++c) {
+        unsigned long long v = h[c];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+        if ((threadIdx.x & 31) == c) mine = v;
+    }
+    add_hashes(col, width, mine, hashes);
 }
 
 // Y[:, 0..W) = A X[:, 0..W): V lanes per row, lane h takes entries
@@ -205,7 +261,7 @@ __global__ void __launch_bounds__(kThreads) spmm_kernel(const int32_t* __restric
                 const double a = __ldg(val + k);
                 const double* xr = X + (int64_t)__ldg(col + k) * W;
                 double xv[W];
-                load_row<W>(xr, xv);
+                load_row<W, false>(xr, xv);
 #pragma unroll
                 for (int c = 0; c < W; ++c) acc[c] = fma(a, xv[c], acc[c]);
             }
@@ -217,10 +273,10 @@ __global__ void __launch_bounds__(kThreads) spmm_kernel(const int32_t* __restric
         if (mine && lane == 0) {
 #pragma unroll
             for (int c = 0; c < W; ++c) Y[(int64_t)row * W + c] = acc[c];
-            if (hashes) hash_row<W>(b.req, b.n_req, row, acc, h);
+            if (hashes) hash_row<W>(b.col, row, acc, h);
         }
     }
-    if (hashes) flush_hash(b.req, b.n_req, h, hashes);
+    if (hashes) flush_hash(b.col, b.width, h, hashes);
 }
 
 // Rows from a list (one length bucket of a matrix): V lanes per row, lanes
@@ -253,7 +309,7 @@ __global__ void __launch_bounds__(kThreads) spmm_list_kernel(const int32_t* __re
                 const double a = __ldg(val + k);
                 const double* xr = X + (int64_t)__ldg(col + k) * W;
                 double xv[W];
-                load_row<W>(xr, xv);
+                load_row<W, false>(xr, xv);
 #pragma unroll
                 for (int c = 0; c < W; ++c) acc[c] = fma(a, xv[c], acc[c]);
             }
@@ -265,21 +321,103 @@ __global__ void __launch_bounds__(kThreads) spmm_list_kernel(const int32_t* __re
         if (row >= 0 && lane == 0) {
 #pragma unroll
             for (int c = 0; c < W; ++c) Y[(int64_t)row * W + c] = acc[c];
-            if (hashes) hash_row<W>(b.req, b.n_req, row, acc, h);
+            if (hashes) hash_row<W>(b.col, row, acc, h);
         }
     }
-    if (hashes) flush_hash(b.req, b.n_req, h, hashes);
+    if (hashes) flush_hash(b.col, b.width, h, hashes);
+}
+
+// Sums over the warp's lanes of W columns, with the additions of a full
+// xor-butterfly (offsets 16, 8, 4, 2, 1) per column but without its copies: at
+// each of the first steps a lane keeps the half of its columns that its lane
+// bit names and sends the other half, so 8 columns take 4 + 2 + 1 + 1 + 1 FP64
+// additions instead of 8 x 5, and the result is the same bit for bit.  Returns
+// the total of column `col`, which lane_column gives the lane.
+template <int W, typename T>
+__device__ __forceinline__ T reduce_columns(const T (&acc)[W]) {
+    constexpr int P = pow2_columns(W);
+    const int lane = threadIdx.x & 31;
+    T t[P];
+#pragma unroll
+    for (int c = 0; c < P; ++c) t[c] = c < W ? acc[c < W ? c : 0] : T(0);
+    int off = 16;
+#pragma unroll
+    for (int keep = P / 2; keep >= 1; keep /= 2, off /= 2) {
+        const bool hi = (lane & off) != 0;
+#pragma unroll
+        for (int i = 0; i < keep; ++i) {
+            const T send = hi ? t[i] : t[i + keep], mine = hi ? t[i + keep] : t[i];
+            t[i] = mine + __shfl_xor_sync(0xffffffffu, send, off);
+        }
+    }
+#pragma unroll
+    for (int o = 16 / P; o > 0; o /= 2) t[0] += __shfl_xor_sync(0xffffffffu, t[0], o);
+    return t[0];
+}
+
+// The column whose total reduce_columns leaves in this lane, -1 in the lanes
+// that hold a copy or none.
+template <int W>
+__device__ __forceinline__ int lane_column() {
+    constexpr int per = 32 / pow2_columns(W);   // lanes with the same column
+    const int lane = threadIdx.x & 31;
+    return lane % per == 0 && lane / per < W ? lane / per : -1;
+}
+
+// The warp's column sums in shared memory (kMaxW of them), kept there between
+// the units of a block so that they hold no registers and take few atomics.
+__device__ __forceinline__ void clear_sums(unsigned long long* hs) {
+    if ((threadIdx.x & 31) < kMaxW) hs[threadIdx.x & 31] = 0;
+    __syncwarp();
+}
+__device__ __forceinline__ void flush_sums(const BlockCol* col, int width, unsigned long long* hs,
+                                           unsigned long long* hashes) {
+    __syncwarp();
+    add_hashes(col, width, (threadIdx.x & 31) < kMaxW ? hs[threadIdx.x & 31] : 0ull, hashes);
+    __syncwarp();
+}
+
+// Entries j .. j + K - 1 of a slice lane (of `slots` in the slice), whose columns
+// are in c: their values and X rows, the columns of the next U entries into c
+// (so that the next round's X rows wait for no other load), then the FMAs in
+// entry order (slots past the row discarded).
+template <int W, bool PAD, int K, int U>
+__device__ __forceinline__ void sliced_round(const double* vp, const int32_t* cp, const double* __restrict__ X, int j,
+                                             int slots, int len, int (&c)[U], double (&acc)[W]) {
+    constexpr int ld = PAD ? pow2_columns(W) : W;
+    double a[K], x[K][W];
+#pragma unroll
+    for (int u = 0; u < K; ++u) {
+        load_row<W, PAD>(X + (int64_t)c[u] * ld, x[u]);
+        a[u] = __ldg(vp + 32 * (j + u));
+    }
+    if (K == U) {
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (j + K + u < slots) c[u] = __ldg(cp + 32 * (j + K + u));   // uniform over the warp
+    }
+#pragma unroll
+    for (int u = 0; u < K; ++u) {
+        const bool on = j + u < len;
+#pragma unroll
+        for (int i = 0; i < W; ++i) {
+            const double t = fma(a[u], x[u][i], acc[i]);
+            acc[i] = on ? t : acc[i];
+        }
+    }
 }
 
 // One slice of the matrix's sliced layout (the batch's, see
 // spmv_batch_set_lanes), Y = A X on its rows: one lane per row, each column
-// accumulated in entry order (padded slots discarded by a select), two
-// entries' gathers in flight per lane; with `hashes`, the rows' hash terms
-// go into h.
-template <int W>
+// accumulated in entry order, as many entries' X rows in flight per lane as
+// fit the registers (4, or 2 from width 5 on), the last ones in a round of
+// exactly their number; with `hs` (the warp's column sums in shared memory) the
+// rows' hash terms are added to it.
+template <int W, bool PAD>
 __device__ __forceinline__ void sliced_unit(const BatchMat& m, int si, const double* __restrict__ X,
-                                            double* __restrict__ Y, const BlockReq* req, int n_req,
-                                            unsigned long long* hashes, unsigned long long (&h)[kMaxW]) {
+                                            double* __restrict__ Y, const BlockCol* cols,
+                                            unsigned long long* hs) {
+    constexpr int U = W <= 4 ? 4 : 2;
     const int lane = threadIdx.x & 31;
     const BSlice d = m.s_slices[si];
     const int pos = d.pos0 + lane;
@@ -290,44 +428,44 @@ __device__ __forceinline__ void sliced_unit(const BatchMat& m, int si, const dou
     double acc[W];
 #pragma unroll
     for (int c = 0; c < W; ++c) acc[c] = 0.0;
-    for (int j = 0; j < d.len; j += 2) {
-        const int j1 = j + 1 < d.len ? j + 1 : j;
-        const double a0 = __ldg(vp + 32 * j), a1 = __ldg(vp + 32 * j1);
-        const int c0 = __ldg(cp + 32 * j), c1 = __ldg(cp + 32 * j1);
-        double x0[W], x1[W];
-        load_row<W>(X + (int64_t)c0 * W, x0);
-        load_row<W>(X + (int64_t)c1 * W, x1);
-        const bool on0 = j < len, on1 = j + 1 < len;
+    int cols_now[U], j = 0;
 #pragma unroll
-        for (int c = 0; c < W; ++c) {
-            const double t = fma(a0, x0[c], acc[c]);
-            acc[c] = on0 ? t : acc[c];
-        }
-        if (j + 1 < d.len) {   // uniform over the warp
-#pragma unroll
-            for (int c = 0; c < W; ++c) {
-                const double t = fma(a1, x1[c], acc[c]);
-                acc[c] = on1 ? t : acc[c];
-            }
-        }
+    for (int u = 0; u < U; ++u) cols_now[u] = u < d.len ? __ldg(cp + 32 * u) : 0;
+    for (; j + U <= d.len; j += U) sliced_round<W, PAD, U, U>(vp, cp, X, j, d.len, len, cols_now, acc);
+    switch (d.len - j) {   // uniform over the warp
+        case 1: sliced_round<W, PAD, 1, U>(vp, cp, X, j, d.len, len, cols_now, acc); break;
+        case 2: if (U > 2) sliced_round<W, PAD, (U > 2 ? 2 : 1), U>(vp, cp, X, j, d.len, len, cols_now, acc); break;
+        case 3: if (U > 2) sliced_round<W, PAD, (U > 2 ? 3 : 1), U>(vp, cp, X, j, d.len, len, cols_now, acc); break;
+        default: break;
     }
+    unsigned long long terms[W];
+#pragma unroll
+    for (int c = 0; c < W; ++c) terms[c] = 0;
     if (live) {
         const int row = m.s_perm ? __ldg(m.s_perm + pos) : pos;
 #pragma unroll
         for (int c = 0; c < W; ++c) Y[(int64_t)row * W + c] = acc[c];
-        if (hashes) hash_row<W>(req, n_req, row, acc, h);
+        if (hs) {
+#pragma unroll
+            for (int c = 0; c < W; ++c) terms[c] = hash_term(cols[c], row, acc[c]);
+        }
+    }
+    if (hs) {
+        const unsigned long long v = reduce_columns<W>(terms);
+        const int c = lane_column<W>();
+        if (c >= 0) hs[c] += v;
     }
 }
 
 // The sliced layout's long row at position pos, by the whole warp: lane l
 // takes entries l, l+32, ... in order (four in flight), W accumulators
 // each, then a fixed xor-butterfly.
-template <int W>
+template <int W, bool PAD>
 __device__ __forceinline__ void long_unit(const int32_t* __restrict__ ptr, const int32_t* __restrict__ col,
                                           const double* __restrict__ val, const BatchMat& m, int pos,
                                           const double* __restrict__ X, double* __restrict__ Y,
-                                          const BlockReq* req, int n_req, unsigned long long* hashes,
-                                          unsigned long long (&h)[kMaxW]) {
+                                          const BlockCol* cols, unsigned long long* hs) {
+    constexpr int ld = PAD ? pow2_columns(W) : W;
     const int lane = threadIdx.x & 31;
     const int row = m.s_perm ? __ldg(m.s_perm + pos) : pos;
     const int kb = __ldg(ptr + row), ke = __ldg(ptr + row + 1);
@@ -340,7 +478,7 @@ __device__ __forceinline__ void long_unit(const int32_t* __restrict__ ptr, const
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             a[u] = __ldg(val + k + 32 * u);
-            load_row<W>(X + (int64_t)__ldg(col + k + 32 * u) * W, xv[u]);
+            load_row<W, PAD>(X + (int64_t)__ldg(col + k + 32 * u) * ld, xv[u]);
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u)
@@ -350,34 +488,31 @@ __device__ __forceinline__ void long_unit(const int32_t* __restrict__ ptr, const
     for (; k < ke; k += 32) {
         const double a = __ldg(val + k);
         double xv[W];
-        load_row<W>(X + (int64_t)__ldg(col + k) * W, xv);
+        load_row<W, PAD>(X + (int64_t)__ldg(col + k) * ld, xv);
 #pragma unroll
         for (int c = 0; c < W; ++c) acc[c] = fma(a, xv[c], acc[c]);
     }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1)
-#pragma unroll
-        for (int c = 0; c < W; ++c) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], off);
-    if (lane == 0) {
-#pragma unroll
-        for (int c = 0; c < W; ++c) Y[(int64_t)row * W + c] = acc[c];
-        if (hashes) hash_row<W>(req, n_req, row, acc, h);
+    const double y = reduce_columns<W>(acc);
+    const int c = lane_column<W>();
+    if (c >= 0) {
+        Y[(int64_t)row * W + c] = y;
+        if (hs) hs[c] += hash_term(cols[c], row, y);
     }
 }
 
 // A long row of more than 2048 entries by the whole CTA: thread t takes
 // entries t, t+256, ... in order (four in flight), W accumulators each, a
 // fixed xor-butterfly in each warp, then the eight warps' sums added in warp
-// order through shared memory; thread 0 stores the row.  All threads of the
-// CTA call it for the same row.
-template <int W>
+// order through shared memory, a column per thread.  All threads of the CTA
+// call it for the same row.
+template <int W, bool PAD>
 __device__ __forceinline__ void long_cta_unit(const int32_t* __restrict__ ptr, const int32_t* __restrict__ col,
                                               const double* __restrict__ val, const BatchMat& m, int pos,
                                               const double* __restrict__ X, double* __restrict__ Y,
-                                              const BlockReq* req, int n_req, unsigned long long* hashes,
-                                              unsigned long long (&h)[kMaxW]) {
+                                              const BlockCol* cols, unsigned long long* hs) {
+    constexpr int ld = PAD ? pow2_columns(W) : W;
     __shared__ double s_part[kThreads / 32][kMaxW];
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int t = threadIdx.x, warp = t >> 5;
     const int row = m.s_perm ? __ldg(m.s_perm + pos) : pos;
     const int kb = __ldg(ptr + row), ke = __ldg(ptr + row + 1);
     double acc[W];
@@ -389,7 +524,7 @@ __device__ __forceinline__ void long_cta_unit(const int32_t* __restrict__ ptr, c
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             a[u] = __ldg(val + k + kThreads * u);
-            load_row<W>(X + (int64_t)__ldg(col + k + kThreads * u) * W, xv[u]);
+            load_row<W, PAD>(X + (int64_t)__ldg(col + k + kThreads * u) * ld, xv[u]);
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u)
@@ -399,28 +534,20 @@ __device__ __forceinline__ void long_cta_unit(const int32_t* __restrict__ ptr, c
     for (; k < ke; k += kThreads) {
         const double a = __ldg(val + k);
         double xv[W];
-        load_row<W>(X + (int64_t)__ldg(col + k) * W, xv);
+        load_row<W, PAD>(X + (int64_t)__ldg(col + k) * ld, xv);
 #pragma unroll
         for (int c = 0; c < W; ++c) acc[c] = fma(a, xv[c], acc[c]);
     }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1)
-#pragma unroll
-        for (int c = 0; c < W; ++c) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], off);
-    if (lane == 0) {
-#pragma unroll
-        for (int c = 0; c < W; ++c) s_part[warp][c] = acc[c];
-    }
+    const double part = reduce_columns<W>(acc);
+    const int c = lane_column<W>();
+    if (c >= 0) s_part[warp][c] = part;
     __syncthreads();
-    if (t == 0) {
+    if (t < W) {
+        double y = s_part[0][t];
 #pragma unroll
-        for (int c = 0; c < W; ++c) acc[c] = s_part[0][c];
-        for (int w = 1; w < kThreads / 32; ++w)
-#pragma unroll
-            for (int c = 0; c < W; ++c) acc[c] += s_part[w][c];
-#pragma unroll
-        for (int c = 0; c < W; ++c) Y[(int64_t)row * W + c] = acc[c];
-        if (hashes) hash_row<W>(req, n_req, row, acc, h);
+        for (int w = 1; w < kThreads / 32; ++w) y += s_part[w][t];
+        Y[(int64_t)row * W + t] = y;
+        if (hs) hs[t] += hash_term(cols[t], row, y);
     }
     __syncthreads();   // s_part is reused by the CTA's next unit
 }
@@ -432,173 +559,161 @@ __host__ __device__ __forceinline__ int long_units(const BatchMat& m) {
 }
 
 // Long-row unit u of a matrix by the calling CTA (all its threads).
-template <int W>
+template <int W, bool PAD>
 __device__ __forceinline__ void long_units_run(const int32_t* ptr, const int32_t* col, const double* val,
                                                const BatchMat& m, int u, const double* X, double* Y,
-                                               const BlockReq* req, int n_req, unsigned long long* hashes,
-                                               unsigned long long (&h)[kMaxW]) {
+                                               const BlockCol* cols, unsigned long long* hs) {
     if (u < m.n_vlong) {
-        long_cta_unit<W>(ptr, col, val, m, u, X, Y, req, n_req, hashes, h);
+        long_cta_unit<W, PAD>(ptr, col, val, m, u, X, Y, cols, hs);
     } else {
         const int pos = m.n_vlong + (u - m.n_vlong) * (kThreads / 32) + (int)(threadIdx.x >> 5);
-        if (pos < m.n_long) long_unit<W>(ptr, col, val, m, pos, X, Y, req, n_req, hashes, h);
+        if (pos < m.n_long) long_unit<W, PAD>(ptr, col, val, m, pos, X, Y, cols, hs);
     }
 }
 
-// One block over the sliced layout: one warp per slice (grid-stride).
-// Registers capped so that 4 CTAs (widths 1-3) or 3 CTAs (widths 4-8) fit an
-// SM without spills; uncapped, width 4 took 128 registers (2 CTAs).
-template <int W>
-__global__ void __launch_bounds__(kThreads, (W <= 3 ? 4 : 3)) spmm_sliced_kernel(BatchMat m, const double* __restrict__ X,
-                                                               double* __restrict__ Y, BlockDesc b,
-                                                               unsigned long long* __restrict__ hashes) {
-    unsigned long long h[kMaxW];
-#pragma unroll
-    for (int r = 0; r < kMaxW; ++r) h[r] = 0;
-    const int nw = (int)gridDim.x * (kThreads / 32);
-    for (int si = (int)blockIdx.x * (kThreads / 32) + (int)(threadIdx.x >> 5); si < m.n_slices; si += nw)
-        sliced_unit<W>(m, si, X, Y, b.req, b.n_req, hashes, h);
-    if (hashes) flush_hash(b.req, b.n_req, h, hashes);
+// Work units of a block, one per CTA: its matrix's long-row units and its
+// slices eight at a time, one per warp.
+__host__ __device__ __forceinline__ int block_units(const BatchMat& m) {
+    return long_units(m) + (m.n_slices + kThreads / 32 - 1) / (kThreads / 32);
 }
 
-// One block's long rows (positions [0, n_long)): its long-row units, one per
-// CTA (grid-stride).
-template <int W>
-__global__ void __launch_bounds__(kThreads) spmm_long_kernel(const int32_t* __restrict__ ptr,
-                                                             const int32_t* __restrict__ col,
-                                                             const double* __restrict__ val, BatchMat m,
-                                                             const double* __restrict__ X, double* __restrict__ Y,
-                                                             BlockDesc b, unsigned long long* __restrict__ hashes) {
-    unsigned long long h[kMaxW];
-#pragma unroll
-    for (int r = 0; r < kMaxW; ++r) h[r] = 0;
-    const int units = long_units(m);
+// Unit u of a block.  The long-row units (bound by the FP64 pipe) are spread
+// evenly among the slices (bound by their loads), so that the two overlap; both
+// come longest first.
+template <int W, bool PAD>
+__device__ __forceinline__ void block_unit(const int32_t* ptr, const int32_t* col, const double* val,
+                                           const BatchMat& m, int u, const double* X, double* Y,
+                                           const BlockCol* cols, unsigned long long* hs) {
+    const long long nl = long_units(m), n = block_units(m);
+    const int k = (int)(u * nl / n);   // long-row units before this one
+    if ((int)((u + 1) * nl / n) > k) {
+        long_units_run<W, PAD>(ptr, col, val, m, k, X, Y, cols, hs);
+    } else {
+        const int si = (u - k) * (kThreads / 32) + (int)(threadIdx.x >> 5);
+        if (si < m.n_slices) sliced_unit<W, PAD>(m, si, X, Y, cols, hs);
+    }
+}
+
+// One block over the sliced layout (CTAs grid-stride over its units).
+// Registers capped so that 4 CTAs (widths 1-3) or 3 CTAs (widths 4-8) fit an
+// SM without spills; uncapped, width 4 took 128 registers (2 CTAs).
+template <int W, bool PAD>
+__global__ void __launch_bounds__(kThreads, (W <= 3 ? 4 : 3)) spmm_block_kernel(const int32_t* __restrict__ ptr,
+                                                                                const int32_t* __restrict__ col,
+                                                                                const double* __restrict__ val,
+                                                                                BatchMat m,
+                                                                                const double* __restrict__ X,
+                                                                                double* __restrict__ Y, BlockDesc b,
+                                                                                unsigned long long* __restrict__ hashes) {
+    spmvk::pdl_wait();   // X is drawn by the kernel before this one
+    __shared__ unsigned long long s_hash[kThreads / 32][kMaxW];
+    unsigned long long* hs = hashes ? s_hash[threadIdx.x >> 5] : nullptr;
+    if (hs) clear_sums(hs);
+    const int units = block_units(m);
     for (int u = (int)blockIdx.x; u < units; u += (int)gridDim.x)
-        long_units_run<W>(ptr, col, val, m, u, X, Y, b.req, b.n_req, hashes, h);
-    if (hashes) flush_hash(b.req, b.n_req, h, hashes);
+        block_unit<W, PAD>(ptr, col, val, m, u, X, Y, b.col, hs);
+    if (hs) flush_sums(b.col, b.width, hs, hashes);
 }
 
 // ---------------------------------------------------------------- groups
 // A group: up to kGroupMax blocks, possibly of different matrices and
-// widths, run by one launch per kernel kind.  Block i's X sits at x_off
-// (doubles from the pool base), its Y right after (n x width each); its
-// slices are the group's units [unit0, next unit0), its long rows the long
-// units [long0, next long0).
+// widths, run by one launch that draws their X and one that multiplies.  Block i's X sits at x_off
+// (doubles from the pool base; n x pow2_columns(width)), its Y right after
+// (n x width); its units
+// (block_unit) are the group's units [unit0, next unit0).
 constexpr int kGroupMax = 64;
 
 struct GroupBlock {
     BlockReq req[kMaxW];
+    BlockCol col[kMaxW];
     long long x_off;
     int n_req, width, m, n;
-    int unit0, long0, pad0, pad1;
+    int unit0, pad0, pad1, pad2;
 };
 
 __global__ void gen_group_kernel(double* __restrict__ pool, const GroupBlock* __restrict__ g) {
     const GroupBlock& b = g[blockIdx.y];
-    gen_x(pool + b.x_off, b.n, b.width, b.req, b.n_req, (int)(blockIdx.x * blockDim.x + threadIdx.x),
+    gen_x(pool + b.x_off, b.n, b.width, pow2_columns(b.width), b.req, b.n_req, (int)(blockIdx.x * blockDim.x + threadIdx.x),
           (int)(gridDim.x * blockDim.x));
 }
 
-// Units [0, units) of a group, one warp per unit (grid-stride); LONG picks
-// the long-row units.  The unit's block is found by binary search over the
-// blocks' first units; each unit's hash terms are flushed before the next.
-template <bool LONG>
-__global__ void __launch_bounds__(kThreads) spmm_group_kernel(const BatchMat* __restrict__ mats,
-                                                              const int32_t* __restrict__ ptr,
-                                                              const int32_t* __restrict__ col,
-                                                              const double* __restrict__ val,
-                                                              double* __restrict__ pool,
-                                                              const GroupBlock* __restrict__ g, int nb, int units,
-                                                              unsigned long long* __restrict__ hashes) {
+// Units [0, units) of a group, one per CTA (grid-stride).  The unit's block is
+// found by binary search over the blocks' first units; the hash sums are flushed
+// when the block changes.
+__global__ void __launch_bounds__(kThreads, 3) spmm_group_kernel(const BatchMat* __restrict__ mats,
+                                                                 const int32_t* __restrict__ ptr,
+                                                                 const int32_t* __restrict__ col,
+                                                                 const double* __restrict__ val,
+                                                                 double* __restrict__ pool,
+                                                                 const GroupBlock* __restrict__ g, int nb, int units,
+                                                                 unsigned long long* __restrict__ hashes) {
     __shared__ int s_first[kGroupMax + 1];
-    for (int i = threadIdx.x; i <= nb; i += blockDim.x) s_first[i] = i < nb ? (LONG ? g[i].long0 : g[i].unit0) : units;
+    for (int i = threadIdx.x; i <= nb; i += blockDim.x) s_first[i] = i < nb ? g[i].unit0 : units;
     __syncthreads();
-    unsigned long long h[kMaxW];
-#pragma unroll
-    for (int r = 0; r < kMaxW; ++r) h[r] = 0;
-    // slice units one per warp; long-row units one per CTA (long_units)
-    const int nw = LONG ? (int)gridDim.x : (int)gridDim.x * (kThreads / 32);
-    const int u0 = LONG ? (int)blockIdx.x : (int)blockIdx.x * (kThreads / 32) + (int)(threadIdx.x >> 5);
-    for (int u = u0; u < units; u += nw) {
+    __shared__ unsigned long long s_hash[kThreads / 32][kMaxW];
+    unsigned long long* hs = hashes ? s_hash[threadIdx.x >> 5] : nullptr;
+    if (hs) clear_sums(hs);
+    int at = -1;   // block of the unit before
+    for (int u = (int)blockIdx.x; u < units; u += (int)gridDim.x) {
         int lo = 0, hi = nb - 1;   // the last block whose first unit is <= u
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
             if (s_first[mid] <= u) lo = mid;
             else hi = mid - 1;
         }
-        const GroupBlock& b = g[lo];
-        const BatchMat m = mats[b.m];
-        double* X = pool + b.x_off;
-        double* Y = X + (int64_t)b.n * b.width;
-        const int k = u - s_first[lo];
-        if (LONG) {
-            const int32_t* mp = ptr + m.ptr_off;
-            const int32_t* mc = col + m.ent_off;
-            const double* mv = val + m.ent_off;
-            switch (b.width) {
-                case 1: long_units_run<1>(mp, mc, mv, m, k, X, Y, b.req, b.n_req, hashes, h); break;
-                case 2: long_units_run<2>(mp, mc, mv, m, k, X, Y, b.req, b.n_req, hashes, h); break;
-                case 3: long_units_run<3>(mp, mc, mv, m, k, X, Y, b.req, b.n_req, hashes, h); break;
-                case 4: long_units_run<4>(mp, mc, mv, m, k, X, Y, b.req, b.n_req, hashes, h); break;
-                case 5: long_units_run<5>(mp, mc, mv, m, k, X, Y, b.req, b.n_req, hashes, h); break;
-                case 6: long_units_run<6>(mp, mc, mv, m, k, X, Y, b.req, b.n_req, hashes, h); break;
-                case 7: long_units_run<7>(mp, mc, mv, m, k, X, Y, b.req, b.n_req, hashes, h); break;
-                default: long_units_run<8>(mp, mc, mv, m, k, X, Y, b.req, b.n_req, hashes, h); break;
-            }
-        } else {
-            switch (b.width) {
-                case 1: sliced_unit<1>(m, k, X, Y, b.req, b.n_req, hashes, h); break;
-                case 2: sliced_unit<2>(m, k, X, Y, b.req, b.n_req, hashes, h); break;
-                case 3: sliced_unit<3>(m, k, X, Y, b.req, b.n_req, hashes, h); break;
-                case 4: sliced_unit<4>(m, k, X, Y, b.req, b.n_req, hashes, h); break;
-                case 5: sliced_unit<5>(m, k, X, Y, b.req, b.n_req, hashes, h); break;
-                case 6: sliced_unit<6>(m, k, X, Y, b.req, b.n_req, hashes, h); break;
-                case 7: sliced_unit<7>(m, k, X, Y, b.req, b.n_req, hashes, h); break;
-                default: sliced_unit<8>(m, k, X, Y, b.req, b.n_req, hashes, h); break;
-            }
+        if (hs && at >= 0 && at != lo) {
+            flush_sums(g[at].col, g[at].width, hs, hashes);
+            clear_sums(hs);
         }
-        if (hashes) flush_hash(b.req, b.n_req, h, hashes);
+        at = lo;
+        const GroupBlock& b = g[lo];
+        const BatchMat& m = mats[b.m];
+        double* X = pool + b.x_off;
+        double* Y = X + (int64_t)b.n * pow2_columns(b.width);
+        const int k = u - s_first[lo];
+        const int32_t* mp = ptr + m.ptr_off;
+        const int32_t* mc = col + m.ent_off;
+        const double* mv = val + m.ent_off;
+        switch (b.width) {
+            case 1: block_unit<1, true>(mp, mc, mv, m, k, X, Y, b.col, hs); break;
+            case 2: block_unit<2, true>(mp, mc, mv, m, k, X, Y, b.col, hs); break;
+            case 3: block_unit<3, true>(mp, mc, mv, m, k, X, Y, b.col, hs); break;
+            case 4: block_unit<4, true>(mp, mc, mv, m, k, X, Y, b.col, hs); break;
+            case 5: block_unit<5, true>(mp, mc, mv, m, k, X, Y, b.col, hs); break;
+            case 6: block_unit<6, true>(mp, mc, mv, m, k, X, Y, b.col, hs); break;
+            case 7: block_unit<7, true>(mp, mc, mv, m, k, X, Y, b.col, hs); break;
+            default: block_unit<8, true>(mp, mc, mv, m, k, X, Y, b.col, hs); break;
+        }
     }
+    if (hs && at >= 0) flush_sums(g[at].col, g[at].width, hs, hashes);
 }
 
-cudaError_t launch_sliced(const BlockDesc& b, const int32_t* ptr, const int32_t* col, const double* val,
+cudaError_t launch_sliced(const BlockDesc& b, bool pad, const int32_t* ptr, const int32_t* col, const double* val,
                           const BatchMat& M, const double* X, double* Y, int num_sms, unsigned long long* hashes,
                           cudaStream_t s, int64_t& launches) {
-    constexpr int WPB = kThreads / 32;
-    launches += (M.n_slices > 0) + (M.n_long > 0);
-    if (M.n_slices > 0) {
-        const int grid = std::min((M.n_slices + WPB - 1) / WPB, num_sms * 8);
-#define SPMM_SL(w) spmm_sliced_kernel<w><<<grid, kThreads, 0, s>>>(M, X, Y, b, hashes)
-        switch (b.width) {
-            case 1: SPMM_SL(1); break;
-            case 2: SPMM_SL(2); break;
-            case 3: SPMM_SL(3); break;
-            case 4: SPMM_SL(4); break;
-            case 5: SPMM_SL(5); break;
-            case 6: SPMM_SL(6); break;
-            case 7: SPMM_SL(7); break;
-            default: SPMM_SL(8); break;
-        }
-#undef SPMM_SL
-        const cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
+    const int units = block_units(M);
+    if (units == 0) return cudaSuccess;
+    ++launches;
+    // skewed matrices: up to 24 CTAs per SM, so that the hardware hands out units
+    // of uneven length (600 000 Zipf rows, width 8: 132 us against 182 us with
+    // one resident wave); else one wave, whose warps go on to their next slice
+    // without a new CTA (7-point 80 x 81 x 80, width 8: 76 us against 82 us)
+    const int per_sm = M.s_perm ? 24 : b.width <= 3 ? 4 : 3;
+    const int grid = std::min(units, num_sms * per_sm);
+#define SPMM_BLOCK(w) \
+    return launch_pdl(pad ? spmm_block_kernel<w, true> : spmm_block_kernel<w, false>, \
+                      dim3(grid), dim3(kThreads), 0, s, ptr, col, val, M, X, Y, b, hashes)
+    switch (b.width) {
+        case 1: SPMM_BLOCK(1);
+        case 2: SPMM_BLOCK(2);
+        case 3: SPMM_BLOCK(3);
+        case 4: SPMM_BLOCK(4);
+        case 5: SPMM_BLOCK(5);
+        case 6: SPMM_BLOCK(6);
+        case 7: SPMM_BLOCK(7);
+        default: SPMM_BLOCK(8);
     }
-    if (M.n_long > 0) {
-        const int grid = std::min(long_units(M), num_sms * 8);
-#define SPMM_LG(w) spmm_long_kernel<w><<<grid, kThreads, 0, s>>>(ptr, col, val, M, X, Y, b, hashes)
-        switch (b.width) {
-            case 1: SPMM_LG(1); break;
-            case 2: SPMM_LG(2); break;
-            case 3: SPMM_LG(3); break;
-            case 4: SPMM_LG(4); break;
-            case 5: SPMM_LG(5); break;
-            case 6: SPMM_LG(6); break;
-            case 7: SPMM_LG(7); break;
-            default: SPMM_LG(8); break;
-        }
-#undef SPMM_LG
-    }
-    return cudaGetLastError();
+#undef SPMM_BLOCK
 }
 
 template <int V>
@@ -725,7 +840,14 @@ int sfail(int code, const std::string& m) {
     return code;
 }
 
-cudaError_t launch_block(spmv_server* sv, int m, const BlockDesc& b, double* X, double* Y,
+// Whether a block's X has the padded leading dimension of the pool (sliced
+// layout; the CSR-layout kernels read X with leading dimension width).
+bool pads(const spmv_server* sv, int m) { return sv->mats->mats[m].lanes == kBatchSliced; }
+int x_columns(const spmv_server* sv, int m, int width) { return pads(sv, m) ? pow2_columns(width) : width; }
+
+// One block: its X drawn, then its product.  `pad`: X has x_columns columns and
+// starts at a multiple of 32 bytes; else its leading dimension is the width.
+cudaError_t launch_block(spmv_server* sv, int m, const BlockDesc& b, bool pad, double* X, double* Y,
                          unsigned long long* hashes, cudaStream_t s) {
     spmv_batch* bt = sv->mats;
     const BatchMat& M = bt->mats[m];
@@ -733,7 +855,7 @@ cudaError_t launch_block(spmv_server* sv, int m, const BlockDesc& b, double* X, 
     if (n == 0) return cudaSuccess;
     sv->launches += 2;   // X generator, product over the short rows (or the slices)
     int g = (int)std::min<int64_t>(((int64_t)n * b.width + kThreads - 1) / kThreads, (int64_t)sv->num_sms * 8);
-    gen_x_kernel<<<g, kThreads, 0, s>>>(X, n, b);
+    gen_x_kernel<<<g, kThreads, 0, s>>>(X, n, pad ? pow2_columns(b.width) : b.width, b);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int32_t* ptr = bt->ptr + M.ptr_off;
@@ -741,7 +863,7 @@ cudaError_t launch_block(spmv_server* sv, int m, const BlockDesc& b, double* X, 
     const double* val = bt->val + M.ent_off;
     if (M.lanes == kBatchSliced) {
         sv->launches -= 1;
-        return launch_sliced(b, ptr, col, val, M, X, Y, sv->num_sms, hashes, s, sv->launches);
+        return launch_sliced(b, pad, ptr, col, val, M, X, Y, sv->num_sms, hashes, s, sv->launches);
     }
     const int V = sv->lanes[m];
     int grid = (int)std::min<int64_t>((n + (kThreads / V) - 1) / (kThreads / V), (int64_t)sv->num_sms * 8);
@@ -924,7 +1046,10 @@ int spmv_serve_single(spmv_server* sv, int matrix, int width, uint64_t seed, dou
     b.n_req = 1;
     b.width = width;
     b.req[0] = BlockReq{seed, 0, width, 0, 0};
-    spmvk::check_cuda(launch_block(sv, matrix, b, x_dev, y_dev, nullptr, s), "single request");
+    set_columns(b.req, 1, b.col);
+    // the caller's X has leading dimension width: the padded one's where they agree
+    const bool pad = pads(sv, matrix) && pow2_columns(width) == width && reinterpret_cast<uintptr_t>(x_dev) % 32 == 0;
+    spmvk::check_cuda(launch_block(sv, matrix, b, pad, x_dev, y_dev, nullptr, s), "single request");
     SERVE_CATCH
     return SPMV_OK;
 }
@@ -1044,7 +1169,7 @@ int spmv_serve_run(spmv_server* sv, int64_t n_req, const int32_t* matrix, const 
                 if (slot[i].busy) continue;
                 if (grouped && per_group > 1) {
                     GroupBlock* hg = sv->h_group[i];
-                    int nb = 0, units = 0, longs = 0, max_elems = 0;
+                    int nb = 0, units = 0, max_elems = 0;
                     bool out_of_memory = false;
                     while (nb < per_group && queued > 0 && !out_of_memory) {
                         const int m = oldest();
@@ -1054,7 +1179,7 @@ int spmv_serve_run(spmv_server* sv, int64_t n_req, const int32_t* matrix, const 
                         int take = 0, wsum = 0;
                         while (take < (int)q.size() && take < kMaxW && wsum + width[q[take]] <= kMaxW)
                             wsum += width[q[take++]];
-                        const size_t bytes = (size_t)2 * Mm.n * wsum * sizeof(double);
+                        const size_t bytes = (size_t)Mm.n * (x_columns(sv, m, wsum) + wsum) * sizeof(double);
                         const long long off = sv->pool.alloc(bytes);
                         if (off < 0) {
                             ++waits_mem;
@@ -1070,14 +1195,13 @@ int spmv_serve_run(spmv_server* sv, int64_t n_req, const int32_t* matrix, const 
                             slot[i].reqs.push_back(r);
                             q.pop_front();
                         }
+                        set_columns(gb.req, gb.n_req, gb.col);
                         gb.x_off = off / (long long)sizeof(double);
                         gb.width = wsum;
                         gb.m = m;
                         gb.n = Mm.n;
                         gb.unit0 = units;
-                        gb.long0 = longs;
-                        units += Mm.n_slices;
-                        longs += long_units(Mm);
+                        units += block_units(Mm);
                         max_elems = std::max(max_elems, Mm.n * wsum);
                         queued -= take;
                         pend_width[m] -= wsum;
@@ -1098,15 +1222,11 @@ int spmv_serve_run(spmv_server* sv, int64_t n_req, const int32_t* matrix, const 
                         ++sv->launches;
                     }
                     if (units > 0) {
-                        const int gs = std::min((units + 7) / 8, sv->num_sms * 8);
-                        spmm_group_kernel<false><<<gs, kThreads, 0, st>>>(bt->d_mats, bt->ptr, bt->col, bt->val, pool,
-                                                                         sv->d_group[i], nb, units, hs);
-                        ++sv->launches;
-                    }
-                    if (longs > 0) {
-                        const int gl = std::min(longs, sv->num_sms * 8);   // one CTA per long-row unit
-                        spmm_group_kernel<true><<<gl, kThreads, 0, st>>>(bt->d_mats, bt->ptr, bt->col, bt->val, pool,
-                                                                        sv->d_group[i], nb, longs, hs);
+                        // one resident wave: 200 requests on 12 matrices
+                        // 4.56 ms against 4.94 ms with 24 CTAs per SM
+                        const int gs = std::min(units, sv->num_sms * 3);
+                        spmm_group_kernel<<<gs, kThreads, 0, st>>>(bt->d_mats, bt->ptr, bt->col, bt->val, pool,
+                                                                  sv->d_group[i], nb, units, hs);
                         ++sv->launches;
                     }
                     spmvk::check_cuda(cudaGetLastError(), "group launch");
@@ -1128,7 +1248,8 @@ int spmv_serve_run(spmv_server* sv, int64_t n_req, const int32_t* matrix, const 
                     ++take;
                     if (mode == SPMV_SERVE_PLAIN) break;   // one request per launch
                 }
-                const size_t bytes = (size_t)2 * n * wsum * sizeof(double);   // X and Y, ld wsum
+                const int xc = x_columns(sv, m, wsum);
+                const size_t bytes = (size_t)n * (xc + wsum) * sizeof(double);   // X and Y
                 const long long off = sv->pool.alloc(bytes);
                 if (off < 0) {   // over budget: wait for memory to free up
                     ++waits_mem;
@@ -1144,11 +1265,12 @@ int spmv_serve_run(spmv_server* sv, int64_t n_req, const int32_t* matrix, const 
                     q.pop_front();
                 }
                 b.width = wsum;
+                set_columns(b.req, b.n_req, b.col);
                 queued -= (int64_t)reqs.size();
                 pend_width[m] -= wsum;
                 double* X = reinterpret_cast<double*>(sv->pool.ptr(off));
-                double* Y = X + (size_t)n * b.width;
-                spmvk::check_cuda(launch_block(sv, m, b, X, Y, hash_out ? sv->d_hash : nullptr,
+                double* Y = X + (size_t)n * xc;
+                spmvk::check_cuda(launch_block(sv, m, b, pads(sv, m), X, Y, hash_out ? sv->d_hash : nullptr,
                                                sv->streams[i]),
                                   "block launch");
                 spmvk::check_cuda(cudaEventRecord(sv->events[i], sv->streams[i]), "event");
