@@ -370,6 +370,10 @@ int spmv_apply_host_pipelined(spmv_part* part, const double* x_host, double* y_h
  *   every copy costs a few microseconds beyond its bytes, so in a stream of
  *   products, where the next product's transfers already fill the link,
  *   fewer copies can be faster.  The results do not depend on the flags.
+ *   Without SPMV_HOST_X_BLOCKS, streams of products with at most 600 000 P
+ *   rows (two products: 131 072 P, one: 65 536 P) run each operation in one
+ *   launch over all ranks on compute_stream and return y in one copy, whatever
+ *   SPMV_HOST_Y_PARTS says.
  *   Streams: as spmv_apply_host_pipelined (the two must differ).  Returns
  *   after every y_k has arrived.  The second pair of device vectors (16 n
  *   bytes) is allocated by the first call and kept with the plan.

@@ -378,9 +378,13 @@ void issue(spmv_part* pt, const int32_t* order, const int32_t* stream_of, int n_
     std::vector<char> used(n_streams, 0);
     for (int v = 0; v < n_ops; ++v) used[stream_of[v]] = 1;
     // start vertex: fork every other used stream from the origin
-    check_cuda(cudaEventRecord(pt->fork_ev, origin), "fork record");
-    for (int s = 1; s < n_streams; ++s)
-        if (used[s]) check_cuda(cudaStreamWaitEvent(streams[s], pt->fork_ev, 0), "fork wait");
+    bool forked = false;
+    for (int s = 1; s < n_streams; ++s) {
+        if (!used[s]) continue;
+        if (!forked) check_cuda(cudaEventRecord(pt->fork_ev, origin), "fork record");
+        forked = true;
+        check_cuda(cudaStreamWaitEvent(streams[s], pt->fork_ev, 0), "fork wait");
+    }
     // which ops feed a successor bound to another stream (any successor in
     // relaxed mode)
     std::vector<char> cross(n_ops, 0);
@@ -955,6 +959,7 @@ void host_path_setup(spmv_part* pt) {
     if (!pt->io_x) {
         pt->io_x = static_cast<double*>(spmvk::dev_alloc(pt, (size_t)pt->n * sizeof(double)));
         pt->io_y = static_cast<double*>(spmvk::dev_alloc(pt, (size_t)pt->n * sizeof(double)));
+        check_cuda(cudaDeviceSynchronize(), "synchronize");   // zero-filled before other streams write
     }
     while ((int)pt->io_ev.size() < 3 * P + 5) {
         cudaEvent_t e;
@@ -1088,6 +1093,49 @@ int64_t host_product(spmv_part* pt, const double* x_host, double* y_host, double
     return launches;
 }
 
+// The same product for the stream of small ones: x in one copy, one launch per
+// operation over all ranks, one after another on compute_stream (which then
+// also orders the send and receive buffers' uses), y in one copy.  14 calls
+// where the form above makes 23 + 10 P, with no event between the operations.
+// Same kernels on the same rows.
+int64_t host_product_coarse(spmv_part* pt, const double* x_host, double* y_host, double* xd, double* yd,
+                            cudaStream_t copy_stream, cudaStream_t compute_stream, int slot) {
+    const int P = pt->P;
+    cudaStream_t out_stream = pt->io_out;
+    cudaEvent_t* ev = pt->io_ev.data();
+    const cudaEvent_t x_here = ev[0], done = ev[2 * P], x_free = ev[3 * P + 1 + slot], y_free = ev[3 * P + 3 + slot];
+    auto wait = [](cudaStream_t s, cudaEvent_t e) { check_cuda(cudaStreamWaitEvent(s, e, 0), "wait"); };
+    auto record = [](cudaEvent_t e, cudaStream_t s) { check_cuda(cudaEventRecord(e, s), "event"); };
+    const size_t bytes = (size_t)pt->n * sizeof(double);
+    wait(copy_stream, x_free);
+    check_cuda(cudaMemcpyAsync(xd, x_host, bytes, cudaMemcpyHostToDevice, copy_stream), "copy x in");
+    record(x_here, copy_stream);
+    wait(compute_stream, x_here);
+    wait(compute_stream, y_free);
+    int64_t launches = op_local(pt, -1, xd, yd, compute_stream);
+    launches += op_pack(pt, -1, xd, compute_stream);
+    record(x_free, compute_stream);
+    launches += op_copy(pt, -1, compute_stream);
+    launches += op_remote(pt, -1, yd, compute_stream);
+    record(done, compute_stream);
+    wait(out_stream, done);
+    check_cuda(cudaMemcpyAsync(y_host, yd, bytes, cudaMemcpyDeviceToHost, out_stream), "copy y out");
+    record(y_free, out_stream);
+    return launches;
+}
+
+// Whether a stream of `count` products takes host_product_coarse (x in one
+// copy).  It saves the host's calls and the events between the operations; the
+// form rank by rank lets a product's first rows leave while its last ranks
+// compute, which only a short stream of large products feels.  27-point, us per
+// call, rank by rank and here: 20^3 4 ranks 4 products 169 and 78, 64^3 1 product
+// 81 and 78, 80^3 4 products 282 and 229, 90^3 1 product 125 and 138, 130^3 4
+// products 733 and 714, 16 products 2818 and 2374.
+bool host_coarse(const spmv_part* pt, int64_t count) {
+    const int64_t per_rank = count == 1 ? 65536 : count == 2 ? 131072 : 600000;
+    return pt->n <= per_rank * pt->P;
+}
+
 }  // namespace
 
 int spmv_apply_host_pipelined(spmv_part* pt, const double* x_host, double* y_host, cudaStream_t copy_stream,
@@ -1123,10 +1171,18 @@ int spmv_apply_host_many(spmv_part* pt, int64_t count, const double* x_host, int
     if (!pt->io_x2) {
         pt->io_x2 = static_cast<double*>(spmvk::dev_alloc(pt, (size_t)pt->n * sizeof(double)));
         pt->io_y2 = static_cast<double*>(spmvk::dev_alloc(pt, (size_t)pt->n * sizeof(double)));
+        check_cuda(cudaDeviceSynchronize(), "synchronize");   // zero-filled before other streams write
     }
     int64_t launches = 0;
+    const bool coarse = !(flags & SPMV_HOST_X_BLOCKS) && host_coarse(pt, count);
     for (int64_t k = 0; k < count; ++k) {
         const int slot = (int)(k & 1);
+        if (coarse) {
+            launches += host_product_coarse(pt, x_host + k * x_stride, y_host + k * y_stride,
+                                            slot ? pt->io_x2 : pt->io_x, slot ? pt->io_y2 : pt->io_y, copy_stream,
+                                            compute_stream, slot);
+            continue;
+        }
         launches += host_product(pt, x_host + k * x_stride, y_host + k * y_stride, slot ? pt->io_x2 : pt->io_x,
                                  slot ? pt->io_y2 : pt->io_y, copy_stream, compute_stream, slot,
                                  (flags & SPMV_HOST_X_BLOCKS) != 0, (flags & SPMV_HOST_Y_PARTS) != 0);

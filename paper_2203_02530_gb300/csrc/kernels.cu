@@ -378,10 +378,15 @@ static cudaError_t run_tile(const CsrArgs& a, const Tile* tiles, int tb, int te,
         if (e != cudaSuccess) return e;
         if (dev < 64) configured.fetch_or(1ull << dev, std::memory_order_acq_rel);
     }
-    int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, csr_tile_kernel<U, S>, kTileWarps * 32, smem);
-    if (e != cudaSuccess) return e;
-    if (occ < 1) return cudaErrorInvalidConfiguration;
+    // CTAs per SM by stage size (a query costs the host about a microsecond)
+    static std::atomic<int> known[kTileMaxEntries / 32 + 1];
+    int occ = dev == 0 ? known[cap / 32].load(std::memory_order_relaxed) : 0;
+    if (occ == 0) {
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, csr_tile_kernel<U, S>, kTileWarps * 32, smem);
+        if (e != cudaSuccess) return e;
+        if (occ < 1) return cudaErrorInvalidConfiguration;
+        if (dev == 0) known[cap / 32].store(occ, std::memory_order_relaxed);
+    }
     int grid = num_sms * occ;
     const int need = (te - tb + kTileWarps - 1) / kTileWarps;
     if (grid > need) grid = need;

@@ -123,21 +123,22 @@ lib = _load()
 
 
 def _ptr(a):
+    """Address of a tensor, an array or an int (ctypes takes ints for pointers)."""
     if a is None:
         return None
     if hasattr(a, "data_ptr"):
-        return ctypes.c_void_p(a.data_ptr())
+        return a.data_ptr()
     if isinstance(a, np.ndarray):
-        return a.ctypes.data_as(ctypes.c_void_p)
-    return ctypes.c_void_p(int(a))
+        return a.ctypes.data
+    return int(a)
 
 
 def _stream(s):
     if s is None:
         return None
     if hasattr(s, "cuda_stream"):
-        return ctypes.c_void_p(s.cuda_stream)
-    return ctypes.c_void_p(int(s))
+        return s.cuda_stream
+    return int(s)
 
 
 def spmv_last_error():
@@ -225,9 +226,11 @@ def spmv_schedule_run(h, op_order, stream_of_op, streams, x_dev, y_dev,
     """Run, capture or replay one implementation; returns the graph handle."""
     order = np.ascontiguousarray(op_order, dtype=np.int32)
     smap = np.ascontiguousarray(stream_of_op, dtype=np.int32)
-    sarr = (ctypes.c_void_p * len(streams))(*[_stream(s).value for s in streams])
+    sarr = (ctypes.c_void_p * len(streams))(*[_stream(s) for s in streams])
     g = ctypes.c_int64(int(graph_handle))
-    _check(lib.spmv_schedule_run(h, _ptr(order), _ptr(smap), len(order), sarr,
+    # a replay reads neither the order nor the stream map
+    replay = (int(flags) & ~(RUN_RELAXED | RUN_DEFER)) == RUN_REPLAY
+    _check(lib.spmv_schedule_run(h, None if replay else _ptr(order), None if replay else _ptr(smap), len(order), sarr,
                                  len(streams), _ptr(x_dev), _ptr(y_dev), int(flags),
                                  ctypes.byref(g)))
     return g.value
