@@ -202,7 +202,11 @@ __device__ __forceinline__ void long_round(const CsrArgs& a, const double* xb, i
 // YP: the layout has a y row per position (sa.ypos; sorted remote layouts).
 // GRP: the units after the long rows are the sorted layout's groups
 // (sell_group) instead of its slices; a group of one slice is that slice.
-template <int U, int MINB, typename CT, bool YP = false, bool GRP = false>
+// LNG: the launch has long rows; without them their code (rounds of 8 entries)
+// does not hold registers that the slices' rounds need (at 48 and 40 registers a
+// thread they spilled 44 and 68 bytes; 27-point 150^3 with 16-bit deltas, param
+// 107: 159.6 us per step against 161.5 us, bound by FP64 at 143 us and HBM at 138).
+template <int U, int MINB, typename CT, bool YP = false, bool GRP = false, bool LNG = true>
 __global__ void __launch_bounds__(256, MINB) csr_sell_kernel(CsrArgs a, SellArgs sa) {
     // the previous kernel of this stream is done (unless independent, or
     // the wait is deferred to the first access to y)
@@ -213,7 +217,7 @@ __global__ void __launch_bounds__(256, MINB) csr_sell_kernel(CsrArgs a, SellArgs
     const uint64_t pol_keep = sell_policy_evict_last();
     const int lane = threadIdx.x & 31;
     const int nwarps = (int)gridDim.x * 8;
-    const int n_long = sa.long_end - sa.long_begin;
+    const int n_long = LNG ? sa.long_end - sa.long_begin : 0;
     const int n_units = n_long + (sa.slice_end - sa.slice_begin);
     int u0 = (int)blockIdx.x * 8 + (int)(threadIdx.x >> 5), u_end = n_units, stride = nwarps;
     if (sa.cta_off) {
@@ -222,7 +226,7 @@ __global__ void __launch_bounds__(256, MINB) csr_sell_kernel(CsrArgs a, SellArgs
         stride = 8;
     }
     for (; u0 < u_end; u0 += stride) {
-        if (u0 < n_long) {
+        if (LNG && u0 < n_long) {
             const SellLong L = sa.longs[sa.long_begin + u0];
             const int kb = L.k0, ke = L.k1;
             const double* xb = a.x + L.xoff;
@@ -534,11 +538,16 @@ cudaError_t launch_sell(const CsrArgs& a, const SellArgs& sa, int param, bool de
     const int grid = sell_grid(param, units, num_sms);
     if (grid <= 0) return cudaErrorInvalidValue;
     if (sell_param_balanced(param) != (sa.cta_off != nullptr)) return cudaErrorInvalidValue;
+    const bool lng = sa.long_end > sa.long_begin;
 #define SELL_LAUNCH(u, b)                                                                        \
     e = sa.groups && sa.ypos                                                                             \
             ? launch_pdl(csr_sell_kernel<u, b, int32_t, true, (u >= 8)>, dim3(grid), dim3(256), 0, st, a, sa) \
         : sa.groups                                                                                            \
             ? launch_pdl(csr_sell_kernel<u, b, int32_t, false, (u >= 8)>, dim3(grid), dim3(256), 0, st, a, sa) \
+        : delta16 && !lng                                                                                      \
+            ? launch_pdl(csr_sell_kernel<u, b, int16_t, false, false, (u < 8)>, dim3(grid), dim3(256), 0, st, a, sa) \
+        : !sa.ypos && !lng                                                                                     \
+            ? launch_pdl(csr_sell_kernel<u, b, int32_t, false, false, (u < 8)>, dim3(grid), dim3(256), 0, st, a, sa) \
         : delta16 ? launch_pdl(csr_sell_kernel<u, b, int16_t>, dim3(grid), dim3(256), 0, st, a, sa)      \
         : sa.ypos ? launch_pdl(csr_sell_kernel<u, b, int32_t, true>, dim3(grid), dim3(256), 0, st, a, sa) \
                   : launch_pdl(csr_sell_kernel<u, b, int32_t>, dim3(grid), dim3(256), 0, st, a, sa)
