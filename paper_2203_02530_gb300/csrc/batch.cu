@@ -1117,6 +1117,7 @@ void batch_host_setup(spmv_batch* b) {
         b->io_x = static_cast<double*>(balloc(b, (size_t)b->total_rows * sizeof(double)));
         b->io_y = static_cast<double*>(balloc(b, (size_t)b->total_rows * sizeof(double)));
         b->io_tickets = static_cast<int*>(balloc(b, 4 * 64 * sizeof(int)));
+        spmvk::check_cuda(cudaDeviceSynchronize(), "synchronize");   // zero-filled before other streams write
     }
     while ((int)b->io_ev.size() < 2 * 64 + 4) {
         cudaEvent_t e;
@@ -1441,6 +1442,7 @@ int spmv_batch_run_host_many(spmv_batch* b, int64_t count, const double* x_host,
     if (!b->io_x2) {
         b->io_x2 = static_cast<double*>(balloc(b, (size_t)b->total_rows * sizeof(double)));
         b->io_y2 = static_cast<double*>(balloc(b, (size_t)b->total_rows * sizeof(double)));
+        spmvk::check_cuda(cudaDeviceSynchronize(), "synchronize");   // zero-filled before other streams write
     }
     for (int64_t k = 0; k < count; ++k) {
         const int slot = (int)(k & 1);
