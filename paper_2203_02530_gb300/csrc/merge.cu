@@ -15,11 +15,11 @@
 // What bounds it: the scattered x gathers (38 us for 10.8 M at the rate of
 // random reads) and the FP64 pipe (about 14 FP64 instructions per 8 entries of
 // a lane, 0.51 of the pipe).  Power-law matrix of 700 001 rows, 10.8 M entries:
-// 70 us; the form before, tiles of 2048 items staged in shared memory per CTA
+// 68 us (70 us with 16-byte loads); the form before, tiles of 2048 items staged in shared memory per CTA
 // and walked item by item (48 M warp instructions against 19 M, 24 warps per SM,
 // a path search of 22 dependent shared-memory reads a thread, and a launch of
 // its own that computed the tiles), took 154 us.  7-point stencil of 12 696
-// rows: 6.5 us against 14.2 us.
+// rows: 6.2 us against 14.3 us.
 #include "internal.h"
 #include "pdl.cuh"
 
@@ -105,7 +105,9 @@ __device__ __forceinline__ void put(const CsrArgs& a, int row, double v) {
 // PLAN: ranges come from the plan's table, whose arrays are padded past their
 // ends.  Else the warp finds its range of `items` merge items by itself, and
 // the arrays are the caller's: the vector loads stop at the last entry.
-template <bool PLAN>
+// A32: values and columns start at multiples of 32 bytes (a plan's do), so a
+// lane's entries are three 32-byte loads instead of six of 16 bytes.
+template <bool PLAN, bool A32>
 __global__ void __launch_bounds__(MERGE_NT, 4) merge_kernel(CsrArgs a, const MergeTile* __restrict__ tiles,
                                                             int tile_begin, int tile_end, int items,
                                                             Carry* __restrict__ carries) {
@@ -154,15 +156,27 @@ __global__ void __launch_bounds__(MERGE_NT, 4) merge_kernel(CsrArgs a, const Mer
             double v[MERGE_LANE];
             int32_t col[MERGE_LANE];
             if (e < k1 && (PLAN || e + MERGE_LANE <= a.nnz_total)) {
-                const int4 c0 = __ldg(reinterpret_cast<const int4*>(a.col + e));
-                const int4 c1 = __ldg(reinterpret_cast<const int4*>(a.col + e + 4));
-                col[0] = c0.x; col[1] = c0.y; col[2] = c0.z; col[3] = c0.w;
-                col[4] = c1.x; col[5] = c1.y; col[6] = c1.z; col[7] = c1.w;
+                if (A32) {
+                    asm("ld.global.nc.v8.s32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                        : "=r"(col[0]), "=r"(col[1]), "=r"(col[2]), "=r"(col[3]), "=r"(col[4]), "=r"(col[5]),
+                          "=r"(col[6]), "=r"(col[7])
+                        : "l"(a.col + e));
 #pragma unroll
-                for (int u = 0; u < MERGE_LANE; u += 2) {
-                    const double2 p = __ldg(reinterpret_cast<const double2*>(a.val + e + u));
-                    v[u] = p.x;
-                    v[u + 1] = p.y;
+                    for (int u = 0; u < MERGE_LANE; u += 4)
+                        asm("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];"
+                            : "=d"(v[u]), "=d"(v[u + 1]), "=d"(v[u + 2]), "=d"(v[u + 3])
+                            : "l"(a.val + e + u));
+                } else {
+                    const int4 c0 = __ldg(reinterpret_cast<const int4*>(a.col + e));
+                    const int4 c1 = __ldg(reinterpret_cast<const int4*>(a.col + e + 4));
+                    col[0] = c0.x; col[1] = c0.y; col[2] = c0.z; col[3] = c0.w;
+                    col[4] = c1.x; col[5] = c1.y; col[6] = c1.z; col[7] = c1.w;
+#pragma unroll
+                    for (int u = 0; u < MERGE_LANE; u += 2) {
+                        const double2 p = __ldg(reinterpret_cast<const double2*>(a.val + e + u));
+                        v[u] = p.x;
+                        v[u + 1] = p.y;
+                    }
                 }
             } else {
 #pragma unroll
@@ -318,8 +332,9 @@ static cudaError_t run_merge(const CsrArgs& a, const MergeTile* tiles, int tile_
     const int n = tile_end - tile_begin;
     int grid = num_sms * 4;   // __launch_bounds__
     if (grid > (n + MERGE_WARPS - 1) / MERGE_WARPS) grid = (n + MERGE_WARPS - 1) / MERGE_WARPS;
-    cudaError_t e = launch_pdl(merge_kernel<PLAN>, dim3(grid), dim3(MERGE_NT), 0, s, a, tiles, tile_begin, tile_end,
-                               items, carries);
+    const bool a32 = PLAN || ((reinterpret_cast<uintptr_t>(a.col) | reinterpret_cast<uintptr_t>(a.val)) & 31) == 0;
+    cudaError_t e = launch_pdl(a32 ? merge_kernel<PLAN, true> : merge_kernel<PLAN, PLAN>, dim3(grid), dim3(MERGE_NT), 0, s,
+                               a, tiles, tile_begin, tile_end, items, carries);
     if (e != cudaSuccess) return e;
     return launch_pdl(merge_fixup_kernel, dim3((n + 255) / 256), dim3(256), 0, s, a, carries, tile_begin, tile_end);
 }
