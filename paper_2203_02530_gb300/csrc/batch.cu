@@ -1257,34 +1257,32 @@ int spmv_batch_create(int count, const int64_t* n, const int64_t* const* row_ptr
     std::vector<BatchPiece> pieces;
     size_t slots = 0, cut_rows = 0;
     for (int m = 0; m < count; ++m) {
-        for (int64_t i = 0; i < n[m]; ++i) {
-            const int64_t len = row_ptr[m][i + 1] - row_ptr[m][i];
-            if (len <= b->piece_len) continue;
-            const int np = (int)((len + b->piece_len - 1) / b->piece_len);
-            for (int p = 0; p < np; ++p)
-                b->pieces[m].push_back(BatchPiece{(int)i, p, np, (int)slots, (int)cut_rows});
-            slots += np;
-            ++cut_rows;
-        }
-        pieces.insert(pieces.end(), b->pieces[m].begin(), b->pieces[m].end());
-    }
-    for (int m = 0; m < count; ++m) {
         const BatchMat& M = b->mats[m];
         const int64_t base = n[m] > 0 ? row_ptr[m][0] : 0;
-        for (int64_t i = 0; i <= n[m]; ++i)
-            hptr[(size_t)(M.ptr_off + i)] = n[m] > 0 ? (int32_t)(row_ptr[m][i] - base) : 0;
         for (int64_t k = 0; k < b->nnz[m]; ++k) {
             hcol[(size_t)(M.ent_off + k)] = col_idx[m][base + k];
             hval[(size_t)(M.ent_off + k)] = vals[m][base + k];
         }
         for (int64_t r = 0; r < n[m]; r += kItemRows) {
             const int64_t e = std::min<int64_t>(n[m], r + kItemRows);
-            b->csr_items[m].push_back(BatchItem{m, 0, (int)r, (int)e});
             int64_t whole = 0;   // entries of the rows that are not cut
-            for (int64_t i = r; i < e; ++i)
-                if (row_ptr[m][i + 1] - row_ptr[m][i] <= b->piece_len) whole += row_ptr[m][i + 1] - row_ptr[m][i];
+            for (int64_t i = r; i < e; ++i) {
+                const int64_t len = row_ptr[m][i + 1] - row_ptr[m][i];
+                hptr[(size_t)(M.ptr_off + i + 1)] = (int32_t)(row_ptr[m][i + 1] - base);
+                if (len <= b->piece_len) {
+                    whole += len;
+                    continue;
+                }
+                const int np = (int)((len + b->piece_len - 1) / b->piece_len);
+                for (int p = 0; p < np; ++p)
+                    b->pieces[m].push_back(BatchPiece{(int)i, p, np, (int)slots, (int)cut_rows});
+                slots += np;
+                ++cut_rows;
+            }
+            b->csr_items[m].push_back(BatchItem{m, 0, (int)r, (int)e});
             b->csr_cost[m].push_back(whole + 8 * (e - r));
         }
+        pieces.insert(pieces.end(), b->pieces[m].begin(), b->pieces[m].end());
     }
     b->ptr = static_cast<int32_t*>(balloc(b, hptr.size() * 4));
     b->col = static_cast<int32_t*>(balloc(b, hcol.size() * 4));
@@ -1292,10 +1290,10 @@ int spmv_batch_create(int count, const int64_t* n, const int64_t* const* row_ptr
     b->d_mats = static_cast<BatchMat*>(balloc(b, b->mats.size() * sizeof(BatchMat)));
     b->ticket = static_cast<int*>(balloc(b, 2 * sizeof(int)));
     b->d_pieces = static_cast<BatchPiece*>(balloc(b, pieces.size() * sizeof(BatchPiece)));
-    for (int set = 0; set < 2; ++set) {
-        b->piece_sum[set] = static_cast<double*>(balloc(b, slots * sizeof(double)));
-        b->piece_cnt[set] = static_cast<int*>(balloc(b, cut_rows * sizeof(int)));   // zeroed
-    }
+    b->piece_sum[0] = static_cast<double*>(balloc(b, 2 * slots * sizeof(double)));
+    b->piece_sum[1] = b->piece_sum[0] + slots;
+    b->piece_cnt[0] = static_cast<int*>(balloc(b, 2 * cut_rows * sizeof(int)));   // zeroed
+    b->piece_cnt[1] = b->piece_cnt[0] + cut_rows;
     if (!pieces.empty())
         spmvk::check_cuda(cudaMemcpy(b->d_pieces, pieces.data(), pieces.size() * sizeof(BatchPiece),
                                      cudaMemcpyHostToDevice), "pieces");
