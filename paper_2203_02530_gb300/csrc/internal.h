@@ -128,9 +128,9 @@ cudaError_t launch_pairs(const CsrArgs& a, const Tile* tiles, int tile_begin, in
                          int lanes, int num_sms, cudaStream_t s);
 cudaError_t launch_merge(const CsrArgs& a, const MergeTile* tiles, int tile_begin,
                          int tile_end, Carry* carries, int num_sms, cudaStream_t s);
-cudaError_t launch_merge_partition(const int32_t* ptr, int row_begin, int row_end, int32_t xoff,
+cudaError_t launch_merge_partition(const int32_t* ptr, int row_begin, int row_end, int32_t xoff, int per,
                                    MergeTile* tiles, int n_tiles, cudaStream_t s);
-int merge_items_per_tile();   // of a plan's ranges
+int merge_plan_items(int64_t items);   // merge items per range of a plan's product of `items` in all
 // Plan-free merge product: its ranges (one carry each) and its launch.
 int64_t merge_free_ranges(int64_t items);
 cudaError_t launch_merge_free(const CsrArgs& a, Carry* carries, int num_sms, cudaStream_t s);

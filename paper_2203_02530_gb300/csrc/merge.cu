@@ -4,7 +4,7 @@
 // rows + entries items (Merrill and Garland's merge-based CSR), and every
 // warp takes a range of the path, so all do the same work however long the
 // rows are.  A warp walks its entries 256 at a time, eight consecutive ones a
-// lane: 16-byte loads, eight x gathers in flight, eight FMAs.  Rows that end
+// lane: 32-byte loads, eight x gathers in flight, eight FMAs.  Rows that end
 // within a lane's entries are told by byte flags in shared memory, which the
 // lanes that hold the row ends set; a row cut between lanes is finished by a
 // segmented scan over the lanes, one cut between chunks by the warp's running
@@ -15,11 +15,11 @@
 // What bounds it: the scattered x gathers (38 us for 10.8 M at the rate of
 // random reads) and the FP64 pipe (about 14 FP64 instructions per 8 entries of
 // a lane, 0.51 of the pipe).  Power-law matrix of 700 001 rows, 10.8 M entries:
-// 68 us (70 us with 16-byte loads); the form before, tiles of 2048 items staged in shared memory per CTA
-// and walked item by item (48 M warp instructions against 19 M, 24 warps per SM,
-// a path search of 22 dependent shared-memory reads a thread, and a launch of
-// its own that computed the tiles), took 154 us.  7-point stencil of 12 696
-// rows: 6.2 us against 14.3 us.
+// 68 us (70 us with 16-byte loads); the form before, tiles of 2048 items staged
+// in shared memory per CTA and walked item by item (48 M warp instructions
+// against 19 M, 24 warps per SM, a path search of 22 dependent shared-memory
+// reads a thread, and a launch of its own that computed the tiles), took 154 us.
+// 7-point stencil of 12 696 rows: 6.2 us against 14.3 us.
 #include "internal.h"
 #include "pdl.cuh"
 
@@ -42,10 +42,15 @@ constexpr int kErrTimeout = 6;
 
 // Items per range.  A chunk starts at a multiple of MERGE_LANE entries, so a
 // range of MERGE_CHUNK m - MERGE_LANE items never needs more than m chunks.
-// Plans use a fixed length (two chunks); plan-free products the length that
-// gives 4864 ranges (152 SMs x 32 warps: one wave of equal ranges), at least
-// one chunk.  It depends on the matrix alone, so results do too.
-constexpr int MERGE_PLAN_ITEMS = 2 * MERGE_CHUNK - MERGE_LANE;
+// Plans use one chunk while that makes at most two ranges for every warp in
+// flight, else two; plan-free products the length that gives 4864 ranges
+// (152 SMs x 32 warps: one wave of equal ranges), at least one chunk.  It
+// depends on the matrix alone, so results do too.
+// One chunk against two, replayed schedules of per-rank / whole launches (us):
+// band matrix of 22 760 rows 20.8 / 10.8 against 26.6 / 13.3, of 200 000 rows
+// (2.2 M items) 30.6 / 22.4 against 33.5 / 21.9, 7-point stencil on 60^3 24.4 /
+// 15.1 against 27.4 / 15.4; above the line power-law 1 M rows 156 / 111 against
+// 143 / 110, 27-point on 91^3 101 / 85.6 against 99.7 / 83.4.
 constexpr int MERGE_RANGES = 4864;
 
 int64_t range_items(int64_t items) {
@@ -298,7 +303,7 @@ __global__ void __launch_bounds__(256) merge_fixup_kernel(CsrArgs a, const Carry
 // Merge-path coordinates of every range boundary of a plan, computed on the
 // device from a CSR row pointer: range t covers diagonals [t*ITEMS, (t+1)*ITEMS).
 __global__ void merge_partition_kernel(const int32_t* __restrict__ ptr, int row_begin, int row_end,
-                                       int32_t xoff, MergeTile* __restrict__ tiles, int n_tiles) {
+                                       int32_t xoff, int per, MergeTile* __restrict__ tiles, int n_tiles) {
     const int t = (int)(blockIdx.x * blockDim.x + threadIdx.x);
     if (t >= n_tiles) return;
     const int k_base = __ldg(ptr + row_begin);
@@ -306,8 +311,8 @@ __global__ void merge_partition_kernel(const int32_t* __restrict__ ptr, int row_
     const int b_len = __ldg(ptr + row_end) - k_base;
     const int items = a_len + b_len;
     auto A = [&](int i) { return __ldg(ptr + row_begin + i + 1) - k_base; };
-    const int d0 = t * MERGE_PLAN_ITEMS;
-    const int d1 = d0 + MERGE_PLAN_ITEMS < items ? d0 + MERGE_PLAN_ITEMS : items;
+    const int d0 = t * per;
+    const int d1 = d0 + per < items ? d0 + per : items;
     const int i0 = path_search(d0, a_len, b_len, A);
     const int i1 = path_search(d1, a_len, b_len, A);
     MergeTile m{};
@@ -321,7 +326,9 @@ __global__ void merge_partition_kernel(const int32_t* __restrict__ ptr, int row_
 
 }  // namespace
 
-int merge_items_per_tile() { return MERGE_PLAN_ITEMS; }
+int merge_plan_items(int64_t items) {
+    return MERGE_CHUNK * (items <= 2 * (int64_t)MERGE_RANGES * MERGE_CHUNK ? 1 : 2) - MERGE_LANE;
+}
 
 // `items` (plan-free): merge items per range; else ranges [tile_begin, tile_end)
 // of the plan's table.
@@ -352,10 +359,10 @@ cudaError_t launch_merge_free(const CsrArgs& a, Carry* carries, int num_sms, cud
                             s);
 }
 
-cudaError_t launch_merge_partition(const int32_t* ptr, int row_begin, int row_end, int32_t xoff,
+cudaError_t launch_merge_partition(const int32_t* ptr, int row_begin, int row_end, int32_t xoff, int per,
                                    MergeTile* tiles, int n_tiles, cudaStream_t s) {
     if (n_tiles <= 0) return cudaSuccess;
-    merge_partition_kernel<<<(n_tiles + 127) / 128, 128, 0, s>>>(ptr, row_begin, row_end, xoff, tiles,
+    merge_partition_kernel<<<(n_tiles + 127) / 128, 128, 0, s>>>(ptr, row_begin, row_end, xoff, per, tiles,
                                                                  n_tiles);
     return cudaGetLastError();
 }

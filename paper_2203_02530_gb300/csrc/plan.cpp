@@ -322,7 +322,7 @@ void build_tiles(spmv_part* pt) {
 // pointers the kernels use.
 void build_merge_tiles(spmv_part* pt) {
     const int P = pt->P;
-    const int items = merge_items_per_tile();
+    const int items_l = merge_plan_items(pt->n + pt->nnz_l), items_r = merge_plan_items(pt->n_rr + pt->nnz_r);
     std::vector<int32_t> l_ptr_b(P + 1), rr_ptr_b(P + 1);
     for (int p = 0; p <= P; ++p) {
         check_cuda(cudaMemcpy(&l_ptr_b[p], pt->l_ptr + pt->bounds[p], 4, cudaMemcpyDeviceToHost), "merge plan");
@@ -333,8 +333,8 @@ void build_merge_tiles(spmv_part* pt) {
     for (int p = 0; p < P; ++p) {
         const int64_t li = (pt->bounds[p + 1] - pt->bounds[p]) + (int64_t)(l_ptr_b[p + 1] - l_ptr_b[p]);
         const int64_t ri = (pt->rr_off[p + 1] - pt->rr_off[p]) + (int64_t)(rr_ptr_b[p + 1] - rr_ptr_b[p]);
-        pt->lmtile_off[p + 1] = pt->lmtile_off[p] + (li + items - 1) / items;
-        pt->rmtile_off[p + 1] = pt->rmtile_off[p] + (ri + items - 1) / items;
+        pt->lmtile_off[p + 1] = pt->lmtile_off[p] + (li + items_l - 1) / items_l;
+        pt->rmtile_off[p + 1] = pt->rmtile_off[p] + (ri + items_r - 1) / items_r;
     }
     free_one(pt, pt->lmtiles);
     free_one(pt, pt->rmtiles);
@@ -346,10 +346,10 @@ void build_merge_tiles(spmv_part* pt) {
     pt->rcarry = static_cast<Carry*>(dev_alloc(pt, (size_t)pt->rmtile_off[P] * sizeof(Carry)));
     for (int p = 0; p < P; ++p) {
         check_cuda(launch_merge_partition(pt->l_ptr, (int)pt->bounds[p], (int)pt->bounds[p + 1],
-                                          (int32_t)pt->bounds[p], pt->lmtiles + pt->lmtile_off[p],
+                                          (int32_t)pt->bounds[p], items_l, pt->lmtiles + pt->lmtile_off[p],
                                           (int)(pt->lmtile_off[p + 1] - pt->lmtile_off[p]), 0),
                    "merge partition");
-        check_cuda(launch_merge_partition(pt->rr_ptr, (int)pt->rr_off[p], (int)pt->rr_off[p + 1], 0,
+        check_cuda(launch_merge_partition(pt->rr_ptr, (int)pt->rr_off[p], (int)pt->rr_off[p + 1], 0, items_r,
                                           pt->rmtiles + pt->rmtile_off[p],
                                           (int)(pt->rmtile_off[p + 1] - pt->rmtile_off[p]), 0),
                    "merge partition");

@@ -58,3 +58,31 @@ def test_merge_ranges_exact(name):
             part.run(order, [0] * 12, [s], args[3], y)
             s.synchronize()
             assert np.array_equal(y.cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("n", [115_000, 135_000])
+def test_plan_range_lengths(n):
+    """A plan's ranges are one chunk up to 2 x 4864 x 256 items, else two: a
+    local product on each side of the line, a small remote one."""
+    from paper_2203_02530_gb300 import spmv
+    torch = torch_cuda()
+    rng = np.random.default_rng(n)
+    lens = rng.integers(0, 41, size=n)
+    rp = np.zeros(n + 1, dtype=np.int64)
+    np.cumsum(lens, out=rp[1:])
+    assert (n + rp[-1] > 2 * 4864 * 256) == (n == 135_000)
+    rows = np.repeat(np.arange(n), lens)
+    ci = np.clip(rows + rng.integers(-300, 301, size=rp[-1]), 0, n - 1).astype(np.int32)
+    va = rng.integers(-4, 5, size=rp[-1]).astype(np.float64)
+    x = rng.integers(-4, 5, size=n).astype(np.float64)
+    want = oracle.csr_spmv(n, rp, ci, va, x)
+    s, x_d = torch.cuda.Stream(), dev(x)
+    for gran in (spmv.COARSE, spmv.PER_PARTITION):
+        ops = 3 if gran else 1
+        order = [4 * p + k for k in range(4) for p in range(ops)]
+        with spmv.Part(n, rp, ci, va, 3, gran) as part:
+            part.set_variant(spmv.VARIANT_MERGE, 0)
+            y = synced(torch.full((n,), float("nan"), dtype=torch.float64, device="cuda"))
+            part.run(order, [0] * len(order), [s], x_d, y)
+            s.synchronize()
+            assert np.array_equal(y.cpu().numpy(), want), gran
