@@ -129,18 +129,20 @@ spmvk::CsrArgs remote_args(spmv_part* pt, double* y) {
     return a;
 }
 
-// Each op returns the number of kernels it launched.
-int op_pack(spmv_part* pt, int q, const double* x, cudaStream_t s) {
+// Each op returns the number of kernels it launched.  exchange (every
+// rank's pack only): the packed slots go to the receive buffer too, which is
+// the COPY that follows.
+int op_pack(spmv_part* pt, int q, const double* x, cudaStream_t s, bool exchange = false) {
     if (q < 0) {
         if (pt->dry_run) return pt->n_send > 0;
-        check_cuda(spmvk::launch_gather(x, pt->send_idx, nullptr, pt->sendbuf, pt->n_send, pt->num_sms, s,
-                                        pt->cur_pdl),
+        check_cuda(spmvk::launch_gather(x, pt->send_idx, nullptr, pt->sendbuf, exchange ? pt->recvbuf : nullptr,
+                                        pt->n_send, pt->num_sms, s, pt->cur_pdl),
                    "pack");
         return pt->n_send > 0;
     }
     const int64_t c = pt->pack_off[q + 1] - pt->pack_off[q];
     if (pt->dry_run) return c > 0;
-    check_cuda(spmvk::launch_gather(x, pt->send_idx, pt->pack_pos + pt->pack_off[q], pt->sendbuf, c,
+    check_cuda(spmvk::launch_gather(x, pt->send_idx, pt->pack_pos + pt->pack_off[q], pt->sendbuf, nullptr, c,
                                     pt->num_sms, s, pt->cur_pdl),
                "pack");
     return c > 0;
@@ -232,8 +234,8 @@ int op_remote(spmv_part* pt, int p, double* y, cudaStream_t s) {
 // PACK of one halo segment: its send slots [a, b) <- x
 int op_pack_segment(spmv_part* pt, const spmv_part::Seg& g, const double* x, cudaStream_t s) {
     if (pt->dry_run) return g.b > g.a;
-    check_cuda(spmvk::launch_gather(x, pt->send_idx + g.a, nullptr, pt->sendbuf + g.a, g.b - g.a, pt->num_sms, s,
-                                    pt->cur_pdl),
+    check_cuda(spmvk::launch_gather(x, pt->send_idx + g.a, nullptr, pt->sendbuf + g.a, nullptr, g.b - g.a,
+                                    pt->num_sms, s, pt->cur_pdl),
                "pack segment");
     return g.b > g.a;
 }
@@ -1094,10 +1096,10 @@ int64_t host_product(spmv_part* pt, const double* x_host, double* y_host, double
 }
 
 // The same product for the stream of small ones: x in one copy, one launch per
-// operation over all ranks, one after another on compute_stream (which then
-// also orders the send and receive buffers' uses), y in one copy.  14 calls
-// where the form above makes 23 + 10 P, with no event between the operations.
-// Same kernels on the same rows.
+// operation over all ranks (pack and exchange in one), one after another on
+// compute_stream (which then also orders the send and receive buffers' uses), y
+// in one copy.  13 calls where the form above makes 23 + 10 P, with no event
+// between the operations.  Same sums in the same order.
 int64_t host_product_coarse(spmv_part* pt, const double* x_host, double* y_host, double* xd, double* yd,
                             cudaStream_t copy_stream, cudaStream_t compute_stream, int slot) {
     const int P = pt->P;
@@ -1113,9 +1115,8 @@ int64_t host_product_coarse(spmv_part* pt, const double* x_host, double* y_host,
     wait(compute_stream, x_here);
     wait(compute_stream, y_free);
     int64_t launches = op_local(pt, -1, xd, yd, compute_stream);
-    launches += op_pack(pt, -1, xd, compute_stream);
+    launches += op_pack(pt, -1, xd, compute_stream, true);
     record(x_free, compute_stream);
-    launches += op_copy(pt, -1, compute_stream);
     launches += op_remote(pt, -1, yd, compute_stream);
     record(done, compute_stream);
     wait(out_stream, done);
@@ -1130,7 +1131,8 @@ int64_t host_product_coarse(spmv_part* pt, const double* x_host, double* y_host,
 // compute, which only a short stream of large products feels.  27-point, us per
 // call, rank by rank and here: 20^3 4 ranks 4 products 169 and 78, 64^3 1 product
 // 81 and 78, 80^3 4 products 282 and 229, 90^3 1 product 125 and 138, 130^3 4
-// products 733 and 714, 16 products 2818 and 2374.
+// products 733 and 714, 16 products 2818 and 2374.  (Pack and exchange in one
+// launch, measured later, takes 2 to 5 % more off the streams here.)
 bool host_coarse(const spmv_part* pt, int64_t count) {
     const int64_t per_rank = count == 1 ? 65536 : count == 2 ? 131072 : 600000;
     return pt->n <= per_rank * pt->P;

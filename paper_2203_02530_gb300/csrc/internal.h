@@ -109,8 +109,9 @@ struct CsrArgs {
 };
 
 // Launchers (kernels.cu).  All return cudaGetLastError() after the launch.
-cudaError_t launch_gather(const double* x, const int32_t* idx, const int32_t* pos,
-                          double* dst, int64_t count, int num_sms, cudaStream_t s, int pdl = 0);
+// launch_gather: `also` (may be null): a second array that gets the same slots.
+cudaError_t launch_gather(const double* x, const int32_t* idx, const int32_t* pos, double* dst, double* also,
+                          int64_t count, int num_sms, cudaStream_t s, int pdl = 0);
 cudaError_t launch_copy(const double* src, double* dst, int64_t count, int num_sms,
                         cudaStream_t s, int pdl = 0);
 cudaError_t launch_tile(const CsrArgs& a, const Tile* tiles, int tile_begin, int tile_end, bool one_sum, int param,
