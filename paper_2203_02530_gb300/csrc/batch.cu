@@ -18,6 +18,7 @@
 // by HBM and the x gathers (48 matrices of up to 1 M rows, sliced: 205 us
 // against 217 us; two lanes a row 361 against 386 us).
 #include "batch.h"
+#include "pieces.h"
 
 #include <cuda_runtime.h>
 
@@ -35,6 +36,8 @@ constexpr int kThreads = 256;
 using spmvk::BatchItem;
 using spmvk::BatchPiece;
 using spmvk::BSlice;
+using spmvk::piece_count;
+using spmvk::piece_size;
 
 constexpr int kSliced = 64;   // lanes value selecting the sliced layout
 
@@ -79,20 +82,21 @@ __device__ __forceinline__ int32_t ld_stream(const int32_t* p) {
 
 constexpr int kLongRow = 64;   // rows longer than this are summed by a whole warp
 
-// One row summed by the 32 lanes of a warp: lane l takes entries l, l+32,
+// The n entries from col / val on (a row or a piece of one), summed by the 32
+// lanes of a warp: lane l takes entries l, l+32,
 // ... in order (D of them in flight), then a fixed xor-butterfly; every lane
 // returns the total, the same for every D.  D = 4 leaves registers for many
 // warps, which hide each other's latency; D = 16 also loads the columns one
 // round ahead, for launches with so few warps that a long row's chain of
 // load-then-gather rounds is what the launch waits for.
 template <int D>
-__device__ __forceinline__ double warp_row(const int32_t* col, const double* val, const double* x, int kb, int ke,
+__device__ __forceinline__ double warp_row(const int32_t* col, const double* val, const double* x, int n,
                                            uint64_t pol) {
     const int lane = threadIdx.x & 31;
     double part = 0.0;
-    int k = kb + lane;
+    int k = lane;
     if (D <= 4) {
-        for (; k + 32 * (D - 1) < ke; k += 32 * D) {
+        for (; k + 32 * (D - 1) < n; k += 32 * D) {
             double v[D], xv[D];
 #pragma unroll
             for (int u = 0; u < D; ++u) {
@@ -102,26 +106,26 @@ __device__ __forceinline__ double warp_row(const int32_t* col, const double* val
 #pragma unroll
             for (int u = 0; u < D; ++u) part = fma(v[u], xv[u], part);
         }
-        for (; k < ke; k += 32) part = fma(__ldg(val + k), ldg_keep(x + __ldg(col + k), pol), part);
+        for (; k < n; k += 32) part = fma(__ldg(val + k), ldg_keep(x + __ldg(col + k), pol), part);
     } else {
         int32_t c[D];
 #pragma unroll
-        for (int u = 0; u < D; ++u) c[u] = k + 32 * u < ke ? __ldg(col + k + 32 * u) : 0;
-        for (int base = kb; base < ke; base += 32 * D, k += 32 * D) {
+        for (int u = 0; u < D; ++u) c[u] = k + 32 * u < n ? __ldg(col + k + 32 * u) : 0;
+        for (int base = 0; base < n; base += 32 * D, k += 32 * D) {
             double v[D], xv[D];
 #pragma unroll
             for (int u = 0; u < D; ++u) {
-                const bool m = k + 32 * u < ke;
+                const bool m = k + 32 * u < n;
                 v[u] = m ? __ldg(val + k + 32 * u) : 0.0;
                 xv[u] = m ? ldg_keep(x + c[u], pol) : 0.0;
             }
 #pragma unroll
-            for (int u = 0; u < D; ++u) c[u] = k + 32 * (D + u) < ke ? __ldg(col + k + 32 * (D + u)) : 0;
+            for (int u = 0; u < D; ++u) c[u] = k + 32 * (D + u) < n ? __ldg(col + k + 32 * (D + u)) : 0;
 #pragma unroll
             for (int u = 0; u < D; ++u) {
-                if (base + 32 * u >= ke) break;   // warp-uniform
+                if (base + 32 * u >= n) break;   // warp-uniform
                 const double t = fma(v[u], xv[u], part);
-                part = k + 32 * u < ke ? t : part;
+                part = k + 32 * u < n ? t : part;
             }
         }
     }
@@ -148,14 +152,16 @@ template <int D, bool INLINE>
 __device__ __forceinline__ void long_row(const int32_t* col, const double* val, const double* x, double* y, int row,
                                          int kb, int ke, int piece_len, uint64_t pol) {
     const int lane = threadIdx.x & 31;
+    col += kb;
+    val += kb;
     if (ke - kb <= piece_len) {
-        const double t = warp_row<D>(col, val, x, kb, ke, pol);
+        const double t = warp_row<D>(col, val, x, ke - kb, pol);
         if (lane == 0) y[row] = t;
     } else if (INLINE) {
         double acc = 0.0;
-        int p = 0;
-        for (int k = kb; k < ke; k += piece_len, ++p) {
-            const double t = warp_row<D>(col, val, x, k, k + piece_len < ke ? k + piece_len : ke, pol);
+        const int pieces = piece_count(ke - kb, piece_len);
+        for (int p = 0; p < pieces; ++p, col += piece_len, val += piece_len) {
+            const double t = warp_row<D>(col, val, x, piece_size(ke - kb, piece_len, p), pol);
             if (lane == (p & 31)) acc += t;
         }
         acc = piece_total(acc);
@@ -465,10 +471,9 @@ __device__ __forceinline__ void batch_long(const BatchArgs& a, const BatchMat& m
                                            uint64_t pol) {
     if (!INLINE && piece) {
         const int32_t* ptr = a.ptr + m.ptr_off + a.pieces[p0].row;
-        const int kb = __ldg(ptr) + a.pieces[p0].part * a.piece_len;
-        int ke = __ldg(ptr + 1);
-        if (kb + a.piece_len < ke) ke = kb + a.piece_len;
-        const double t = warp_row<D>(a.col + m.ent_off, a.val + m.ent_off, a.x + m.row_off, kb, ke, pol);
+        const int rb = __ldg(ptr), len = __ldg(ptr + 1) - rb, part = a.pieces[p0].part;
+        const long long at = m.ent_off + rb + part * a.piece_len;
+        const double t = warp_row<D>(a.col + at, a.val + at, a.x + m.row_off, piece_size(len, a.piece_len, part), pol);
         publish_piece(a.pieces + p0, a.piece_sum, a.piece_cnt, a.y + m.row_off, t);
         return;
     }
@@ -1273,7 +1278,7 @@ int spmv_batch_create(int count, const int64_t* n, const int64_t* const* row_ptr
                     whole += len;
                     continue;
                 }
-                const int np = (int)((len + b->piece_len - 1) / b->piece_len);
+                const int np = piece_count((int)len, b->piece_len);
                 for (int p = 0; p < np; ++p)
                     b->pieces[m].push_back(BatchPiece{(int)i, p, np, (int)slots, (int)cut_rows});
                 slots += np;
