@@ -449,7 +449,7 @@ int spmv_csr_error(int64_t* out);
  * 2048 entries (by the batch's size) in pieces of that length whose sums are
  * added, in a fixed order, so y is the same, bit for
  * bit, as with spmv_batch_run_separate, which launches the same row code
- * once per matrix.  Not part of the paper's method: a way of running many
+ * once per matrix (and a second time for the rows cut into pieces).  Not part of the paper's method: a way of running many
  * of its SpMVs at once.  One spmv_batch_run of a batch may be in flight at a
  * time.
  * spmv_batch_create: `count` matrices given as HOST CSR arrays (n[m],

@@ -93,6 +93,8 @@ struct spmv_batch {
     spmvk::BatchPiece* d_pieces = nullptr;
     double* piece_sum[2] = {nullptr, nullptr};
     int* piece_cnt[2] = {nullptr, nullptr};
+    int* d_cut_rows = nullptr;           // the rows that are cut, matrix by matrix
+    std::vector<int> cut_off;            // count+1
     size_t device_bytes = 0;
     std::vector<void*> allocs;
     // CSR released (spmv_batch_release_csr): ptr/col/val then hold only the
