@@ -54,8 +54,8 @@ struct BatchArgs {
     int piece_len;            // a row longer than this is cut into pieces
     const BatchPiece* pieces;
     double* piece_sum;
-    int* piece_cnt;
-    int* ticket;
+    unsigned* piece_cnt;
+    unsigned* ticket;
 };
 
 __device__ __forceinline__ uint64_t policy_evict_last() {
@@ -157,10 +157,12 @@ __device__ __forceinline__ void long_row(const int32_t* col, const double* val, 
 }
 
 // Sum t of a piece into its slot; the warp that completes the row adds the
-// row's slots, lane l taking slots l, l+32, ... in order, and sets the counter
-// back to zero.  Not inlined: its few live values would otherwise push the
-// sliced persistent kernel out of its 40 registers.
-__device__ __noinline__ void publish_piece(const BatchPiece* piece, double* piece_sum, int* piece_cnt, double* y,
+// row's slots, lane l taking slots l, l+32, ... in order.  The counter wraps to
+// zero by itself with the row's last piece; launches take every piece once, so
+// that it is right again after any of them, also after ones that overlapped
+// (whose own results are not).  Not inlined: its few live values would otherwise
+// push the sliced persistent kernel out of its 40 registers.
+__device__ __noinline__ void publish_piece(const BatchPiece* piece, double* piece_sum, unsigned* piece_cnt, double* y,
                                            double t) {
     const BatchPiece& pc = *piece;
     const int lane = threadIdx.x & 31;
@@ -168,17 +170,14 @@ __device__ __noinline__ void publish_piece(const BatchPiece* piece, double* piec
     if (lane == 0) {
         piece_sum[pc.first + pc.part] = t;
         __threadfence();
-        last = atomicAdd(piece_cnt + pc.cidx, 1) == pc.nparts - 1;
+        last = atomicInc(piece_cnt + pc.cidx, (unsigned)pc.nparts - 1) == (unsigned)pc.nparts - 1;
     }
     if (!__shfl_sync(0xffffffffu, last, 0)) return;
     __threadfence();
     double acc = 0.0;
     for (int p = lane; p < pc.nparts; p += 32) acc += __ldcg(piece_sum + pc.first + p);
     acc = piece_total(acc);
-    if (lane == 0) {
-        y[pc.row] = acc;
-        piece_cnt[pc.cidx] = 0;   // ready for the next launch
-    }
+    if (lane == 0) y[pc.row] = acc;
 }
 
 // The long rows flagged in `mask` (bit = the lane holding the row's kb, ke
@@ -574,6 +573,17 @@ __global__ void __launch_bounds__(256) batch_segment_copy_kernel(const int64_t* 
     }
 }
 
+// The next unit of a persistent launch for the calling warp, n_units or more
+// when none is left.  A launch of W warps makes n_units + W claims (each warp
+// leaves with its first that fails), so the ticket wraps there: it is zero again
+// after the launch without a reset before the next one, and launches that
+// overlapped have still taken every unit once each in all.
+__device__ __forceinline__ int claim_unit(const BatchArgs& a) {
+    unsigned t = 0;
+    if ((threadIdx.x & 31) == 0) t = atomicInc(a.ticket, (unsigned)a.n_units + gridDim.x * (kThreads / 32) - 1);
+    return (int)__shfl_sync(0xffffffffu, t, 0);
+}
+
 // Persistent: every warp claims units (units[0 .. n_units)) with an atomic
 // ticket until none is left (no block-wide barrier: warps never wait for each
 // other).  One kernel for the CSR modes (shared-memory slices for the staged
@@ -584,9 +594,7 @@ __global__ void __launch_bounds__(kThreads, 4) batch_persistent_kernel(BatchArgs
     const uint64_t pol = policy_evict_last();
     const int w = threadIdx.x >> 5;
     for (;;) {
-        int t = 0;
-        if ((threadIdx.x & 31) == 0) t = atomicAdd(a.ticket, 1);
-        t = __shfl_sync(0xffffffffu, t, 0);
+        const int t = claim_unit(a);
         if (t >= a.n_units) break;
         const BatchItem u = a.units[t];
         batch_item<4>(a, u, pol, s_val[w], s_col[w]);
@@ -596,9 +604,7 @@ __global__ void __launch_bounds__(kThreads, 4) batch_persistent_kernel(BatchArgs
 __global__ void __launch_bounds__(kThreads, 6) batch_sliced_persistent_kernel(BatchArgs a) {
     const uint64_t pol = policy_evict_last();
     for (;;) {
-        int t = 0;
-        if ((threadIdx.x & 31) == 0) t = atomicAdd(a.ticket, 1);
-        t = __shfl_sync(0xffffffffu, t, 0);
+        const int t = claim_unit(a);
         if (t >= a.n_units) break;
         const BatchItem u = a.units[t];
         batch_item_sliced<4>(a, u, pol);
@@ -606,8 +612,7 @@ __global__ void __launch_bounds__(kThreads, 6) batch_sliced_persistent_kernel(Ba
 }
 
 // Small batches: the units dealt to the warps of one wave in claim order, with
-// no ticket (nothing to reset before the launch, no atomic before the first
-// load) and with 128 registers a thread for the long rows' deep rounds: what
+// no ticket (no atomic before the first load) and with 128 registers a thread for the long rows' deep rounds: what
 // such a launch takes is the chain of dependent loads of its longest unit,
 // not bandwidth.
 __global__ void __launch_bounds__(kThreads, 2) batch_small_kernel(BatchArgs a) {
@@ -1138,10 +1143,10 @@ namespace {
 // 2 events per chunk (x arrived, y computed), then x free and y free for each
 // pair of device vectors of the streamed path.
 void batch_host_setup(spmv_batch* b) {
-    if (!b->io_x) {
+    if (!b->io_tickets) {
         b->io_x = static_cast<double*>(balloc(b, (size_t)b->total_rows * sizeof(double)));
         b->io_y = static_cast<double*>(balloc(b, (size_t)b->total_rows * sizeof(double)));
-        b->io_tickets = static_cast<int*>(balloc(b, 4 * 64 * sizeof(int)));
+        b->io_tickets = static_cast<unsigned*>(balloc(b, 2 * 64 * sizeof(unsigned)));
         spmvk::check_cuda(cudaDeviceSynchronize(), "synchronize");   // zero-filled before other streams write
     }
     while ((int)b->io_ev.size() < 2 * 64 + 4) {
@@ -1156,7 +1161,7 @@ void batch_host_setup(spmv_batch* b) {
 // products on two pairs of device vectors: its copies in wait until the
 // products that read the same pair's previous x are done, and its products
 // until the same pair's previous y has gone out (all products run on
-// s_compute, so the chunk tickets are reset after the previous product).
+// s_compute, so a chunk's ticket is zero again before the next product's).
 void batch_host_product(spmv_batch* b, const double* x_host, double* y_host, double* xd, double* yd, int chunks,
                         cudaStream_t s_in, cudaStream_t s_compute, cudaStream_t s_out, int slot) {
     cudaEvent_t x_free = slot >= 0 ? b->io_ev[2 * 64 + slot] : nullptr;
@@ -1194,8 +1199,6 @@ void batch_host_product(spmv_batch* b, const double* x_host, double* y_host, dou
     // each chunk's units are a contiguous run of the claim order (per
     // layout), run by the persistent kernels with a ticket of their own
     if (y_free) spmvk::check_cuda(cudaStreamWaitEvent(s_compute, y_free, 0), "wait");
-    spmvk::check_cuda(cudaMemsetAsync(b->io_tickets, 0, (size_t)4 * ch.size() * sizeof(int), s_compute),
-                      "chunk tickets");
     const int cp1 = b->count + 1;
     for (size_t c = 0; c < ch.size(); ++c) {
         spmvk::check_cuda(cudaStreamWaitEvent(s_compute, b->io_ev[2 * c], 0), "wait");
@@ -1205,7 +1208,7 @@ void batch_host_product(spmv_batch* b, const double* x_host, double* y_host, dou
             BatchArgs pa = a;
             pa.units = b->d_units + o0;
             pa.n_units = o1 - o0;
-            pa.ticket = b->io_tickets + 4 * c + 2 * part;
+            pa.ticket = b->io_tickets + 2 * c + part;
             launch_units(b, pa, part == 0, s_compute);
         }
         spmvk::check_cuda(cudaEventRecord(b->io_ev[2 * c + 1], s_compute), "event");
@@ -1316,11 +1319,11 @@ int spmv_batch_create(int count, const int64_t* n, const int64_t* const* row_ptr
     b->col = static_cast<int32_t*>(balloc(b, hcol.size() * 4));
     b->val = static_cast<double*>(balloc(b, hval.size() * 8));
     b->d_mats = static_cast<BatchMat*>(balloc(b, b->mats.size() * sizeof(BatchMat)));
-    b->ticket = static_cast<int*>(balloc(b, 2 * sizeof(int)));
+    b->ticket = static_cast<unsigned*>(balloc(b, 2 * sizeof(unsigned)));   // zeroed
     b->d_pieces = static_cast<BatchPiece*>(balloc(b, pieces.size() * sizeof(BatchPiece)));
     b->piece_sum[0] = static_cast<double*>(balloc(b, 2 * slots * sizeof(double)));
     b->piece_sum[1] = b->piece_sum[0] + slots;
-    b->piece_cnt[0] = static_cast<int*>(balloc(b, 2 * cut_rows.size() * sizeof(int)));   // zeroed
+    b->piece_cnt[0] = static_cast<unsigned*>(balloc(b, 2 * cut_rows.size() * sizeof(unsigned)));   // zeroed
     b->piece_cnt[1] = b->piece_cnt[0] + cut_rows.size();
     b->d_cut_rows = static_cast<int*>(balloc(b, cut_rows.size() * sizeof(int)));
     if (!cut_rows.empty())
@@ -1422,8 +1425,6 @@ int spmv_batch_run(spmv_batch* b, const double* x, double* y, cudaStream_t s) {
     if (b->total_rows > 0 && (!x || !y)) spmvk::fail(SPMV_EINVAL, "x_dev or y_dev is NULL");
     if (b->n_units == 0) return SPMV_OK;
     const int n_sl = b->n_sliced_units, n_csr = b->n_units - b->n_sliced_units;
-    if (!small_launch(b, n_sl) || !small_launch(b, n_csr))
-        spmvk::check_cuda(cudaMemsetAsync(b->ticket, 0, 2 * sizeof(int), s), "ticket reset");
     BatchArgs a = args_of(b, x, y);
     if (n_sl > 0) {
         a.units = b->d_units_full;

@@ -75,13 +75,13 @@ struct spmv_batch {
     int32_t* col = nullptr;
     double* val = nullptr;
     spmvk::BatchMat* d_mats = nullptr;
-    int* ticket = nullptr;
+    unsigned* ticket = nullptr;          // one per layout (zero between launches)
     double* io_x = nullptr;              // device vectors of the host-buffer path (built on first use)
     double* io_y = nullptr;
     double* io_x2 = nullptr;             // the second pair of the streamed host-buffer path
     double* io_y2 = nullptr;
     std::vector<cudaEvent_t> io_ev;      // per chunk (64): x arrived, y computed; then x free, y free per pair
-    int* io_tickets = nullptr;           // per chunk: a ticket per layout (4 ints)
+    unsigned* io_tickets = nullptr;      // per chunk: a ticket per layout
     std::vector<int> unit_off;           // 2 x (count+1): start of matrix m's units in each part of d_units
     int n_items = 0;                     // items (kinds 0 to 2)
     int n_units = 0;                     // work units
@@ -92,7 +92,7 @@ struct spmv_batch {
     std::vector<std::vector<spmvk::BatchPiece>> pieces;
     spmvk::BatchPiece* d_pieces = nullptr;
     double* piece_sum[2] = {nullptr, nullptr};
-    int* piece_cnt[2] = {nullptr, nullptr};
+    unsigned* piece_cnt[2] = {nullptr, nullptr};
     int* d_cut_rows = nullptr;           // the rows that are cut, matrix by matrix
     std::vector<int> cut_off;            // count+1
     size_t device_bytes = 0;

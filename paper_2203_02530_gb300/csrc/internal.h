@@ -80,7 +80,7 @@ struct SellArgs {
     const int32_t* perm;     // per position: row; nullptr = position is the row
     int slice_begin, slice_end, long_begin, long_end;
     double* long_part;       // partial sums of the pieces of cut rows
-    int* long_cnt;           // per cut row: pieces done (zero between launches)
+    unsigned* long_cnt;           // per cut row: pieces done (zero between launches)
     const int32_t* cta_off;  // nullptr: units round-robin over the warps; else
                              // CTA b takes units [cta_off[b], cta_off[b + 1])
     const int32_t* ypos;     // per position: its y row (row order and row map

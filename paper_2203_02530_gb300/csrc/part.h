@@ -117,7 +117,7 @@ struct spmv_part {
         int32_t* ypos = nullptr;          // REMOTE, sorted: y row of each position (perm, then the row map)
         int16_t* col16 = nullptr;         // column - row deltas (LOCAL only), once built
         double* long_part = nullptr;      // partial sums of cut long rows
-        int* long_cnt = nullptr;          // pieces done per cut long row
+        unsigned* long_cnt = nullptr;          // pieces done per cut long row
         spmvk::SellSlice* groups = nullptr;   // sorted layouts: the slices in groups (kSellGroup)
         std::vector<int64_t> group_off;   // P+1
         std::vector<int32_t> h_slice_len; // per slice: its longest row's entries

@@ -475,7 +475,7 @@ static int64_t build_sell_part(spmv_part* pt, spmv_part::SellPart& sp, const std
     sp.slices = upload(pt, slices);
     sp.longs = upload(pt, longs);
     sp.long_part = static_cast<double*>(dev_alloc(pt, (size_t)n_slots * sizeof(double)));
-    sp.long_cnt = static_cast<int*>(dev_alloc(pt, (size_t)n_cut * sizeof(int)));   // zeroed
+    sp.long_cnt = static_cast<unsigned*>(dev_alloc(pt, (size_t)n_cut * sizeof(unsigned)));   // zeroed
     sp.len = upload(pt, len);
     sp.perm = any_sorted ? upload(pt, perm) : nullptr;
     sp.val = static_cast<double*>(dev_alloc(pt, (size_t)off * 8));

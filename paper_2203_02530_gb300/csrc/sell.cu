@@ -272,12 +272,13 @@ __global__ void __launch_bounds__(256, MINB) csr_sell_kernel(CsrArgs a, SellArgs
                     // adds its pieces in piece order (independent of timing)
                     sa.long_part[L.slot] = part;
                     __threadfence();
-                    if (atomicAdd(sa.long_cnt + L.cidx, 1) == L.nparts - 1) {
+                    // the counter wraps to zero with the row's last piece: right again
+                    // after overlapped launches (whose own results are not)
+                    if (atomicInc(sa.long_cnt + L.cidx, (unsigned)L.nparts - 1) == (unsigned)L.nparts - 1) {
                         __threadfence();
                         double sum = 0.0;
                         for (int i = 0; i < L.nparts; ++i) sum += __ldcg(sa.long_part + L.first + i);
                         sell_store(a, L.row, sum);
-                        sa.long_cnt[L.cidx] = 0;   // ready for the next launch
                     }
                 }
             }
