@@ -1079,7 +1079,10 @@ int spmv_serve_run(spmv_server* sv, int64_t n_req, const int32_t* matrix, const 
             spmvk::check_cuda(cudaMalloc(reinterpret_cast<void**>(&sv->d_hash), (size_t)n_req * 8 + 8), "hashes");
             sv->hash_cap = (size_t)n_req;
         }
-        spmvk::check_cuda(cudaMemset(sv->d_hash, 0, (size_t)n_req * 8 + 8), "hashes");
+        // zeroed before any slot adds to them: the slots' streams do not wait for
+        // the default stream, which may have the caller's work queued
+        spmvk::check_cuda(cudaMemsetAsync(sv->d_hash, 0, (size_t)n_req * 8 + 8, sv->streams[0]), "hashes");
+        spmvk::check_cuda(cudaStreamSynchronize(sv->streams[0]), "hashes");
     }
     struct Inflight {
         bool busy = false;
