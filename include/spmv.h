@@ -134,7 +134,7 @@ enum {
     SPMV_Q_LAST_WAITS = 15,       /* stream waits issued for DAG edges by the last issue */
     SPMV_Q_ERROR = 16,            /* device error word (0 = none); synchronises */
     SPMV_Q_LOCAL_VARIANT = 17,
-    SPMV_Q_N_LOCAL_TILES = 18,    /* 32-row tiles of the LOCAL product */
+    SPMV_Q_N_LOCAL_TILES = 18,    /* TILE and WARP tiles of the LOCAL product */
     SPMV_Q_LAST_LAUNCHES = 19,    /* kernels launched by the last issue */
     SPMV_Q_REMOTE_VARIANT = 20,   /* 100 * variant + param of the REMOTE product
                                      (SPMV_Q_LOCAL_VARIANT: of the LOCAL one) */
@@ -181,12 +181,13 @@ int spmv_part_dag(const spmv_part* part, int32_t* edges_host, int64_t cap_pairs,
 /* Kernel variant of the LOCAL and REMOTE products (every variant gives the
  * same y within the FP64 bound; each is deterministic on its own).
  *   TILE   param = geometry 0..4 (8, 14, 4, 7 or 16 x gathers in flight per
- *          lane): tiles of 32 rows staged in shared memory by bulk copies,
- *          each by one warp, one thread per row, one DFMA per entry into
- *          two sums, of the entries at even and at odd places, that are
- *          added at the end (geometry 3: one sum); rows longer than 64
- *          entries (and, in a tile with such a row, those longer than 32)
- *          by the whole warp
+ *          lane): tiles of up to 32 rows and 1792 entries staged in shared
+ *          memory by bulk copies, each by one warp, one thread per row, one
+ *          DFMA per entry into two sums, of the entries at even and at odd
+ *          places, that are added at the end (geometry 3: one sum); in a
+ *          tile with a row longer than 64 entries the rows longer than 32 by
+ *          the whole warp where that takes less; rows longer than 1024 by a
+ *          whole CTA
  *   VECTOR param = lanes per row (2..32), 4 entries per lane per step with
  *          128-bit loads
  *   PAIRS  param = lanes per row (1, 2, 4, 8), one aligned pair of entries per

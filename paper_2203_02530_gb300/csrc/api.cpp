@@ -157,9 +157,6 @@ int op_copy(spmv_part* pt, int p, cudaStream_t s) {
 }
 
 int launch_product(spmv_part* pt, const spmvk::CsrArgs& a, bool remote, int p, cudaStream_t s) {
-    const std::vector<int64_t>& off = remote ? pt->rtile_off : pt->ltile_off;
-    const int tb = (int)(p < 0 ? 0 : off[p]);
-    const int te = (int)(p < 0 ? off[pt->P] : off[p + 1]);
     const int var = pt->variant[remote ? 1 : 0];
     const int param = pt->vparam[remote ? 1 : 0];
     if (var == SPMV_VARIANT_MERGE) {
@@ -202,7 +199,6 @@ int launch_product(spmv_part* pt, const spmvk::CsrArgs& a, bool remote, int p, c
         check_cuda(spmvk::launch_sell(al, sa, param, var == SPMV_VARIANT_SELL16, pt->num_sms, s), "sliced product");
         return (sa.slice_end > sa.slice_begin || sa.long_end > sa.long_begin) ? 1 : 0;
     }
-    const spmvk::Tile* tiles = remote ? pt->rtiles : pt->ltiles;
     if (var == SPMV_VARIANT_VECTOR || var == SPMV_VARIANT_PAIRS) {
         const std::vector<int64_t>& bo = remote ? pt->rblock_off : pt->lblock_off;
         const int bb = (int)(p < 0 ? 0 : bo[p]);
@@ -214,13 +210,17 @@ int launch_product(spmv_part* pt, const spmvk::CsrArgs& a, bool remote, int p, c
         else
             check_cuda(spmvk::launch_pairs(a, blocks, bb, be, param, pt->num_sms, s), "pair product");
         return be > bb;
-    } else {
-        if (pt->dry_run) return te > tb;
-        check_cuda(spmvk::launch_tile(a, tiles, tb, te, var == SPMV_VARIANT_WARP, param, pt->tile_cap[remote ? 1 : 0],
-                                      pt->num_sms, s),
-                   "tile product");
     }
-    return te > tb;
+    const spmv_part::TilePart& tp = pt->tile[remote ? 1 : 0];
+    const int first = p < 0 ? 0 : p, last = p < 0 ? pt->P : p + 1;   // ranks
+    const double rows = (double)(tp.row_ent[last] - tp.row_ent[first]);
+    const double all = rows + (double)(tp.tile_ent[last] - tp.tile_ent[first]);
+    const spmvk::TileSpan t{tp.tiles, (int)tp.tile_off[first], (int)tp.tile_off[last],
+                            tp.rows, (int)tp.row_off[first], (int)tp.row_off[last], all > 0 ? rows / all : 0.0, tp.cap};
+    const bool any = t.end > t.begin || t.row_end > t.row_begin;
+    if (!pt->dry_run && any)
+        check_cuda(spmvk::launch_tile(a, t, var == SPMV_VARIANT_WARP, param, pt->num_sms, s), "tile product");
+    return any;
 }
 
 int op_local(spmv_part* pt, int p, const double* x, double* y, cudaStream_t s) {
@@ -590,7 +590,7 @@ int spmv_part_query(const spmv_part* pt, int what, int part_idx, int64_t* out) {
         case SPMV_Q_LOCAL_VARIANT: *out = pt->variant[0] * 100 + pt->vparam[0]; break;
         case SPMV_Q_REMOTE_VARIANT: *out = pt->variant[1] * 100 + pt->vparam[1]; break;
         case SPMV_Q_SELL_ENTRIES: *out = pt->sell_entries; break;
-        case SPMV_Q_N_LOCAL_TILES: *out = pt->ltile_off.empty() ? 0 : pt->ltile_off[pt->P]; break;
+        case SPMV_Q_N_LOCAL_TILES: *out = pt->tile[0].tile_off.empty() ? 0 : pt->tile[0].tile_off[pt->P]; break;
         case SPMV_Q_LAST_LAUNCHES: *out = pt->last_launches; break;
         case SPMV_Q_LAST_DEFERRED: *out = pt->last_deferred; break;
         default: fail(SPMV_EINVAL, "unknown query %d", what);

@@ -13,15 +13,29 @@ namespace spmvk {
 
 // Tile of rows [r0, r1) of a CSR with entries [k0, k1); xoff is added to every
 // column index before x is read.  flags (tiles of the staged kernel): TILE_LONG
-// a row longer than kSellLong entries, TILE_WIDE more entries than the stage.
+// rows longer than 32 entries are summed by the whole warp, TILE_WIDE more
+// entries than the stage.
 struct Tile {
     int32_t r0, r1, k0, k1;
     int32_t xoff, flags, pad0, pad1;
 };
 static_assert(sizeof(Tile) == 32, "tile descriptor is two int4");
 enum { TILE_LONG = 1, TILE_WIDE = 2 };
-constexpr int kTileRows = 32;
-constexpr int kTileMaxEntries = 1792;   // 21.5 KB of stage per warp, 10 warps per SM
+constexpr int kTileRows = 32;           // at most, and at most
+constexpr int kTileMaxEntries = 1792;   // entries: 21.5 KB of stage per warp, 8 warps per SM
+constexpr int kTileCtaRow = 1024;       // a longer row is summed by a whole CTA
+
+// What one launch of the staged kernel takes: tiles [begin, end) and the rows
+// longer than kTileCtaRow (one per Tile) [row_begin, row_end), which hold
+// row_share of the entries.
+struct TileSpan {
+    const Tile* tiles;
+    int begin, end;
+    const Tile* rows;
+    int row_begin, row_end;
+    double row_share;
+    int cap;   // entries of a warp's stage
+};
 
 // Merge-path range: merge items [d0, d1) of the (row ends, entries) merge of
 // one rank's CSR; (r0, k0) is the path coordinate at d0, (r1, k1) at d1.
@@ -114,8 +128,7 @@ cudaError_t launch_gather(const double* x, const int32_t* idx, const int32_t* po
                           int64_t count, int num_sms, cudaStream_t s, int pdl = 0);
 cudaError_t launch_copy(const double* src, double* dst, int64_t count, int num_sms,
                         cudaStream_t s, int pdl = 0);
-cudaError_t launch_tile(const CsrArgs& a, const Tile* tiles, int tile_begin, int tile_end, bool one_sum, int param,
-                        int cap, int num_sms, cudaStream_t s);
+cudaError_t launch_tile(const CsrArgs& a, const TileSpan& t, bool one_sum, int param, int num_sms, cudaStream_t s);
 bool tile_param_supported(int param);
 int tile_stage_cap(int entries);   // stage size (entries) for tiles of up to `entries`
 cudaError_t launch_vector(const CsrArgs& a, const Tile* tiles, int tile_begin, int tile_end,

@@ -15,6 +15,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
 
 namespace spmvk {
@@ -215,11 +216,14 @@ cudaError_t launch_copy(const double* src, double* dst, int64_t count, int num_s
 // Warps never wait for each other.
 //
 // A tile whose entries do not fit the stage (TILE_WIDE) is summed the same
-// way straight from global memory.  In a tile with a row longer than kSellLong
-// entries (TILE_LONG) every row longer than kTileWarpRow is summed by the
-// whole warp instead (lane l takes entries l, l+32, ..., then a fixed
-// butterfly), so a long row costs its 32nd part.  Each row is summed in a
-// fixed order whatever the grid, the stream or the schedule.
+// way straight from global memory.  In a tile of TILE_LONG every row longer than
+// kTileWarpRow is summed by the whole warp instead (lane l takes entries l, l+32,
+// ..., then a fixed butterfly), so a long row costs its 32nd part.  A row longer
+// than kTileCtaRow is a chain of too many rounds even for a warp and goes to a
+// CTA (tile_row), in launches that have such rows (ROWS): their first CTAs take
+// the rows, as many as the rows' share of the entries, the others the tiles.
+// Each row is summed in a fixed order whatever the grid, the stream or the
+// schedule, and no launch keeps anything for the next.
 //
 // What bounds it: HBM and the FP64 pipe once enough warps are resident, and
 // the stages decide how many: one stage per warp, as large as 98 % of the
@@ -227,11 +231,17 @@ cudaError_t launch_copy(const double* src, double* dst, int64_t count, int num_s
 // where two stages of half as many warps or block-wide tiles of 128 rows took
 // longer.  LOCAL products: 27-point 91^3 (19.9 M entries) 51 us against 77 us
 // with block-wide double-buffered tiles and 71 us with two stages per warp;
-// 7-point 120^3 34 us against 93 us; power-law 1 M rows 126 us against 2600 us
-// (long rows one per thread); 27-point 20^3 4.5 us against 5.0 us.
+// 7-point 120^3 33 us against 93 us; 27-point 20^3 4.5 us against 5.0 us.  Long
+// rows are bound by their chains of load-then-gather rounds, so by how many warps
+// share them: 400 rows of 20 000 entries 21 us (a warp for 32 of them in turn 2941
+// us, block-wide tiles 41 us), 4000 of 3000 51 us (632 and 1426 us), one of
+// 1 000 000 among 100 000 of 5 550 us (4439 and 592 us), power-law 1 M rows in one
+// rank 143 us (160 us).
 // ------------------------------------------------------------------------
-constexpr int kTileWarps = 4;      // warps per CTA
 constexpr int kTileWarpRow = 32;   // in a TILE_LONG tile, longer rows go to the whole warp
+// warps per CTA: more for a row than for tiles, whose warps never wait for each other
+template <bool ROWS>
+constexpr int kTileCtaWarps = ROWS ? 8 : 4;
 
 struct StageLayout {   // of one warp's stage for up to `cap` entries (a multiple of 32)
     int col_off, bytes;
@@ -239,12 +249,63 @@ struct StageLayout {   // of one warp's stage for up to `cap` entries (a multipl
         : col_off((cap + 2) * 8), bytes((cap + 2) * 8 + (cap + 8) * 4) {}
 };
 
-template <int U, int S>
-__global__ void __launch_bounds__(kTileWarps * 32, U > 9 ? 8 : 10) csr_tile_kernel(CsrArgs a,
-                                                                                    const Tile* __restrict__ tiles,
-                                                                                    int tile_begin, int tile_end,
-                                                                                    int cap) {
+// One row, entries [d.k0, d.k1), by the CTA: thread t takes entries t, t + T, ...
+// (T threads, 8 of them in flight, the next columns loaded ahead), a fixed
+// butterfly in each warp, then the warps' sums in warp order.
+template <int WARPS>
+__device__ __forceinline__ void tile_row(const CsrArgs& a, const Tile& d, uint64_t pol_keep) {
+    constexpr int T = WARPS * 32, D = 8;
+    __shared__ double s_part[WARPS];
+    const unsigned n = (unsigned)(d.k1 - d.k0), t = threadIdx.x;   // unsigned: n + T D may pass 2^31
+    const int32_t* col = a.col + d.k0;
+    const double* val = a.val + d.k0;
+    const double* xb = a.x + d.xoff;
+    double part = 0.0;
+    int32_t c[D];
+#pragma unroll
+    for (int u = 0; u < D; ++u) c[u] = t + T * u < n ? __ldg(col + t + T * u) : 0;
+    for (unsigned base = 0; base < n; base += T * D) {
+        const unsigned k = base + t;
+        double vv[D], xv[D];
+#pragma unroll
+        for (int u = 0; u < D; ++u) {
+            const bool m = k + T * u < n;
+            xv[u] = m ? ldg_keep(xb + c[u], pol_keep) : 0.0;
+            vv[u] = m ? __ldg(val + k + T * u) : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < D; ++u) c[u] = k + T * (D + u) < n ? __ldg(col + k + T * (D + u)) : 0;
+#pragma unroll
+        for (int u = 0; u < D; ++u) {
+            const double p = fma(vv[u], xv[u], part);
+            part = k + T * u < n ? p : part;
+        }
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
+    if ((t & 31) == 0) s_part[t >> 5] = part;
+    __syncthreads();
+    if (t == 0) {
+        double sum = s_part[0];
+#pragma unroll
+        for (int w = 1; w < WARPS; ++w) sum += s_part[w];
+        store_row(a, d.r0, sum);
+    }
+    __syncthreads();   // s_part is rewritten for the next row
+}
+
+template <int U, int S, bool ROWS>
+__global__ void __launch_bounds__(kTileCtaWarps<ROWS> * 32, (ROWS ? 4 : U > 9 ? 8 : 10))
+    csr_tile_kernel(CsrArgs a, const Tile* __restrict__ tiles, int tile_begin, int tile_end, int cap,
+                    const Tile* __restrict__ rows, int row_begin, int row_end, int row_ctas) {
     pdl_begin(a.pdl);  // the previous kernel of this stream is done (unless independent)
+    constexpr int kTileWarps = kTileCtaWarps<ROWS>;
+    const int cta = (int)blockIdx.x - (ROWS ? row_ctas : 0);   // among those that take tiles
+    if (ROWS && cta < 0) {
+        for (int r = row_begin + (int)blockIdx.x; r < row_end; r += row_ctas)
+            tile_row<kTileWarps>(a, rows[r], policy_evict_last());
+        return;
+    }
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) uint64_t bars[kTileWarps];
     const uint64_t pol_stream = policy_evict_first();
@@ -262,7 +323,7 @@ __global__ void __launch_bounds__(kTileWarps * 32, U > 9 ? 8 : 10) csr_tile_kern
     }
     __syncwarp();
     uint32_t parity = 0;
-    for (int t = tile_begin + (int)blockIdx.x * kTileWarps + w; t < tile_end; t += (int)gridDim.x * kTileWarps) {
+    for (int t = tile_begin + cta * kTileWarps + w; t < tile_end; t += ((int)gridDim.x - (ROWS ? row_ctas : 0)) * kTileWarps) {
         const Tile d = tiles[t];
         const bool staged = d.flags == 0;
         const int va = d.k0 & ~1, ca = d.k0 & ~3;
@@ -345,22 +406,22 @@ __global__ void __launch_bounds__(kTileWarps * 32, U > 9 ? 8 : 10) csr_tile_kern
         if (live && mine) store_row(a, row, S == 2 ? sum[0] + sum[1] : sum[0]);
         for (unsigned todo = __ballot_sync(0xffffffffu, !mine); todo; todo &= todo - 1) {
             const int src = __ffs(todo) - 1;
-            const int k0 = __shfl_sync(0xffffffffu, kb, src), k1 = k0 + __shfl_sync(0xffffffffu, len, src);
+            const int k0 = __shfl_sync(0xffffffffu, kb, src), n = __shfl_sync(0xffffffffu, len, src);
             double part = 0.0;
 #pragma unroll 1
-            for (int k = k0; k < k1; k += 32 * 4) {
+            for (int k = lane; k - lane < n; k += 32 * 4) {
                 double xv[4], vv[4];
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                    const bool m = k + 32 * u + lane < k1;
-                    vv[u] = m ? __ldg(a.val + k + 32 * u + lane) : 0.0;
-                    xv[u] = m ? ldg_keep(xb + __ldg(a.col + k + 32 * u + lane), pol_keep) : 0.0;
+                    const bool m = k + 32 * u < n;
+                    vv[u] = m ? __ldg(a.val + k0 + k + 32 * u) : 0.0;
+                    xv[u] = m ? ldg_keep(xb + __ldg(a.col + k0 + k + 32 * u), pol_keep) : 0.0;
                 }
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                    if (k + 32 * u >= k1) break;   // warp-uniform
+                    if (k - lane + 32 * u >= n) break;   // warp-uniform
                     const double p = fma(vv[u], xv[u], part);
-                    part = k + 32 * u + lane < k1 ? p : part;
+                    part = k + 32 * u < n ? p : part;
                 }
             }
 #pragma unroll
@@ -376,43 +437,47 @@ int tile_stage_cap(int entries) {
     return cap < 64 ? 64 : cap > kTileMaxEntries ? kTileMaxEntries : cap;
 }
 
-template <int U, int S>
-static cudaError_t run_tile(const CsrArgs& a, const Tile* tiles, int tb, int te, int cap, int num_sms,
-                            cudaStream_t s) {
-    const size_t smem = (size_t)kTileWarps * StageLayout(cap).bytes;
+template <int U, int S, bool ROWS>
+static cudaError_t run_tile(const CsrArgs& a, const TileSpan& t, int num_sms, cudaStream_t s) {
+    constexpr int kTileWarps = kTileCtaWarps<ROWS>;
+    const size_t smem = (size_t)kTileWarps * StageLayout(t.cap).bytes;
     static std::atomic<unsigned long long> configured{0};   // one bit per device ordinal
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev >= 64 || !(configured.load(std::memory_order_acquire) >> dev & 1ull)) {
-        e = cudaFuncSetAttribute(csr_tile_kernel<U, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(csr_tile_kernel<U, S, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  kTileWarps * StageLayout(kTileMaxEntries).bytes);
         if (e != cudaSuccess) return e;
         if (dev < 64) configured.fetch_or(1ull << dev, std::memory_order_acq_rel);
     }
     // CTAs per SM by stage size (a query costs the host about a microsecond)
     static std::atomic<int> known[kTileMaxEntries / 32 + 1];
-    int occ = dev == 0 ? known[cap / 32].load(std::memory_order_relaxed) : 0;
+    int occ = dev == 0 ? known[t.cap / 32].load(std::memory_order_relaxed) : 0;
     if (occ == 0) {
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, csr_tile_kernel<U, S>, kTileWarps * 32, smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, csr_tile_kernel<U, S, ROWS>, kTileWarps * 32, smem);
         if (e != cudaSuccess) return e;
         if (occ < 1) return cudaErrorInvalidConfiguration;
-        if (dev == 0) known[cap / 32].store(occ, std::memory_order_relaxed);
+        if (dev == 0) known[t.cap / 32].store(occ, std::memory_order_relaxed);
     }
-    int grid = num_sms * occ;
-    const int need = (te - tb + kTileWarps - 1) / kTileWarps;
-    if (grid > need) grid = need;
-    return launch_pdl(csr_tile_kernel<U, S>, dim3(grid), dim3(kTileWarps * 32), smem, s, a, tiles, tb, te, cap);
+    const int most = num_sms * occ, need = (t.end - t.begin + kTileWarps - 1) / kTileWarps;
+    int row_ctas = 0;
+    if (ROWS) {
+        row_ctas = need > 0 ? std::min(std::max((int)(t.row_share * most), 1), most - 1) : most;
+        row_ctas = std::min(row_ctas, t.row_end - t.row_begin);
+    }
+    const int grid = row_ctas + std::min(need, most - row_ctas);
+    return launch_pdl(csr_tile_kernel<U, S, ROWS>, dim3(grid), dim3(kTileWarps * 32), smem, s, a, t.tiles,
+                      t.begin, t.end, t.cap, t.rows, t.row_begin, t.row_end, row_ctas);
 }
 
 bool tile_param_supported(int param) { return param >= 0 && param < 5; }
 
 // Geometries: gathers in flight per lane.  TILE keeps two sums a row (geometry
 // 3: one), WARP one.
-cudaError_t launch_tile(const CsrArgs& a, const Tile* tiles, int tile_begin, int tile_end, bool one_sum, int param,
-                        int cap, int num_sms, cudaStream_t s) {
-    if (tile_end <= tile_begin) return cudaSuccess;
-#define TILE_RUN(u, sums) return run_tile<u, sums>(a, tiles, tile_begin, tile_end, cap, num_sms, s)
+cudaError_t launch_tile(const CsrArgs& a, const TileSpan& t, bool one_sum, int param, int num_sms, cudaStream_t s) {
+    const bool rows = t.row_end > t.row_begin;
+#define TILE_RUN(u, sums) return rows ? run_tile<u, sums, true>(a, t, num_sms, s) : run_tile<u, sums, false>(a, t, num_sms, s)
     switch (one_sum ? param + 5 : param) {
         case 0: TILE_RUN(8, 2);
         case 1: TILE_RUN(14, 2);

@@ -86,12 +86,15 @@ struct spmv_part {
     // after the rank's LOCAL product; the host path copies it out early)
     std::vector<std::pair<int64_t, int64_t>> io_free;
 
-    // 32-row tiles of the staged kernel and its stage size, LOCAL and REMOTE
-    spmvk::Tile* ltiles = nullptr;
-    spmvk::Tile* rtiles = nullptr;
-    int tile_cap[2] = {0, 0};
-    std::vector<int64_t> ltile_off;   // P+1
-    std::vector<int64_t> rtile_off;   // P+1
+    // tiles of the staged kernel, LOCAL and REMOTE: per rank (P+1 offsets) its
+    // tiles, its rows of a CTA each and the entries of either
+    struct TilePart {
+        spmvk::Tile* tiles = nullptr;
+        spmvk::Tile* rows = nullptr;
+        std::vector<int64_t> tile_off, row_off, tile_ent, row_ent;
+        int cap = 0;   // entries of a warp's stage
+    };
+    TilePart tile[2];
     // fixed 256-row blocks (vector and pair kernels)
     spmvk::Tile* lblocks = nullptr;
     spmvk::Tile* rblocks = nullptr;

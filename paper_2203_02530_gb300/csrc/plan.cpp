@@ -237,19 +237,66 @@ void build_plan(spmv_part* pt, int64_t n, const int64_t* rp, const int32_t* ci,
     pt->err = static_cast<int*>(dev_alloc(pt, sizeof(int)));
 }
 
-// 32-row tiles of one CSR row range.
+// Tiles of one CSR row range: consecutive rows while they are at most kTileRows
+// and hold at most kTileMaxEntries, so that a tile fits a stage and rows of
+// hundreds of entries still make tiles for many warps; rows longer than
+// kTileCtaRow go to `rows`, a CTA each.  For tile_kinds, pad0 and pad1 are the
+// tile's FP64 instructions with the rows longer than 32 entries summed by the
+// whole warp (a step per 32 entries and 5 to add the lanes) and with a row per
+// lane (the longest row's entries); 0 in tiles without a row longer than
+// kSellLong.
 static void tile_range(const std::vector<int32_t>& ptr, int64_t rb, int64_t re, int32_t xoff,
-                       std::vector<Tile>& out) {
-    for (int64_t r = rb; r < re; r += kTileRows) {
-        const int64_t e = std::min<int64_t>(re, r + kTileRows);
-        int32_t flags = 0;
-        for (int64_t i = r; i < e; ++i)
-            if (ptr[(size_t)i + 1] - ptr[(size_t)i] > kSellLong) flags = TILE_LONG;
-        out.push_back(Tile{(int32_t)r, (int32_t)e, ptr[(size_t)r], ptr[(size_t)e], xoff, flags, 0, 0});
+                       std::vector<Tile>& out, std::vector<Tile>& rows) {
+    auto len = [&](int64_t r) { return ptr[(size_t)r + 1] - ptr[(size_t)r]; };
+    auto add = [&](std::vector<Tile>& to, int64_t r0, int64_t r1, int32_t flags) {
+        to.push_back(Tile{(int32_t)r0, (int32_t)r1, ptr[(size_t)r0], ptr[(size_t)r1], xoff, flags, 0, 0});
+    };
+    for (int64_t r = rb; r < re;) {
+        const int64_t start = r;
+        int32_t cnt = 0, most = 0, most_short = 0, by_warp = 0;
+        for (; r < re && r - start < kTileRows && len(r) <= kTileCtaRow && cnt + len(r) <= kTileMaxEntries; ++r) {
+            cnt += len(r);
+            most = std::max(most, len(r));
+            if (len(r) > 32) by_warp += (len(r) + 31) / 32 + 5;
+            else most_short = std::max(most_short, len(r));
+        }
+        if (r == start) {
+            add(rows, r, r + 1, 0);
+            ++r;
+            continue;
+        }
+        add(out, start, r, 0);
+        if (most > kSellLong) {
+            out.back().pad0 = most_short + by_warp;
+            out.back().pad1 = most;
+        }
     }
 }
 
-// Stage size for a product's tiles: what 98 % of those without long rows need
+// Which tiles are TILE_LONG: those with a few long rows among short ones, where
+// summing rows by the whole warp takes fewer instructions.  Tiles of rows as long
+// as each other take more, but need no stage, which leaves 40 warps per SM
+// instead of 8: all of a product's are TILE_LONG where theirs are fewer than 2.5
+// times as many, else none, since the largest stage counts for every warp.
+// 50 000 rows of 65 to 100 entries (1.8 times) 33 us against 58 us with stages
+// for some; 200 000 rows of 33 to 66 (3.4 times) 69 us against 224 us.
+static void tile_kinds(std::vector<Tile>& tiles) {
+    int64_t by_warp = 0, by_lane = 0;
+    for (Tile& t : tiles) {
+        if (t.pad0 < t.pad1) {
+            t.flags = TILE_LONG;
+        } else {
+            by_warp += t.pad0;
+            by_lane += t.pad1;
+        }
+    }
+    for (Tile& t : tiles) {
+        if (t.pad1 > 0 && 2 * by_warp < 5 * by_lane) t.flags = TILE_LONG;
+        t.pad0 = t.pad1 = 0;
+    }
+}
+
+// Stage size for a product's tiles: what 98 % of those not TILE_LONG need
 // (a few wide tiles then do not cost every warp its shared memory); the
 // others are marked TILE_WIDE.
 static int tile_stage(std::vector<Tile>& tiles) {
@@ -278,21 +325,27 @@ void build_tiles(spmv_part* pt) {
     const int P = pt->P;
     const std::vector<int32_t> l_ptr = download(pt->l_ptr, (size_t)pt->n + 1);
     const std::vector<int32_t> rr_ptr = download(pt->rr_ptr, (size_t)pt->n_rr + 1);
-    std::vector<Tile> lt, rt;
-    pt->ltile_off.assign(P + 1, 0);
-    pt->rtile_off.assign(P + 1, 0);
-    for (int p = 0; p < P; ++p) {
-        pt->ltile_off[p] = (int64_t)lt.size();
-        tile_range(l_ptr, pt->bounds[p], pt->bounds[p + 1], (int32_t)pt->bounds[p], lt);
-        pt->rtile_off[p] = (int64_t)rt.size();
-        tile_range(rr_ptr, pt->rr_off[p], pt->rr_off[p + 1], 0, rt);
+    for (int part = 0; part < 2; ++part) {
+        spmv_part::TilePart& tp = pt->tile[part];
+        const std::vector<int32_t>& ptr = part ? rr_ptr : l_ptr;
+        const std::vector<int64_t>& first = part ? pt->rr_off : pt->bounds;
+        std::vector<Tile> tiles, rows;
+        for (auto* off : {&tp.tile_off, &tp.row_off, &tp.tile_ent, &tp.row_ent}) off->assign(P + 1, 0);
+        for (int p = 0; p < P; ++p) {
+            const size_t row0 = rows.size();
+            tile_range(ptr, first[p], first[p + 1], part ? 0 : (int32_t)pt->bounds[p], tiles, rows);
+            int64_t in_rows = 0;
+            for (size_t i = row0; i < rows.size(); ++i) in_rows += rows[i].k1 - rows[i].k0;
+            tp.tile_off[p + 1] = (int64_t)tiles.size();
+            tp.row_off[p + 1] = (int64_t)rows.size();
+            tp.row_ent[p + 1] = tp.row_ent[p] + in_rows;
+            tp.tile_ent[p + 1] = tp.tile_ent[p] + (ptr[(size_t)first[p + 1]] - ptr[(size_t)first[p]]) - in_rows;
+        }
+        tile_kinds(tiles);
+        tp.cap = tile_stage(tiles);
+        tp.tiles = upload(pt, tiles);
+        tp.rows = upload(pt, rows);
     }
-    pt->ltile_off[P] = (int64_t)lt.size();
-    pt->rtile_off[P] = (int64_t)rt.size();
-    pt->tile_cap[0] = tile_stage(lt);
-    pt->tile_cap[1] = tile_stage(rt);
-    pt->ltiles = upload(pt, lt);
-    pt->rtiles = upload(pt, rt);
     {
         std::vector<Tile> lb, rb;
         pt->lblock_off.assign(P + 1, 0);
