@@ -529,6 +529,7 @@ int spmv_part_create(int64_t n, const int64_t* row_ptr, const int32_t* col_idx, 
     spmvk::build_plan(pt, n, row_ptr, col_idx, vals);
     spmvk::build_tiles(pt);
     build_dag(pt);
+    spmvk::default_stream_done();
     *out = pt;
     pt = nullptr;
     return SPMV_OK;
@@ -794,6 +795,7 @@ static void prepare_variant(spmv_part* pt, int variant, int param, int op_kind) 
         if (spmvk::sell_param_balanced(param)) {
             if (op_kind != SPMV_OP_REMOTE) spmvk::build_sell_split(pt, 0, param, variant == SPMV_VARIANT_SELL16);
             if (op_kind != SPMV_OP_LOCAL) spmvk::build_sell_split(pt, 1, param, false);
+            spmvk::default_stream_done();
         }
     } else {
         fail(SPMV_EINVAL, "unknown variant %d", variant);
@@ -942,6 +944,7 @@ int spmv_part_io_buffers(spmv_part* pt, double** x_out, double** y_out) {
     if (!pt->io_x) {
         pt->io_x = static_cast<double*>(spmvk::dev_alloc(pt, (size_t)pt->n * sizeof(double)));
         pt->io_y = static_cast<double*>(spmvk::dev_alloc(pt, (size_t)pt->n * sizeof(double)));
+        spmvk::default_stream_done();
     }
     *x_out = pt->io_x;
     *y_out = pt->io_y;
@@ -961,7 +964,7 @@ void host_path_setup(spmv_part* pt) {
     if (!pt->io_x) {
         pt->io_x = static_cast<double*>(spmvk::dev_alloc(pt, (size_t)pt->n * sizeof(double)));
         pt->io_y = static_cast<double*>(spmvk::dev_alloc(pt, (size_t)pt->n * sizeof(double)));
-        check_cuda(cudaDeviceSynchronize(), "synchronize");   // zero-filled before other streams write
+        spmvk::default_stream_done();
     }
     while ((int)pt->io_ev.size() < 3 * P + 5) {
         cudaEvent_t e;
@@ -1173,7 +1176,7 @@ int spmv_apply_host_many(spmv_part* pt, int64_t count, const double* x_host, int
     if (!pt->io_x2) {
         pt->io_x2 = static_cast<double*>(spmvk::dev_alloc(pt, (size_t)pt->n * sizeof(double)));
         pt->io_y2 = static_cast<double*>(spmvk::dev_alloc(pt, (size_t)pt->n * sizeof(double)));
-        check_cuda(cudaDeviceSynchronize(), "synchronize");   // zero-filled before other streams write
+        spmvk::default_stream_done();
     }
     int64_t launches = 0;
     const bool coarse = !(flags & SPMV_HOST_X_BLOCKS) && host_coarse(pt, count);

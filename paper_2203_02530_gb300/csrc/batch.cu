@@ -855,6 +855,7 @@ void upload_items(spmv_batch* b) {
     put(b->d_items, b->items_cap, all);
     put(b->d_units, b->units_cap, order);
     put(b->d_units_full, b->units_full_cap, full);
+    spmvk::default_stream_done();
 }
 
 // Sliced layout of matrix m.  Natural row order when no row is longer than
@@ -1029,6 +1030,7 @@ void batch_release_csr(spmv_batch* b) {
     for (int m = 0; m < b->count; ++m) b->mats[m].ent_off = ent_off[m];
     spmvk::check_cuda(cudaMemcpy(b->d_mats, b->mats.data(), b->mats.size() * sizeof(BatchMat), cudaMemcpyHostToDevice),
                       "matrix table");
+    spmvk::default_stream_done();
     b->csr_released = true;
 }
 
@@ -1074,6 +1076,7 @@ void batch_restore_csr(spmv_batch* b) {
     for (int m = 0; m < b->count; ++m) b->mats[m].ent_off = b->full_ent_off[m];
     spmvk::check_cuda(cudaMemcpy(b->d_mats, b->mats.data(), b->mats.size() * sizeof(BatchMat), cudaMemcpyHostToDevice),
                       "matrix table");
+    spmvk::default_stream_done();
     b->h_full_ptr.clear();
     b->full_ent_off.clear();
     b->csr_released = false;
@@ -1147,7 +1150,7 @@ void batch_host_setup(spmv_batch* b) {
         b->io_x = static_cast<double*>(balloc(b, (size_t)b->total_rows * sizeof(double)));
         b->io_y = static_cast<double*>(balloc(b, (size_t)b->total_rows * sizeof(double)));
         b->io_tickets = static_cast<unsigned*>(balloc(b, 2 * 64 * sizeof(unsigned)));
-        spmvk::check_cuda(cudaDeviceSynchronize(), "synchronize");   // zero-filled before other streams write
+        spmvk::default_stream_done();
     }
     while ((int)b->io_ev.size() < 2 * 64 + 4) {
         cudaEvent_t e;
@@ -1382,6 +1385,7 @@ int spmv_batch_set_lanes(spmv_batch* b, int m, int lanes) {
                                  cudaMemcpyHostToDevice),
                       "lanes");
     if (changed) upload_items(b);
+    else spmvk::default_stream_done();
     BATCH_CATCH
     return SPMV_OK;
 }
@@ -1473,7 +1477,7 @@ int spmv_batch_run_host_many(spmv_batch* b, int64_t count, const double* x_host,
     if (!b->io_x2) {
         b->io_x2 = static_cast<double*>(balloc(b, (size_t)b->total_rows * sizeof(double)));
         b->io_y2 = static_cast<double*>(balloc(b, (size_t)b->total_rows * sizeof(double)));
-        spmvk::check_cuda(cudaDeviceSynchronize(), "synchronize");   // zero-filled before other streams write
+        spmvk::default_stream_done();
     }
     for (int64_t k = 0; k < count; ++k) {
         const int slot = (int)(k & 1);

@@ -193,6 +193,7 @@ void restore_csr(spmv_part* pt);
 // all ranks) takes the layout's groups.
 bool sell_grouped(const spmv_part* pt, int part_idx, int site, int param);
 const int32_t* sell_split(const spmv_part* pt, int part_idx, bool grouped, int site, int grid);
-void* dev_alloc(spmv_part* pt, size_t bytes);
+void* dev_alloc(spmv_part* pt, size_t bytes);   // zero-filled on the default stream
+void default_stream_done();
 void free_plan(spmv_part* pt);
 }  // namespace spmvk

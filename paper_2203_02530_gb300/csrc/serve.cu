@@ -962,6 +962,7 @@ int spmv_serve_create(spmv_batch* mats, int n_streams, int64_t budget_bytes, spm
         if (!all.empty())
             spmvk::check_cuda(cudaMemcpy(sv->bucket_rows, all.data(), all.size() * 4, cudaMemcpyHostToDevice),
                               "row buckets");
+        spmvk::default_stream_done();
     }
     // the pool holds the X/Y blocks of every block in flight; beyond what
     // the slots can ever hold at once the budget is never used, so it is
