@@ -462,40 +462,24 @@ def run_ours(args, world, rank, local, fp64=None):
             sched = [(order, [0] * part.n_ops, evaluate(order, [0] * part.n_ops))]
         by_mode[run_mode] = sorted(sched, key=lambda r: r[2])
     run_mode = min(by_mode, key=lambda m: by_mode[m][0][2])
-    sched = by_mode[run_mode]
-    mode_flag = {"strict": 0, "relaxed": spmv.RUN_RELAXED, "defer": spmv.RUN_DEFER,
-                 "relaxed+defer": spmv.RUN_RELAXED | spmv.RUN_DEFER}[run_mode]
-    order, smap, t_best = sched[0]
     # the variants were tuned on launches timed one after another; a program
     # overlaps its kernels (a per-rank program its ranks', a deferred remote
-    # product the local product's tail), so the best program is re-timed with
-    # the three fastest LOCAL x three fastest REMOTE variants of the tuning and
-    # the fastest pair kept
+    # product the local product's tail), so the best program of each ordering
+    # mode is re-timed with the fastest variants of the tuning and the fastest
+    # pair kept, with its mode
     in_context = None
-    if len(sched[0][0]) > 1:
-        def top(op):
-            c = sorted(((t, v, p) for (o, v, p), t in tune_times.items() if o == op))
-            return [(v, p) for _, v, p in c[:3]]
-        ev_ctx = search.graph_evaluator(part, streams, x_d, y_d, measurements=3, relaxed="relaxed" in run_mode,
-                                        defer="defer" in run_mode)
-        in_context = {}
-        best = (t_best, tuple(tuned["local"]), tuple(tuned["remote"]))
-        for lv in top(spmv.OP_LOCAL):
-            for rv in top(spmv.OP_REMOTE):
-                try:
-                    part.set_op_variant(spmv.OP_LOCAL, *lv)
-                    part.set_op_variant(spmv.OP_REMOTE, *rv)
-                except spmv.SpmvError:
-                    continue
-                t = ev_ctx(order, smap)
-                in_context["%d,%d/%d,%d" % (lv + rv)] = round(t * 1e6, 2)
-                if t < best[0]:
-                    best = (t, lv, rv)
-        part.set_op_variant(spmv.OP_LOCAL, *best[1])
-        part.set_op_variant(spmv.OP_REMOTE, *best[2])
-        tuned = dict(tuned, local=best[1], remote=best[2])
+    if len(by_mode[run_mode][0][0]) > 1:
+        def evaluator(m):
+            return search.graph_evaluator(part, streams, x_d, y_d, measurements=3, relaxed="relaxed" in m,
+                                          defer="defer" in m)
+        (_, run_mode, lv, rv), table = search.variants_in_context(
+            part, tune_times, tuned, {m: by_mode[m][0][:2] for m in by_mode}, {m: evaluator(m) for m in by_mode})
+        in_context = {"%d,%d/%d,%d" % (a + b): [round(t * 1e6, 2), m] for (a, b), (t, m) in table.items()}
+        if (lv, rv) != (tuple(tuned["local"]), tuple(tuned["remote"])) and mode == "exhaustive":
+            # other variants: the order of the schedules may differ
+            by_mode[run_mode] = sorted(search.exhaustive(part, streams, evaluator(run_mode)), key=lambda r: r[2])
+        tuned = dict(tuned, local=lv, remote=rv)
         variant, vparam = tuned["local"]
-        t_best = best[0]
         # a CSR variant timed here rebuilt the CSR copy: release it again when
         # both kept products are sliced
         if variant in (spmv.VARIANT_SELL, spmv.VARIANT_SELL16) and tuned["remote"][0] == spmv.VARIANT_SELL:
@@ -504,6 +488,10 @@ def run_ours(args, world, rank, local, fp64=None):
             except spmv.SpmvError as e:   # reported through the plan bytes; the products are unaffected
                 print("CSR copy kept: %s" % e, file=sys.stderr)
         plan_bytes["timed"] = part.query(spmv.Q_DEVICE_BYTES)
+    sched = by_mode[run_mode]
+    order, smap = sched[0][:2]
+    mode_flag = {"strict": 0, "relaxed": spmv.RUN_RELAXED, "defer": spmv.RUN_DEFER,
+                 "relaxed+defer": spmv.RUN_RELAXED | spmv.RUN_DEFER}[run_mode]
     t_search = time.perf_counter() - t_search
     spread = sched[-1][2] / sched[0][2]
     g = part.run(order, smap, streams, x_d, y_d, spmv.RUN_CAPTURE | mode_flag)

@@ -85,6 +85,41 @@ def mcts(part, streams, evaluate, iterations, seed=0):
     return tree.run(iterations), tree
 
 
+def variants_in_context(part, times, tuned, programs, evaluators, top=3):
+    """The kernel variants re-timed in whole programs: they were tuned on
+    launches timed one after another, but a program overlaps its kernels.
+
+    Tries the `top` fastest LOCAL x `top` fastest REMOTE variants of `times`
+    ({(op, variant, param): seconds}), and the fastest sliced REMOTE product
+    besides: it is the only one that can sum its rows before waiting for the
+    kernel before it (SPMV_RUN_DEFER), worth more in a program than the tenth of
+    a microsecond by which another variant may win alone.  Each pair is timed in
+    every ordering mode, with that mode's program: `programs` {mode: (order,
+    stream map)}, `evaluators` {mode: evaluate(order, stream map) -> seconds}.
+    The fastest pair is applied; a pair the plan refuses is left out.  Returns
+    (seconds, mode, local, remote) and {(local, remote): (seconds, mode)}."""
+    def ranked(op):
+        return [(v, p) for _, v, p in sorted((t, v, p) for (o, v, p), t in times.items() if o == op)]
+    local, remote = ranked(spmv.OP_LOCAL)[:top], ranked(spmv.OP_REMOTE)
+    sliced = [vp for vp in remote if vp[0] == spmv.VARIANT_SELL]
+    remote = remote[:top]
+    remote += [vp for vp in sliced[:1] if vp not in remote]
+    pairs = [(tuple(tuned["local"]), tuple(tuned["remote"]))]
+    pairs += [(lv, rv) for lv in local for rv in remote if (lv, rv) != pairs[0]]
+    table = {}
+    for lv, rv in pairs:
+        try:
+            part.set_op_variant(spmv.OP_LOCAL, *lv)
+            part.set_op_variant(spmv.OP_REMOTE, *rv)
+        except spmv.SpmvError:
+            continue
+        table[lv, rv] = min((evaluators[m](*programs[m]), m) for m in programs)
+    lv, rv = min(table, key=lambda pair: table[pair][0])
+    part.set_op_variant(spmv.OP_LOCAL, *lv)
+    part.set_op_variant(spmv.OP_REMOTE, *rv)
+    return table[lv, rv] + (lv, rv), table
+
+
 def random_sampling(part, streams, evaluate, count, seed=0, mode="uniform"):
     """Baseline search (Sec. VI: random sampling against MCTS at an equal
     number of measured programs): `count` distinct programs drawn at random
