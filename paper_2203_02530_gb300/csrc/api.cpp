@@ -1332,6 +1332,12 @@ int spmv_part_check(spmv_part* pt, int64_t* bad_out) {
                  t_bhi = put(bhi), t_rr = put(pt->rr_off), t_hlo = put(hlo), t_hhi = put(hhi),
                  t_seg = put(pt->seg_off), t_slo = put(slo), t_shi = put(shi),
                  t_one = put(std::vector<int64_t>{0, pt->n_send});
+    size_t t_group[2] = {0, 0}, t_slice[2] = {0, 0};
+    for (int part = 0; part < 2; ++part)
+        if (pt->sell[part].groups) {
+            t_group[part] = put(pt->sell[part].group_off);
+            t_slice[part] = put(pt->sell[part].slice_off);
+        }
     int64_t* d_tab = nullptr;
     unsigned long long* d_bad = nullptr;
     check_cuda(cudaMalloc(&d_tab, tab.size() * sizeof(int64_t) + 64), "check tables");
@@ -1376,6 +1382,11 @@ int spmv_part_check(spmv_part* pt, int64_t* bad_out) {
                     r = spmvk::launch_check_sell(sp.slices, (int)sp.slice_off[P], sp.len, sp.perm, nullptr,
                                                  sp.col16, sp.entries, npos, 0, xhi, sp.longs, 0, cptr, d_bad,
                                                  sms, 0);
+                // the groups hold the slices that follow one another, those of
+                // more than one slice full rows of one length
+                if (r == cudaSuccess && sp.groups)
+                    r = spmvk::launch_check_groups(sp.groups, sp.group_off[P], d_tab + t_group[part], sp.slices,
+                                                   d_tab + t_slice[part], P, sp.len, npos, d_bad, sms, 0);
                 // the composed y rows of rank p's remote positions are p's rows
                 if (r == cudaSuccess && sp.ypos)
                     r = spmvk::launch_check_list(sp.ypos, pt->n_rr, d_tab + t_rr, P, d_tab + t_blo, d_tab + t_bhi,

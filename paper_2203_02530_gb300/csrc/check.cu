@@ -4,6 +4,7 @@
 // allows it, and count the ones outside.  They never use an index to
 // address memory, so a corrupt plan is reported, not dereferenced.
 #include "internal.h"
+#include "sell_groups.h"
 
 #include <cuda_runtime.h>
 
@@ -108,6 +109,21 @@ __global__ void check_sell_kernel(const SellSlice* __restrict__ slices, int n_sl
     if (mine) atomicAdd(bad, mine);
 }
 
+// Every group of a sorted layout (sell_group_ok).
+__global__ void check_groups_kernel(const SellSlice* __restrict__ groups, int64_t n_groups,
+                                    const int64_t* __restrict__ group_off, const SellSlice* __restrict__ slices,
+                                    const int64_t* __restrict__ slice_off, int P, const uint8_t* __restrict__ len,
+                                    int64_t npos, unsigned long long* bad) {
+    unsigned long long mine = 0;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_groups; i += stride) {
+        const int p = find_seg(group_off, P, i);
+        if (!sell_group_ok(groups, i, group_off[p], group_off[p + 1], slices, slice_off[p], slice_off[p + 1], len, npos))
+            ++mine;
+    }
+    if (mine) atomicAdd(bad, mine);
+}
+
 int grid_for(int64_t items, int num_sms) {
     int64_t g = (items + 255) / 256;
     if (g < 1) g = 1;
@@ -128,6 +144,15 @@ cudaError_t launch_check_list(const int32_t* idx, int64_t count, const int64_t* 
                               const int64_t* hi, unsigned long long* bad, int num_sms, cudaStream_t s) {
     if (count <= 0) return cudaSuccess;
     check_list_kernel<<<grid_for(count, num_sms), 256, 0, s>>>(idx, count, seg, S, lo, hi, bad);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_check_groups(const SellSlice* groups, int64_t n_groups, const int64_t* group_off,
+                                const SellSlice* slices, const int64_t* slice_off, int P, const uint8_t* len,
+                                int64_t npos, unsigned long long* bad, int num_sms, cudaStream_t s) {
+    if (n_groups <= 0) return cudaSuccess;
+    check_groups_kernel<<<grid_for(n_groups, num_sms), 256, 0, s>>>(groups, n_groups, group_off, slices, slice_off, P,
+                                                                    len, npos, bad);
     return cudaGetLastError();
 }
 

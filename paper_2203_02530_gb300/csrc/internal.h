@@ -57,7 +57,9 @@ struct Carry {
 // at off + 32 j + r.
 struct SellSlice {
     int32_t p0, rows, len, xoff;
-    int32_t off, group, pad1, pad2;   // group: slices in the group this descriptor starts (1: the slice alone)
+    // group: slices in the group this descriptor starts (1: the slice alone);
+    // first: in the group table, the index of its first slice
+    int32_t off, group, first, pad2;
 };
 static_assert(sizeof(SellSlice) == 32, "slice descriptor is two int4");
 
@@ -175,6 +177,11 @@ cudaError_t launch_check_csr(const int32_t* ptr, const int32_t* col, int64_t nro
                              unsigned long long* bad, int num_sms, cudaStream_t s);
 cudaError_t launch_check_list(const int32_t* idx, int64_t count, const int64_t* seg, int S, const int64_t* lo,
                               const int64_t* hi, unsigned long long* bad, int num_sms, cudaStream_t s);
+// Groups of a sorted layout, rank p's [group_off[p], group_off[p + 1]) of its
+// slices [slice_off[p], slice_off[p + 1]) (device tables of P + 1).
+cudaError_t launch_check_groups(const SellSlice* groups, int64_t n_groups, const int64_t* group_off,
+                                const SellSlice* slices, const int64_t* slice_off, int P, const uint8_t* len,
+                                int64_t npos, unsigned long long* bad, int num_sms, cudaStream_t s);
 cudaError_t launch_check_sell(const SellSlice* slices, int n_slices, const uint8_t* len, const int32_t* perm,
                               const int32_t* col, const int16_t* col16, int64_t entries, int64_t npos, int64_t x_lo,
                               int64_t x_hi, const SellLong* longs, int n_longs, const int32_t* csr_ptr,

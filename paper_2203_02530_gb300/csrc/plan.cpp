@@ -520,6 +520,7 @@ static int64_t build_sell_part(spmv_part* pt, spmv_part::SellPart& sp, const std
                     ++got;
                 groups.push_back(slices[(size_t)i]);
                 groups.back().group = got == want ? want : 1;
+                groups.back().first = (int32_t)i;
                 i += got == want ? want : 1;
             }
         }
