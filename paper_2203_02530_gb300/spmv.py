@@ -226,7 +226,8 @@ def spmv_schedule_run(h, op_order, stream_of_op, streams, x_dev, y_dev,
     """Run, capture or replay one implementation; returns the graph handle."""
     order = np.ascontiguousarray(op_order, dtype=np.int32)
     smap = np.ascontiguousarray(stream_of_op, dtype=np.int32)
-    sarr = (ctypes.c_void_p * len(streams))(*[_stream(s) for s in streams])
+    # 0 +: an entry that is None is refused, not taken for the default stream
+    sarr = (ctypes.c_void_p * len(streams))(*[0 + _stream(s) for s in streams])
     g = ctypes.c_int64(int(graph_handle))
     # a replay reads neither the order nor the stream map
     replay = (int(flags) & ~(RUN_RELAXED | RUN_DEFER)) == RUN_REPLAY
