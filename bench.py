@@ -588,6 +588,8 @@ def run_ours(args, world, rank, local, fp64=None):
     many_flags = {"x whole, y whole": 0, "x blocks, y whole": spmv.HOST_X_BLOCKS,
                   "x whole, y parts": spmv.HOST_Y_PARTS,
                   "x blocks, y parts": spmv.HOST_X_BLOCKS | spmv.HOST_Y_PARTS}
+    if n <= 600_000 * P:   # with x whole both take one launch per operation and y in one copy
+        del many_flags["x whole, y parts"]
     many_sweep = {}
     for name, fl in many_flags.items():
         spmv.spmv_apply_host_many(part.h, 3, xh, 0, yh, 0, fl, cs, streams[0])
