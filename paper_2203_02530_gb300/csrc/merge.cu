@@ -21,6 +21,7 @@
 // reads a thread, and a launch of its own that computed the tiles), took 154 us.
 // 7-point stencil of 12 696 rows: 6.2 us against 14.3 us.
 #include "internal.h"
+#include "merge_chunks.h"
 #include "pdl.cuh"
 
 #include <cuda_runtime.h>
@@ -36,8 +37,6 @@ namespace {
 
 constexpr int MERGE_NT = 256;                 // threads per CTA
 constexpr int MERGE_WARPS = MERGE_NT / 32;
-constexpr int MERGE_LANE = 8;                 // entries per lane and chunk
-constexpr int MERGE_CHUNK = 32 * MERGE_LANE;  // entries per chunk
 constexpr int kErrTimeout = 6;
 
 // Items per range.  A chunk starts at a multiple of MERGE_LANE entries, so a
@@ -156,11 +155,11 @@ __global__ void __launch_bounds__(MERGE_NT, 4) merge_kernel(CsrArgs a, const Mer
         }
         int cur = r0;          // first row whose end has not been passed
         double open = 0.0;     // partial sum of row `cur` over the chunks so far
-        for (int c = k0 & ~(MERGE_LANE - 1); c < k1; c += MERGE_CHUNK) {
-            const int e = c + MERGE_LANE * lane;
+        for (unsigned c = merge_first_chunk(k0); c < (unsigned)k1; c += MERGE_CHUNK) {
+            const unsigned e = c + MERGE_LANE * lane;
             double v[MERGE_LANE];
             int32_t col[MERGE_LANE];
-            if (e < k1 && (PLAN || e + MERGE_LANE <= a.nnz_total)) {
+            if (e < (unsigned)k1 && (PLAN || e + MERGE_LANE <= (unsigned)a.nnz_total)) {
                 if (A32) {
                     asm("ld.global.nc.v8.s32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                         : "=r"(col[0]), "=r"(col[1]), "=r"(col[2]), "=r"(col[3]), "=r"(col[4]), "=r"(col[5]),
@@ -186,7 +185,7 @@ __global__ void __launch_bounds__(MERGE_NT, 4) merge_kernel(CsrArgs a, const Mer
             } else {
 #pragma unroll
                 for (int u = 0; u < MERGE_LANE; ++u) {
-                    const bool in = e + u < k1;
+                    const bool in = e + u < (unsigned)k1;
                     col[u] = in ? __ldg(a.col + e + u) : 0;
                     v[u] = in ? __ldg(a.val + e + u) : 0.0;
                 }
@@ -194,18 +193,17 @@ __global__ void __launch_bounds__(MERGE_NT, 4) merge_kernel(CsrArgs a, const Mer
             double xv[MERGE_LANE];
 #pragma unroll
             for (int u = 0; u < MERGE_LANE; ++u) {
-                const bool in = e + u >= k0 && e + u < k1;   // neighbours of the range's first and last entries
+                const bool in = merge_in_range(e + u, k0, k1);   // neighbours of the range's first and last entries
                 xv[u] = in ? __ldg(xb + col[u]) : 0.0;
                 v[u] = in ? v[u] : 0.0;
             }
             // flag the last entry of every row that ends in the chunk and has
             // an entry in the range
-            const int ce = c + MERGE_CHUNK;
             int row = cur;
             for (;;) {
                 const int r = row + lane;
-                const int end = r < r1 ? __ldg(a.ptr + r + 1) : INT32_MAX;
-                const bool here = end <= ce;
+                const int end = r < r1 ? __ldg(a.ptr + r + 1) : 0;
+                const bool here = r < r1 && merge_ends_by(end, c);
                 if (here) {
                     const int beg = __ldg(a.ptr + r);
                     if (end > (beg > k0 ? beg : k0)) flag[end - 1 - c] = 1;
