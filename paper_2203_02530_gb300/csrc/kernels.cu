@@ -516,8 +516,9 @@ __global__ void __launch_bounds__(256) csr_vector_kernel(CsrArgs a, const Tile* 
             const int row = rbase + group;
             double sum = 0.0;
             if (row < d.r1) {
-                const int kb = __ldg(a.ptr + row), ke = __ldg(a.ptr + row + 1);
-                for (int k4 = (kb & ~3) + 4 * lane; k4 < ke; k4 += 4 * V) {
+                // unsigned: the step past the last entry may pass 2^31
+                const unsigned kb = __ldg(a.ptr + row), ke = __ldg(a.ptr + row + 1);
+                for (unsigned k4 = (kb & ~3u) + 4 * lane; k4 < ke; k4 += 4 * V) {
                     const int4 c = __ldg(reinterpret_cast<const int4*>(a.col + k4));
                     const double2 v0 = __ldg(reinterpret_cast<const double2*>(a.val + k4));
                     const double2 v1 = __ldg(reinterpret_cast<const double2*>(a.val + k4 + 2));

@@ -167,7 +167,7 @@ __device__ __forceinline__ void sell_group(const CsrArgs& a, const SellArgs& sa,
 // then R FMAs in entry order; in the last round the entries at or past ke
 // are neither loaded nor added.
 template <int R>
-__device__ __forceinline__ void long_round(const CsrArgs& a, const double* xb, int k, int ke, double& part,
+__device__ __forceinline__ void long_round(const CsrArgs& a, const double* xb, unsigned k, unsigned ke, double& part,
                                            uint64_t pol_stream, uint64_t pol_keep) {
     double v[R], xv[R];
 #pragma unroll
@@ -228,17 +228,17 @@ __global__ void __launch_bounds__(256, MINB) csr_sell_kernel(CsrArgs a, SellArgs
     for (; u0 < u_end; u0 += stride) {
         if (LNG && u0 < n_long) {
             const SellLong L = sa.longs[sa.long_begin + u0];
-            const int kb = L.k0, ke = L.k1;
+            const unsigned kb = L.k0, ke = L.k1;   // unsigned: the step past the last entry may pass 2^31
             const double* xb = a.x + L.xoff;
             double part = 0.0;
             if (U >= 8) {
                 // the lane's entries kb + lane, + 32, ... in rounds of 8 (at
                 // most 16 per lane: a piece holds at most 512 entries); the
                 // last round is predicated per entry
-                for (int k = kb + lane; k < ke; k += 256) long_round<8>(a, xb, k, ke, part, pol_stream, pol_keep);
+                for (unsigned k = kb + lane; k < ke; k += 256) long_round<8>(a, xb, k, ke, part, pol_stream, pol_keep);
             } else {
                 // fewer registers: rounds of 4, then the lane's last 2 and 1
-                int k = kb + lane;
+                unsigned k = kb + lane;
                 for (; k + 96 < ke; k += 128) {
                     double v[4], xv[4];
 #pragma unroll

@@ -25,6 +25,7 @@
 #include <deque>
 #include <map>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 using spmvk::BatchMat;
@@ -304,8 +305,10 @@ __global__ void __launch_bounds__(kThreads) spmm_list_kernel(const int32_t* __re
         int row = -1;
         if (wr < n_rows) {
             row = __ldg(rows + wr);
-            const int kb = __ldg(ptr + row), ke = __ldg(ptr + row + 1);
-            for (int k = kb + lane; k < ke; k += V) {
+            // the step past the last of up to 2^31 - 9 entries may pass 2^31
+            using Index = std::conditional_t<(V > 8), unsigned, int>;
+            const Index kb = __ldg(ptr + row), ke = __ldg(ptr + row + 1);
+            for (Index k = kb + lane; k < ke; k += V) {
                 const double a = __ldg(val + k);
                 const double* xr = X + (int64_t)__ldg(col + k) * W;
                 double xv[W];
@@ -468,12 +471,16 @@ __device__ __forceinline__ void long_unit(const int32_t* __restrict__ ptr, const
     constexpr int ld = PAD ? pow2_columns(W) : W;
     const int lane = threadIdx.x & 31;
     const int row = m.s_perm ? __ldg(m.s_perm + pos) : pos;
-    const int kb = __ldg(ptr + row), ke = __ldg(ptr + row + 1);
+    // counted within the row: an index past the last of up to 2^31 - 9 entries
+    // may pass 2^31
+    const int kb = __ldg(ptr + row), n = __ldg(ptr + row + 1) - kb;
+    col += kb;
+    val += kb;
     double acc[W];
 #pragma unroll
     for (int c = 0; c < W; ++c) acc[c] = 0.0;
-    int k = kb + lane;
-    for (; k + 96 < ke; k += 128) {   // four entries per lane in flight
+    int k = lane;
+    for (; k + 96 < n; k += 128) {   // four entries per lane in flight
         double a[4], xv[4][W];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
@@ -485,7 +492,7 @@ __device__ __forceinline__ void long_unit(const int32_t* __restrict__ ptr, const
 #pragma unroll
             for (int c = 0; c < W; ++c) acc[c] = fma(a[u], xv[u][c], acc[c]);
     }
-    for (; k < ke; k += 32) {
+    for (; k < n; k += 32) {
         const double a = __ldg(val + k);
         double xv[W];
         load_row<W, PAD>(X + (int64_t)__ldg(col + k) * ld, xv);
@@ -514,12 +521,14 @@ __device__ __forceinline__ void long_cta_unit(const int32_t* __restrict__ ptr, c
     __shared__ double s_part[kThreads / 32][kMaxW];
     const int t = threadIdx.x, warp = t >> 5;
     const int row = m.s_perm ? __ldg(m.s_perm + pos) : pos;
-    const int kb = __ldg(ptr + row), ke = __ldg(ptr + row + 1);
+    const int kb = __ldg(ptr + row), n = __ldg(ptr + row + 1) - kb;   // n > 2048
+    col += kb;
+    val += kb;
     double acc[W];
 #pragma unroll
     for (int c = 0; c < W; ++c) acc[c] = 0.0;
-    int k = kb + t;
-    for (; k + 3 * kThreads < ke; k += 4 * kThreads) {   // four entries per thread in flight
+    int k = t;
+    for (; k < n - 3 * kThreads; k += 4 * kThreads) {   // four entries per thread in flight
         double a[4], xv[4][W];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
@@ -531,7 +540,7 @@ __device__ __forceinline__ void long_cta_unit(const int32_t* __restrict__ ptr, c
 #pragma unroll
             for (int c = 0; c < W; ++c) acc[c] = fma(a[u], xv[u][c], acc[c]);
     }
-    for (; k < ke; k += kThreads) {
+    for (; (unsigned)k < (unsigned)n; k += kThreads) {
         const double a = __ldg(val + k);
         double xv[W];
         load_row<W, PAD>(X + (int64_t)__ldg(col + k) * ld, xv);
