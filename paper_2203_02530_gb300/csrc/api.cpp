@@ -782,7 +782,7 @@ static void prepare_variant(spmv_part* pt, int variant, int param, int op_kind) 
             fail(SPMV_EINVAL, "pair variant %d not in {1,2,4,8,102,104}", param);
     } else if (variant == SPMV_VARIANT_MERGE) {
         check_cuda(cudaDeviceSynchronize(), "synchronize");
-        if (!pt->lmtiles) spmvk::build_merge_tiles(pt);
+        if (!pt->rcarry) spmvk::build_merge_tiles(pt);   // its last allocation
     } else if (variant == SPMV_VARIANT_SELL || variant == SPMV_VARIANT_SELL16) {
         if (!spmvk::sell_param_supported(param))
             fail(SPMV_EINVAL, "sliced variant %d not in {4,8,9,104..107} (+2000 balanced)", param);
@@ -937,15 +937,22 @@ int spmv_graph_destroy(spmv_part* pt, int64_t handle) {
     return SPMV_OK;
 }
 
+// A pair of device vectors, made on first use: both or, when memory runs out,
+// neither.
+static void make_vectors(spmv_part* pt, double*& x, double*& y) {
+    if (x) return;
+    double* const nx = static_cast<double*>(spmvk::dev_alloc(pt, (size_t)pt->n * sizeof(double)));
+    double* const ny = static_cast<double*>(spmvk::dev_alloc(pt, (size_t)pt->n * sizeof(double)));
+    spmvk::default_stream_done();
+    x = nx;
+    y = ny;
+}
+
 int spmv_part_io_buffers(spmv_part* pt, double** x_out, double** y_out) {
     API_TRY
     check_part(pt);
     need(x_out && y_out, SPMV_EINVAL, "output pointer is NULL");
-    if (!pt->io_x) {
-        pt->io_x = static_cast<double*>(spmvk::dev_alloc(pt, (size_t)pt->n * sizeof(double)));
-        pt->io_y = static_cast<double*>(spmvk::dev_alloc(pt, (size_t)pt->n * sizeof(double)));
-        spmvk::default_stream_done();
-    }
+    make_vectors(pt, pt->io_x, pt->io_y);
     *x_out = pt->io_x;
     *y_out = pt->io_y;
     API_CATCH
@@ -961,11 +968,7 @@ namespace {
 // out are done).
 void host_path_setup(spmv_part* pt) {
     const int P = pt->P;
-    if (!pt->io_x) {
-        pt->io_x = static_cast<double*>(spmvk::dev_alloc(pt, (size_t)pt->n * sizeof(double)));
-        pt->io_y = static_cast<double*>(spmvk::dev_alloc(pt, (size_t)pt->n * sizeof(double)));
-        spmvk::default_stream_done();
-    }
+    make_vectors(pt, pt->io_x, pt->io_y);
     while ((int)pt->io_ev.size() < 3 * P + 5) {
         cudaEvent_t e;
         check_cuda(cudaEventCreateWithFlags(&e, cudaEventDisableTiming), "event");
@@ -1173,11 +1176,7 @@ int spmv_apply_host_many(spmv_part* pt, int64_t count, const double* x_host, int
         fail(SPMV_EINVAL, "y_stride %lld overlaps the results of consecutive products", (long long)y_stride);
     if (pt->n == 0 || count == 0) return SPMV_OK;
     host_path_setup(pt);
-    if (!pt->io_x2) {
-        pt->io_x2 = static_cast<double*>(spmvk::dev_alloc(pt, (size_t)pt->n * sizeof(double)));
-        pt->io_y2 = static_cast<double*>(spmvk::dev_alloc(pt, (size_t)pt->n * sizeof(double)));
-        spmvk::default_stream_done();
-    }
+    make_vectors(pt, pt->io_x2, pt->io_y2);
     int64_t launches = 0;
     const bool coarse = !(flags & SPMV_HOST_X_BLOCKS) && host_coarse(pt, count);
     for (int64_t k = 0; k < count; ++k) {

@@ -746,20 +746,21 @@ struct Unit {
 
 // Tables of the current modes: each matrix's CSR or sliced items, and the
 // work units of the launches in claim order.  A unit is an item or, so that a
-// small batch still fills the chip's warps, a part of one.
+// small batch still fills the chip's warps, a part of one.  The batch changes only
+// once every table is on the device (out of memory leaves it as it was).
 void upload_items(spmv_batch* b) {
     std::vector<BatchItem> all;
-    b->item_off.assign(b->count + 1, 0);
+    std::vector<int> item_off(b->count + 1, 0);
     int64_t n_slices = 0, csr_rows = 0;
     for (int m = 0; m < b->count; ++m) {
-        b->item_off[m] = (int)all.size();
+        item_off[m] = (int)all.size();
         const bool sl = b->mats[m].lanes == kSliced;
         const auto& src = sl ? b->sliced_items[m] : b->csr_items[m];
         all.insert(all.end(), src.begin(), src.end());
         if (sl) n_slices += b->mats[m].n_slices;
         else csr_rows += b->n[m];
     }
-    b->item_off[b->count] = b->n_items = (int)all.size();
+    item_off[b->count] = (int)all.size();
     // rows of a CSR unit: as many (16, one pass of two lanes a row, to 256, an
     // item) as leave 8 units for every warp in flight; 2 units for each took
     // 279 us against 264 us at 4.4 M rows and 106 us against 97 us at 1.5 M
@@ -785,12 +786,12 @@ void upload_items(spmv_batch* b) {
         int64_t cost;
     };
     std::vector<Run> runs;
-    b->unit_off.assign(2 * (b->count + 1), 0);
+    std::vector<int> unit_off(2 * (b->count + 1), 0);
     for (int m = 0, piece = 0; m < b->count; ++m) {
         const int part = b->mats[m].lanes == kSliced ? 0 : 1;
         std::vector<Unit>& u = units[part];
-        b->unit_off[m] = (int)units[0].size();
-        b->unit_off[b->count + 1 + m] = (int)units[1].size();
+        unit_off[m] = (int)units[0].size();
+        unit_off[b->count + 1 + m] = (int)units[1].size();
         runs.clear();
         const int pieces = (int)b->pieces[m].size();
         if (pieces > 0) runs.push_back(Run{3, piece, piece + pieces, 1, long_cost(b->piece_len, 1)});
@@ -806,12 +807,12 @@ void upload_items(spmv_batch* b) {
         for (const Run& r : runs)
             for (int a = r.a; a < r.b; a += r.per) u.push_back(Unit{{m, r.kind, a, std::min(r.b, a + r.per)}, r.cost});
     }
-    b->unit_off[b->count] = b->n_sliced_units = (int)units[0].size();
-    b->unit_off[2 * b->count + 1] = (int)units[1].size();
-    b->n_units = (int)(units[0].size() + units[1].size());
-    for (int m = 0; m <= b->count; ++m) b->unit_off[b->count + 1 + m] += b->n_sliced_units;
+    const int n_sliced_units = (int)units[0].size(), n_units = (int)(units[0].size() + units[1].size());
+    unit_off[b->count] = n_sliced_units;
+    unit_off[2 * b->count + 1] = (int)units[1].size();
+    for (int m = 0; m <= b->count; ++m) unit_off[b->count + 1 + m] += n_sliced_units;
     std::vector<BatchItem> order;
-    order.reserve((size_t)b->n_units);
+    order.reserve((size_t)n_units);
     for (const auto& part : units)
         for (const Unit& u : part) order.push_back(u.w);
     // the whole-batch launch takes the sliced units of the length-sorted
@@ -822,7 +823,7 @@ void upload_items(spmv_batch* b) {
     // mix: 864 us against 894 us; weighting the gather-bound work 1.6 or 2
     // times made no difference); each run keeps the matrix-by-matrix order
     // above, and the host-buffer path keeps that order itself
-    std::vector<BatchItem> full(order.begin(), order.begin() + b->n_sliced_units);
+    std::vector<BatchItem> full(order.begin(), order.begin() + n_sliced_units);
     {
         std::vector<const Unit*> ga, st;
         double ca = 0.0, cs = 0.0;
@@ -842,20 +843,38 @@ void upload_items(spmv_batch* b) {
             }
         }
     }
-    auto put = [&](BatchItem*& d, size_t& cap, const std::vector<BatchItem>& h) {
-        if (h.size() > cap) {
-            if (d) brelease(b, d, cap * sizeof(BatchItem));
-            cap = h.size();
-            d = static_cast<BatchItem*>(balloc(b, cap * sizeof(BatchItem)));
+    struct Table {
+        BatchItem*& d;
+        size_t& cap;
+        const std::vector<BatchItem>& h;
+        BatchItem* fresh = nullptr;
+    } tables[] = {{b->d_items, b->items_cap, all},
+                  {b->d_units, b->units_cap, order},
+                  {b->d_units_full, b->units_full_cap, full}};
+    try {
+        for (Table& t : tables)
+            if (t.h.size() > t.cap) t.fresh = static_cast<BatchItem*>(balloc(b, t.h.size() * sizeof(BatchItem)));
+    } catch (...) {
+        for (Table& t : tables)
+            if (t.fresh) brelease(b, t.fresh, t.h.size() * sizeof(BatchItem));
+        throw;
+    }
+    for (Table& t : tables) {
+        if (t.fresh) {
+            if (t.d) brelease(b, t.d, t.cap * sizeof(BatchItem));
+            t.d = t.fresh;
+            t.cap = t.h.size();
         }
-        if (!h.empty())
-            spmvk::check_cuda(cudaMemcpy(d, h.data(), h.size() * sizeof(BatchItem), cudaMemcpyHostToDevice),
+        if (!t.h.empty())
+            spmvk::check_cuda(cudaMemcpy(t.d, t.h.data(), t.h.size() * sizeof(BatchItem), cudaMemcpyHostToDevice),
                               "work items");
-    };
-    put(b->d_items, b->items_cap, all);
-    put(b->d_units, b->units_cap, order);
-    put(b->d_units_full, b->units_full_cap, full);
+    }
     spmvk::default_stream_done();
+    b->item_off = std::move(item_off);
+    b->unit_off = std::move(unit_off);
+    b->n_items = (int)all.size();
+    b->n_sliced_units = n_sliced_units;
+    b->n_units = n_units;
 }
 
 // Sliced layout of matrix m.  Natural row order when no row is longer than
@@ -1375,17 +1394,26 @@ int spmv_batch_set_lanes(spmv_batch* b, int m, int lanes) {
     spmvk::check_cuda(cudaDeviceSynchronize(), "synchronize");   // no launch may read the tables
     if (lanes != kSliced) batch_restore_csr(b);                    // the CSR modes read every row
     const int lo = m < 0 ? 0 : m, hi = m < 0 ? b->count : m + 1;
+    if (lanes == kSliced)
+        for (int i = lo; i < hi; ++i)
+            if (!b->sliced_built[i]) build_sliced(b, i);
     bool changed = false;
+    std::vector<int> before;
     for (int i = lo; i < hi; ++i) {
-        if (lanes == kSliced && !b->sliced_built[i]) build_sliced(b, i);
         changed = changed || ((b->mats[i].lanes == kSliced) != (lanes == kSliced));
+        before.push_back(b->mats[i].lanes);
         b->mats[i].lanes = lanes;
+    }
+    try {
+        if (changed) upload_items(b);
+    } catch (...) {   // out of memory: the tables and the matrices as they were
+        for (int i = lo; i < hi; ++i) b->mats[i].lanes = before[i - lo];
+        throw;
     }
     spmvk::check_cuda(cudaMemcpy(b->d_mats + lo, b->mats.data() + lo, (size_t)(hi - lo) * sizeof(BatchMat),
                                  cudaMemcpyHostToDevice),
                       "lanes");
-    if (changed) upload_items(b);
-    else spmvk::default_stream_done();
+    spmvk::default_stream_done();
     BATCH_CATCH
     return SPMV_OK;
 }
@@ -1474,7 +1502,7 @@ int spmv_batch_run_host_many(spmv_batch* b, int64_t count, const double* x_host,
         spmvk::fail(SPMV_EINVAL, "y_stride %lld overlaps the results of consecutive products", (long long)y_stride);
     if (b->total_rows == 0 || count == 0) return SPMV_OK;
     batch_host_setup(b);
-    if (!b->io_x2) {
+    if (!b->io_y2) {
         b->io_x2 = static_cast<double*>(balloc(b, (size_t)b->total_rows * sizeof(double)));
         b->io_y2 = static_cast<double*>(balloc(b, (size_t)b->total_rows * sizeof(double)));
         spmvk::default_stream_done();

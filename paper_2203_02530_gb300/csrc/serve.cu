@@ -1086,6 +1086,7 @@ int spmv_serve_run(spmv_server* sv, int64_t n_req, const int32_t* matrix, const 
         if ((size_t)n_req > sv->hash_cap) {
             if (sv->d_hash) cudaFree(sv->d_hash);
             sv->d_hash = nullptr;
+            sv->hash_cap = 0;
             spmvk::check_cuda(cudaMalloc(reinterpret_cast<void**>(&sv->d_hash), (size_t)n_req * 8 + 8), "hashes");
             sv->hash_cap = (size_t)n_req;
         }
