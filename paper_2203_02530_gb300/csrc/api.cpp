@@ -106,7 +106,6 @@ spmvk::CsrArgs local_args(spmv_part* pt, const double* x, double* y) {
     a.accumulate = 0;
     a.n_rows = (int)pt->n;
     a.nnz_total = (int)pt->nnz_l;
-    a.guarded = 0;
     a.err = pt->err;
     a.pdl = pt->cur_pdl;
     return a;
@@ -123,7 +122,6 @@ spmvk::CsrArgs remote_args(spmv_part* pt, double* y) {
     a.accumulate = 1;
     a.n_rows = (int)pt->n_rr;
     a.nnz_total = (int)pt->nnz_r;
-    a.guarded = 0;
     a.err = pt->err;
     a.pdl = pt->cur_pdl;
     return a;
@@ -1243,7 +1241,6 @@ int spmv_csr_merge(int64_t n, int64_t nnz, const int32_t* row_ptr, const int32_t
     a.accumulate = 0;
     a.n_rows = (int)n;
     a.nnz_total = (int)nnz;
-    a.guarded = 1;
     a.err = nullptr;
     a.abort_tile = g_merge_abort_tile.load();
     cudaError_t e = spmvk::launch_merge_free(a, static_cast<spmvk::Carry*>(scratch), sms, s);
@@ -1281,7 +1278,6 @@ int spmv_csr_merge_noalloc(int64_t n, int64_t nnz, const int32_t* row_ptr, const
     a.accumulate = 0;
     a.n_rows = (int)n;
     a.nnz_total = (int)nnz;
-    a.guarded = 1;
     a.err = nullptr;
     a.abort_tile = g_merge_abort_tile.load();
     check_cuda(spmvk::launch_merge_noalloc(a, sms, s), "no-allocation merge product");

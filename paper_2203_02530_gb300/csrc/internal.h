@@ -115,8 +115,7 @@ struct CsrArgs {
     double* y;
     int accumulate;         // 0: y = A x ; 1: y += A x
     int n_rows;             // rows of the CSR row space
-    int nnz_total;          // entries of the CSR (bounds the guarded reads)
-    int guarded;            // 1: arrays are not padded past their ends
+    int nnz_total;          // entries of the CSR (bounds the reads of plan-free products)
     int* err;               // device error word
     int abort_tile;         // test hook of the merge-path kernel: k > 0 makes
                             // ranges k-1 and later give up; 0 = never

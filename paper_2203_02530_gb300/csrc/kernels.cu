@@ -299,6 +299,7 @@ __global__ void __launch_bounds__(kTileCtaWarps<ROWS> * 32, (ROWS ? 4 : U > 9 ? 
     csr_tile_kernel(CsrArgs a, const Tile* __restrict__ tiles, int tile_begin, int tile_end, int cap,
                     const Tile* __restrict__ rows, int row_begin, int row_end, int row_ctas) {
     pdl_begin(a.pdl);  // the previous kernel of this stream is done (unless independent)
+    static_assert(S == 1 || U % 2 == 0, "a round begins at an even place");
     constexpr int kTileWarps = kTileCtaWarps<ROWS>;
     const int cta = (int)blockIdx.x - (ROWS ? row_ctas : 0);   // among those that take tiles
     if (ROWS && cta < 0) {
@@ -378,11 +379,6 @@ __global__ void __launch_bounds__(kTileCtaWarps<ROWS> * 32, (ROWS ? 4 : U > 9 ? 
                         const double p = fma(vv[i], xv[u0 + i], acc);
                         acc = base + u0 + i < cnt ? p : acc;
                     }
-                }
-                if (S == 2 && U % 2 == 1) {   // the next round begins at an odd place
-                    const double even = sum[0];
-                    sum[0] = sum[1];
-                    sum[1] = even;
                 }
             }
         } else {
