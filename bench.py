@@ -151,9 +151,9 @@ def hbm_peak():
 
 
 # the files each profiled kernel is built from (besides the shared headers)
-KERNEL_FILES = {"csr_sell_kernel": ["sell.cu"], "merge_kernel": ["merge.cu"],
-                "batch_sliced_persistent_kernel": ["batch.cu", "batch.h"],
-                "batch_persistent_kernel": ["batch.cu", "batch.h"]}
+KERNEL_FILES = {"csr_sell_kernel": ["sell.cu"], "merge_kernel": ["merge.cu", "merge_chunks.h", "pieces.h"],
+                "batch_sliced_persistent_kernel": ["batch.cu", "batch.h", "pieces.h"],
+                "batch_persistent_kernel": ["batch.cu", "batch.h", "pieces.h"]}
 SHARED_HEADERS = ["internal.h", "pdl.cuh"]
 
 

@@ -434,8 +434,8 @@ int spmv_csr_merge_noalloc(int64_t n, int64_t nnz, const int32_t* row_ptr_dev,
                            const double* x_dev, double* y_dev, cudaStream_t s);
 
 /* Device error word of the plan-free entry points on the current device
- * (0 = none; SPMV_ETIMEOUT's magnitude after a bounded wait gave up); reads
- * and clears it, synchronising the device. */
+ * (0 = none; SPMV_ETIMEOUT's magnitude after a launch that gave up, see
+ * spmv_selftest_merge_abort); reads and clears it, synchronising the device. */
 int spmv_csr_error(int64_t* out);
 
 /*

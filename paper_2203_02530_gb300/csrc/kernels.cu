@@ -3,13 +3,14 @@
 // products y_L = A_L x_L and y += A_R x_R.
 //
 // Design for sm_103a: FP64 FMA issues at 2 lanes/clk/SM on this part, so a
-// CSR product with HBM at full speed is nearly FP64-bound.  Every staged product
-// kernel therefore spends exactly one DFMA per stored entry on the main path
-// (one thread walks a row), and gets coalescing from bulk copies
-// (cp.async.bulk, the TMA engine) of whole tiles into a shared-memory ring
-// instead of from lanes cooperating on a row, which would cost FP64 adds in
-// shuffle reductions.  Every row is summed by one thread in storage order,
-// so results do not depend on the grid, the stream or the schedule.
+// CSR product with HBM at full speed is nearly FP64-bound.  The staged kernel
+// therefore spends one DFMA per stored entry where a lane walks a row (in one or
+// two sums), and gets coalescing from bulk copies (cp.async.bulk, the TMA
+// engine) of whole tiles into a stage of shared memory per warp instead of from
+// lanes cooperating on a row, which costs FP64 adds in shuffle reductions; long
+// rows, where that costs little, go to a whole warp or a whole CTA.  Every row is
+// summed in an order that depends on the matrix and the variant alone, so results
+// do not depend on the grid, the stream or the schedule.
 #include "internal.h"
 #include "pdl.cuh"
 
@@ -116,8 +117,7 @@ __device__ __forceinline__ void store_row(const CsrArgs& a, int row, double sum)
 // operations follow one another (16 products of the 27-point stencil on 80^3
 // 809 -> 772 us, on 20^3 245 -> 221 us; power-law 300 000 rows 1015 -> 983 us).
 // Schedules keep a launch per operation: joining the two there changed nothing
-// (replayed 64 x 64 grid 4.1 us both ways, 150 000-row band matrix 11.8 and
-// 11.8, 10.8 and 11.0 on two streams).
+// (replayed 64 x 64 grid 4.1 us and 150 000-row band matrix 8.7 us both ways).
 // ------------------------------------------------------------------------
 constexpr int kPackIlp = 4;
 

@@ -203,9 +203,11 @@ __device__ __forceinline__ void long_round(const CsrArgs& a, const double* xb, u
 // GRP: the units after the long rows are the sorted layout's groups
 // (sell_group) instead of its slices; a group of one slice is that slice.
 // LNG: the launch has long rows; without them their code (rounds of 8 entries)
-// does not hold registers that the slices' rounds need (at 48 and 40 registers a
-// thread they spilled 44 and 68 bytes; 27-point 150^3 with 16-bit deltas, param
-// 107: 159.6 us per step against 161.5 us, bound by FP64 at 143 us and HBM at 138).
+// does not hold registers that the slices' rounds need (27-point 150^3 with 16-bit
+// deltas, param 107: 159.6 us per step against 161.5 us, bound by FP64 at 143 us
+// and HBM at 138).  With long rows the kernels of 48 and 40 registers a thread
+// still spill: 44 and 68 bytes with slices, 52 and 68 with groups, which always
+// carry that code.
 template <int U, int MINB, typename CT, bool YP = false, bool GRP = false, bool LNG = true>
 __global__ void __launch_bounds__(256, MINB) csr_sell_kernel(CsrArgs a, SellArgs sa) {
     // the previous kernel of this stream is done (unless independent, or

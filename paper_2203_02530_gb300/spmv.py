@@ -312,8 +312,9 @@ def spmv_probe_gather(table_dev, idx_dev, count, ctas_per_sm, out_dev, out_cap, 
 
 
 def spmv_selftest_merge_abort(tile):
-    """Make the plan-free merge launches give up from merge tile `tile` on
-    (-1: off); a test hook of the bounded-wait give-up path."""
+    """Make the plan-free merge launches abandon range `tile` of the merge path
+    and every later one (-1: off); a test hook of the error word and the carries
+    of abandoned ranges."""
     _check(lib.spmv_selftest_merge_abort(int(tile)))
 
 
