@@ -471,11 +471,9 @@ __device__ __forceinline__ void long_unit(const int32_t* __restrict__ ptr, const
     constexpr int ld = PAD ? pow2_columns(W) : W;
     const int lane = threadIdx.x & 31;
     const int row = m.s_perm ? __ldg(m.s_perm + pos) : pos;
-    // counted within the row: an index past the last of up to 2^31 - 9 entries
-    // may pass 2^31
+    // counted within the row: past the last of up to 2^31 - 9 entries an index may
+    // pass 2^31
     const int kb = __ldg(ptr + row), n = __ldg(ptr + row + 1) - kb;
-    col += kb;
-    val += kb;
     double acc[W];
 #pragma unroll
     for (int c = 0; c < W; ++c) acc[c] = 0.0;
@@ -484,8 +482,8 @@ __device__ __forceinline__ void long_unit(const int32_t* __restrict__ ptr, const
         double a[4], xv[4][W];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            a[u] = __ldg(val + k + 32 * u);
-            load_row<W, PAD>(X + (int64_t)__ldg(col + k + 32 * u) * ld, xv[u]);
+            a[u] = __ldg(val + (kb + k) + 32 * u);
+            load_row<W, PAD>(X + (int64_t)__ldg(col + (kb + k) + 32 * u) * ld, xv[u]);
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u)
@@ -493,9 +491,9 @@ __device__ __forceinline__ void long_unit(const int32_t* __restrict__ ptr, const
             for (int c = 0; c < W; ++c) acc[c] = fma(a[u], xv[u][c], acc[c]);
     }
     for (; k < n; k += 32) {
-        const double a = __ldg(val + k);
+        const double a = __ldg(val + (kb + k));
         double xv[W];
-        load_row<W, PAD>(X + (int64_t)__ldg(col + k) * ld, xv);
+        load_row<W, PAD>(X + (int64_t)__ldg(col + (kb + k)) * ld, xv);
 #pragma unroll
         for (int c = 0; c < W; ++c) acc[c] = fma(a, xv[c], acc[c]);
     }
@@ -522,8 +520,6 @@ __device__ __forceinline__ void long_cta_unit(const int32_t* __restrict__ ptr, c
     const int t = threadIdx.x, warp = t >> 5;
     const int row = m.s_perm ? __ldg(m.s_perm + pos) : pos;
     const int kb = __ldg(ptr + row), n = __ldg(ptr + row + 1) - kb;   // n > 2048
-    col += kb;
-    val += kb;
     double acc[W];
 #pragma unroll
     for (int c = 0; c < W; ++c) acc[c] = 0.0;
@@ -532,8 +528,8 @@ __device__ __forceinline__ void long_cta_unit(const int32_t* __restrict__ ptr, c
         double a[4], xv[4][W];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            a[u] = __ldg(val + k + kThreads * u);
-            load_row<W, PAD>(X + (int64_t)__ldg(col + k + kThreads * u) * ld, xv[u]);
+            a[u] = __ldg(val + (kb + k) + kThreads * u);
+            load_row<W, PAD>(X + (int64_t)__ldg(col + (kb + k) + kThreads * u) * ld, xv[u]);
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u)
@@ -541,9 +537,9 @@ __device__ __forceinline__ void long_cta_unit(const int32_t* __restrict__ ptr, c
             for (int c = 0; c < W; ++c) acc[c] = fma(a[u], xv[u][c], acc[c]);
     }
     for (; (unsigned)k < (unsigned)n; k += kThreads) {
-        const double a = __ldg(val + k);
+        const double a = __ldg(val + (kb + k));
         double xv[W];
-        load_row<W, PAD>(X + (int64_t)__ldg(col + k) * ld, xv);
+        load_row<W, PAD>(X + (int64_t)__ldg(col + (kb + k)) * ld, xv);
 #pragma unroll
         for (int c = 0; c < W; ++c) acc[c] = fma(a, xv[c], acc[c]);
     }
