@@ -826,6 +826,7 @@ struct spmv_server {
     Pool pool;
     unsigned long long* d_hash = nullptr;
     size_t hash_cap = 0;
+    cudaEvent_t hash_ev = nullptr;   // d_hash zeroed for the current run
     int num_sms = 0;
     // per matrix: rows longer than short_max[m] in two buckets (8 lanes up to
     // kMidRow entries, 32 lanes above), as row lists
@@ -991,6 +992,7 @@ int spmv_serve_create(spmv_batch* mats, int n_streams, int64_t budget_bytes, spm
         spmvk::check_cuda(cudaMallocHost(reinterpret_cast<void**>(&sv->h_group[i]), kGroupMax * sizeof(GroupBlock)),
                           "group staging");
     }
+    spmvk::check_cuda(cudaEventCreateWithFlags(&sv->hash_ev, cudaEventDisableTiming), "event");
     *out = sv;
     sv = nullptr;
     return SPMV_OK;
@@ -1017,6 +1019,7 @@ int spmv_serve_destroy(spmv_server* sv) {
         if (p) cudaFree(p);
     for (auto p : sv->h_group)
         if (p) cudaFreeHost(p);
+    if (sv->hash_ev) cudaEventDestroy(sv->hash_ev);
     if (sv->d_hash) cudaFree(sv->d_hash);
     if (sv->bucket_rows) cudaFree(sv->bucket_rows);
     delete sv;
@@ -1086,10 +1089,11 @@ int spmv_serve_run(spmv_server* sv, int64_t n_req, const int32_t* matrix, const 
             spmvk::check_cuda(cudaMalloc(reinterpret_cast<void**>(&sv->d_hash), (size_t)n_req * 8 + 8), "hashes");
             sv->hash_cap = (size_t)n_req;
         }
-        // zeroed before any slot adds to them: the slots' streams do not wait for
-        // the default stream, which may have the caller's work queued
+        // zeroed on the first slot's stream, which the other slots wait for
+        // (hashes_zeroed): they do not wait for the default stream, which may have
+        // the caller's work queued
         spmvk::check_cuda(cudaMemsetAsync(sv->d_hash, 0, (size_t)n_req * 8 + 8, sv->streams[0]), "hashes");
-        spmvk::check_cuda(cudaStreamSynchronize(sv->streams[0]), "hashes");
+        spmvk::check_cuda(cudaEventRecord(sv->hash_ev, sv->streams[0]), "event");
     }
     struct Inflight {
         bool busy = false;
@@ -1118,6 +1122,14 @@ int spmv_serve_run(spmv_server* sv, int64_t n_req, const int32_t* matrix, const 
             if (arrival_s[a] < arrival_s[b] || (arrival_s[a] == arrival_s[b] && a < b)) best = k;
         }
         return best;
+    };
+    // before a launch of slot i that adds to the hashes; a wait only while the zeros
+    // are not known to be there (a wait of the host for them cost 7 us a run)
+    bool zeroed = hash_out == nullptr;
+    auto hashes_zeroed = [&](int i) {
+        if (zeroed || i == 0) return;
+        zeroed = cudaEventQuery(sv->hash_ev) == cudaSuccess;
+        if (!zeroed) spmvk::check_cuda(cudaStreamWaitEvent(sv->streams[i], sv->hash_ev, 0), "wait");
     };
     int64_t next = 0, done = 0, blocks = 0, waits_mem = 0, max_inflight = 0, admitted_while_busy = 0;
     const auto t0 = std::chrono::steady_clock::now();
@@ -1220,6 +1232,7 @@ int spmv_serve_run(spmv_server* sv, int64_t n_req, const int32_t* matrix, const 
                     }
                     if (nb == 0) break;   // no memory: wait for completions
                     cudaStream_t st = sv->streams[i];
+                    hashes_zeroed(i);
                     spmvk::check_cuda(cudaMemcpyAsync(sv->d_group[i], hg, (size_t)nb * sizeof(GroupBlock),
                                                       cudaMemcpyHostToDevice, st),
                                       "group table");
@@ -1280,6 +1293,7 @@ int spmv_serve_run(spmv_server* sv, int64_t n_req, const int32_t* matrix, const 
                 pend_width[m] -= wsum;
                 double* X = reinterpret_cast<double*>(sv->pool.ptr(off));
                 double* Y = X + (size_t)n * xc;
+                hashes_zeroed(i);
                 spmvk::check_cuda(launch_block(sv, m, b, pads(sv, m), X, Y, hash_out ? sv->d_hash : nullptr,
                                                sv->streams[i]),
                                   "block launch");
