@@ -14,12 +14,12 @@
 //
 // What bounds it: the scattered x gathers (38 us for 10.8 M at the rate of
 // random reads) and the FP64 pipe (about 14 FP64 instructions per 8 entries of
-// a lane, 0.51 of the pipe).  Power-law matrix of 700 001 rows, 10.8 M entries:
-// 68 us (70 us with 16-byte loads); the form before, tiles of 2048 items staged
-// in shared memory per CTA and walked item by item (48 M warp instructions
-// against 19 M, 24 warps per SM, a path search of 22 dependent shared-memory
-// reads a thread, and a launch of its own that computed the tiles), took 154 us.
-// 7-point stencil of 12 696 rows: 6.2 us against 14.3 us.
+// a lane; 0.70 of the pipe's active cycles on 28.6 M entries).  Power-law matrix
+// of 700 001 rows, 10.8 M entries: 68 us (70 us with 16-byte loads); the form
+// before, tiles of 2048 items staged in shared memory per CTA and walked item by
+// item (48 M warp instructions against 19 M, 24 warps per SM, a path search of 22
+// dependent shared-memory reads a thread, and a launch of its own that computed
+// the tiles), took 154 us.  7-point stencil of 12 696 rows: 6.2 us against 14.3 us.
 #include "internal.h"
 #include "merge_chunks.h"
 #include "pdl.cuh"
